@@ -379,7 +379,9 @@ int bart_set_graph(bart_ctx *ctx, int32_t enable);
  * 0, the default), 8 (where M allows: M divides 256 or 256 divides M) or 32
  * (M = 256, 512 or 1024);
  * tiles_per_item = 32-record tiles per work item (0 = default, scaled with
- * the largest scene).  The results differ only by FP32 summation order.
+ * the scene).  8 and 32 sum every facet at every sample; 16 does so on a
+ * coarse grid per rigid instance where that is exact to the FP32 phasors
+ * (see csrc/band.cuh).  The results differ by FP32 rounding.
  * Errors: EINVAL. */
 int bart_set_synth_layout(bart_ctx *ctx, int32_t samples_per_lane, int32_t tiles_per_item);
 

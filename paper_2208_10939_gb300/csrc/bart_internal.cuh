@@ -25,8 +25,14 @@ constexpr double kEpsT = 1e-9;
 constexpr int kRecVertex = 0;
 constexpr int kRecSeries = 1;
 constexpr int kRecEdge = 2;
+constexpr int kRecPair = 3;           // band rows: the vertex form with one edge's pair together
 constexpr double kSeriesKD = 1.0;     // k_max * (u_max - u_min) below this: series
 constexpr double kEdgeKd = 0.03;      // k_max * min pair gap below this: edge form
+// band rows: below this the pair form (at most 1/2: with k_max * spread >= 1
+// one edge at most is then short); measured on 12 mm rough vehicles, vertex
+// weights down to 0.03 left 1.7e-6 (median) and 5.8e-6 (worst of 30) in the
+// cube, the pair form below 0.5 leaves 0.7e-6 and 2.3e-6
+constexpr double kPairKd = 0.5;
 constexpr double kSincSeries = 0.25;  // |k gamma| below this: sinc by its series
 constexpr int kSeriesTerms = 15;      // p = 0..14
 
@@ -98,12 +104,16 @@ constexpr int kStatusWaitTimeout = 2;   // a bounded device wait expired (see ba
 // fac_lo: per facet 12 floats, the rounding residues of the FP32 centroid
 // and vertex offsets in FacetRec (c - (double)rec.c, dv - (double)rec.dv),
 // so that c and dv are available as double-float pairs
+// box: per instance 8 words whose memset-0 start and atomicMax give its box:
+// ~ord(min corner) 3, ord(max corner) 3, ord(largest squared vertex offset), 0
+// (ord: the order-preserving map of float to unsigned)
 // the world-facet kernel (its t0 argument is updated in replayed frame graphs)
 const void *build_facets_kernel_fn(int *t0_arg_index, int *n_args);
 void launch_build_facets(const MeshDesc *meshes, const InstDev *insts, int n_inst,
                          int64_t F, double t0, double *tri64, float *tri32, double *c64,
                          FacetRec *fac, float *aabb, float *vel32, unsigned int *bounds,
-                         double *ref64, float *ref32, float *fac_lo, cudaStream_t s);
+                         double *ref64, float *ref32, float *fac_lo, unsigned int *box,
+                         cudaStream_t s);
 void launch_morton(const FacetRec *fac, int64_t F, const unsigned int *bounds,
                    uint32_t *keys, int32_t *vals, cudaStream_t s);
 // Stable LSD radix sort of (key, value) pairs on the low `bits` bits.

@@ -11,10 +11,12 @@
 #include <cstring>
 #include <new>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include <nvtx3/nvToolsExt.h>
 
+#include "band.cuh"
 #include "bart_internal.cuh"
 #include "bounce.cuh"
 #include "bartsim.h"
@@ -153,6 +155,15 @@ struct bart_ctx {
     DevBuf<float2> partial;             // mixed-path per-item partial sums
     DevBuf<int32_t> item_off;
     DevBuf<int> item_counter;
+    // band-limited mixed path (band.cuh): instance boxes, tables of the (N, M)
+    // they were made for, plans, references, lists and items
+    DevBuf<unsigned int> box;
+    DevBuf<float> band_tab;
+    BandShape band_sh{};
+    DevBuf<unsigned char> band_ws;
+    DevBuf<int64_t> d_ioff;             // facet offsets of the instances [I + 1]
+    DevBuf<int32_t> d_sinst;            // first instance of each scene [B + 1]
+    DevBuf<float2> band_coarse;
     DevBuf<unsigned long long> counters;   // 0 vertex, 1 series, 2 edge, 3 grazing
     DevBuf<int> status;
     DevBuf<unsigned char> rdm_ws, adc_own;
@@ -258,6 +269,8 @@ struct bart_ctx {
         keys.release(); keys_tmp.release(); sort_temp.release(); vals.release();
         vals_tmp.release(); nodes.release(); parent.release(); leaf_parent.release();
         flags.release(); state.release(); blk_cnt.release(); vis_idx.release();
+        box.release(); band_tab.release(); band_ws.release(); d_ioff.release(); d_sinst.release();
+        band_coarse.release();
         vis_cnt.release(); kin.release(); kquad.release(); partial.release(); item_off.release();
         item_counter.release(); counters.release(); status.release();
         rdm_ws.release(); adc_own.release(); rdm_own.release(); noise_scratch.release();
@@ -640,6 +653,33 @@ int bart_radar_set(bart_ctx *ctx, const bart_radar *r)
 constexpr int kPathAdjoint = 100;
 constexpr int kPathAdjointMixed = 101;
 
+// The mixed path's two evaluations: band-limited (band.cuh) unless
+//  - another lane layout than 16 samples was asked for,
+//  - the delay form is not the facet's own (its bounds are for that form),
+//  - the frame is longer than its tables go,
+//  - the instances are so many and so small that interpolating each over the
+//    cube costs more than summing its facets over it (12 channels of 64 x
+//    256, direct against band-limited synthesis: 1 x 200 facets 0.20 / 0.09
+//    ms, 16 x 160 0.46 / 0.16, 64 x 96 0.48 / 0.37, 64 x 2 0.07 / 0.31, 256 x
+//    160 0.87 / 1.24), or
+//  - the per-instance coarse cubes could exceed 16 GB.
+// A short frame gains too (one sedan, 1 chirp: 0.21 / 0.15 ms).
+static bool use_band(const bart_ctx *ctx, const RadarDev &rd, int64_t F, int I)
+{
+    return ctx->layout_S == 0 && !rd.far_field && !rd.delay_ref && rd.N <= 1024 &&
+           F >= 8 * (int64_t)I * std::min(I, 32) && (int64_t)I * rd.O <= 65535 &&
+           (int64_t)I * rd.O * rd.N * rd.M <= ((int64_t)1 << 31);
+}
+
+// work items to aim for: six per resident warp, so that the last wave is short
+static int synth_band_target()
+{
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return 6 * 16 * std::max(sms, 1);
+}
+
 static int run_frame(bart_ctx *ctx, double t0, int32_t path, void *adc, int32_t dtype,
                      bart_stats *stats)
 {
@@ -692,7 +732,8 @@ static int run_frame(bart_ctx *ctx, double t0, int32_t path, void *adc, int32_t 
     for (int b = 0; b < B; ++b) scene_F[b] = foff[b + 1] - foff[b];
 
     if (md.size() > ctx->d_meshes.cap || (size_t)I > ctx->d_insts.cap ||
-        (size_t)(3 * I) > ctx->vel64.cap)
+        (size_t)(3 * I) > ctx->vel64.cap || (size_t)(I + 1) > ctx->d_ioff.cap ||
+        (size_t)(B + 1) > ctx->d_sinst.cap)
         ctx->tables_dirty = true;
     BART_TRY(ctx->d_meshes.ensure(md.size(), "mesh table"));
     BART_TRY(ctx->d_insts.ensure(I, "instance table"));
@@ -703,6 +744,9 @@ static int run_frame(bart_ctx *ctx, double t0, int32_t path, void *adc, int32_t 
     BART_TRY(ctx->vel32.ensure(4 * I, "instance velocities (f32)"));
     BART_TRY(ctx->ref64.ensure(3 * I, "instance origins"));
     BART_TRY(ctx->ref32.ensure(4 * I, "instance origins (f32)"));
+    BART_TRY(ctx->box.ensure(8 * (size_t)I, "instance boxes"));
+    BART_TRY(ctx->d_ioff.ensure((size_t)I + 1, "instance facet offsets"));
+    BART_TRY(ctx->d_sinst.ensure((size_t)B + 1, "scene instance offsets"));
     BART_TRY(ctx->aabb.ensure(6 * F, "facet boxes"));
     BART_TRY(ctx->fac.ensure(F, "facet records"));
     BART_TRY(ctx->fac_lo.ensure(12 * F, "facet record residues"));
@@ -762,6 +806,14 @@ static int run_frame(bart_ctx *ctx, double t0, int32_t path, void *adc, int32_t 
             for (int k = 0; k < 3; ++k) v[3 * i + k] = ctx->insts[i].vel[k];
         CUDA_TRY(cudaMemcpyAsync(ctx->vel64.p, v.data(), v.size() * sizeof(double),
                                  cudaMemcpyHostToDevice, s), "velocity copy");
+        std::vector<int64_t> ioff(I + 1);
+        for (int i = 0; i < I; ++i) ioff[i] = id[i].off;
+        ioff[I] = F;
+        std::vector<int32_t> sinst = B > 1 ? ctx->scene_first : std::vector<int32_t>{0, I};
+        CUDA_TRY(cudaMemcpyAsync(ctx->d_ioff.p, ioff.data(), ioff.size() * sizeof(int64_t),
+                                 cudaMemcpyHostToDevice, s), "instance offset copy");
+        CUDA_TRY(cudaMemcpyAsync(ctx->d_sinst.p, sinst.data(), sinst.size() * sizeof(int32_t),
+                                 cudaMemcpyHostToDevice, s), "scene instance copy");
         if (B > 1)
             CUDA_TRY(cudaMemcpyAsync(ctx->d_foff.p, foff.data(), (B + 1) * sizeof(int64_t),
                                      cudaMemcpyHostToDevice, s), "scene offset copy");
@@ -773,6 +825,8 @@ static int run_frame(bart_ctx *ctx, double t0, int32_t path, void *adc, int32_t 
                         ? ctx->tpi_override
                         : synth_tiles_per_item(*std::max_element(scene_F.begin(), scene_F.end()));
     int64_t max_items = 0;
+    const bool band = path == BART_PATH_MIXED && use_band(ctx, rd, F, I);
+    BandArgs bt{};
     const bool mixed_rows = path == BART_PATH_MIXED || path == BART_PATH_SPECTRAL ||
                             path == kPathAdjointMixed;
     if (path == BART_PATH_SPECTRAL && ctx->spec_M != rd.M) {
@@ -789,7 +843,62 @@ static int run_frame(bart_ctx *ctx, double t0, int32_t path, void *adc, int32_t 
         // evaluated per record inside the synthesis)
         BART_TRY(ctx->kin.ensure((size_t)A * F * kKinRowWords, "kinematics rows"));
         BART_TRY(ctx->kquad.ensure((size_t)A * F * kKinQuadWords, "kinematics quadratics"));
-        if (path == BART_PATH_MIXED) {
+        if (band) {
+            if (ctx->band_sh.N != rd.N || ctx->band_sh.M != rd.M) {
+                BandShape sh;
+                band_shape(rd.N, rd.M, sh);
+                const BandSizes z = band_sizes(sh);
+                ctx->band_sh = BandShape{};
+                BART_TRY(ctx->band_tab.ensure((size_t)(z.nodes + z.wn + z.wm + z.base), "band tables"));
+                launch_band_tables(sh, ctx->band_tab.p, ctx->band_tab.p + z.nodes,
+                                   reinterpret_cast<int *>(ctx->band_tab.p + z.nodes + z.wn + z.wm),
+                                   ctx->band_tab.p + z.nodes + z.wn, s);
+                CUDA_TRY(cudaGetLastError(), "band table launch");
+                ctx->band_sh = sh;
+            }
+            const BandSizes z = band_sizes(ctx->band_sh);
+            const int64_t V = (int64_t)I * O;
+            bt.sh = ctx->band_sh;
+            bt.nodes = ctx->band_tab.p;
+            bt.wn = bt.nodes + z.nodes;
+            bt.wm = bt.wn + z.wn;
+            bt.base = reinterpret_cast<const int *>(bt.wm + z.wm);
+            bt.I = I;
+            bt.B = B;
+            bt.O = O;
+            bt.chunk_target = synth_band_target();
+            bt.fixed_chunk = 32 * ctx->tpi_override;
+            bt.max_items = band_max_items(bt.sh, V, bt.chunk_target, (int64_t)O * F, bt.fixed_chunk);
+            BART_TRY(ctx->partial.ensure((size_t)bt.max_items * 32 * kBandS, "synthesis partials"));
+            BART_TRY(ctx->band_coarse.ensure((size_t)(V * rd.N * rd.M), "band coarse samples"));
+            bt.box = ctx->box.p;
+            bt.scene_inst = ctx->d_sinst.p;
+            bt.ioff = ctx->d_ioff.p;
+            bt.partial = reinterpret_cast<float4 *>(ctx->partial.p);
+            bt.coarse = ctx->band_coarse.p;
+            // the small arrays in one allocation, widest elements first
+            auto carve = [&](unsigned char *p) -> size_t {
+                size_t n = 0;
+                auto take = [&](auto *&field, int64_t count) {
+                    using T = std::remove_reference_t<decltype(*field)>;
+                    field = reinterpret_cast<T *>(p + n);
+                    n += ((size_t)count * sizeof(T) + 15) / 16 * 16;
+                };
+                take(bt.ref, V * rd.N);
+                take(bt.refn, V * rd.N);
+                take(bt.items, bt.max_items);
+                take(bt.plan, I);
+                take(bt.coff, V);
+                take(bt.vstart, V);
+                take(bt.vcnt, V);
+                take(bt.item0, V + 1);
+                take(bt.item_counter, 1);
+                take(bt.chunk, 1);
+                return n;
+            };
+            BART_TRY(ctx->band_ws.ensure(carve(nullptr), "band plans and items"));
+            carve(ctx->band_ws.p);
+        } else if (path == BART_PATH_MIXED) {
             BART_TRY(ctx->partial.ensure((size_t)synth_partial_words(scene_F.data(), B, rd, rd.N,
                                                                      tpi, ctx->layout_S),
                                          "synthesis partials"));
@@ -835,9 +944,36 @@ static int run_frame(bart_ctx *ctx, double t0, int32_t path, void *adc, int32_t 
         nv.next("bart facets");
         launch_build_facets(ctx->d_meshes.p, ctx->d_insts.p, I, F, t0v, ctx->tri64.p, ctx->tri32.p,
                             ctx->c64.p, ctx->fac.p, ctx->aabb.p, ctx->vel32.p, ctx->bounds.p,
-                            ctx->ref64.p, ctx->ref32.p, ctx->fac_lo.p, s);
+                            ctx->ref64.p, ctx->ref32.p, ctx->fac_lo.p, ctx->box.p, s);
         launches += 1;
         if (tm) CUDA_TRY(cudaEventRecord(ctx->ev[1], s), "cudaEventRecord");
+        SynthArgs a;
+        a.fac = ctx->fac.p;
+        a.tri64 = ctx->tri64.p;
+        a.c64 = ctx->c64.p;
+        a.vel64 = ctx->vel64.p;
+        a.vel32 = ctx->vel32.p;
+        a.ref64 = ctx->ref64.p;
+        a.ref32 = ctx->ref32.p;
+        a.fac_lo = ctx->fac_lo.p;
+        a.vis_idx = ctx->vis_idx.p;
+        a.vis_cnt = ctx->vis_cnt.p;
+        a.VO = B * O;
+        a.vstart = B > 1 ? ctx->vstart.p : nullptr;
+        a.vcnt = B > 1 ? ctx->vcnt.p : ctx->vis_cnt.p;
+        a.F = F;
+        a.kin = nullptr;
+        a.kquad = nullptr;
+        a.out = adc;
+        a.out_c64 = dtype == BART_C64;
+        a.counters = ctx->counters.p;
+        a.item_off = nullptr;
+        a.item_counter = nullptr;
+        a.partial = nullptr;
+        a.tiles_per_item = tpi;
+        a.max_items = 0;
+        a.layout_S = ctx->layout_S;
+        a.rd = rd;
         // the mixed and spectral paths' kinematics rows need only the world
         // facets: they run on a second stream beside the hierarchy build and
         // visibility
@@ -845,6 +981,10 @@ static int run_frame(bart_ctx *ctx, double t0, int32_t path, void *adc, int32_t 
             nv.next("bart kinematics rows");
             CUDA_TRY(cudaEventRecord(ctx->fork_ev, s), "cudaEventRecord");
             CUDA_TRY(cudaStreamWaitEvent(ctx->side, ctx->fork_ev, 0), "cudaStreamWaitEvent");
+            if (band) {
+                launch_band_plan(bt, a, ctx->side);
+                launches += 2;
+            }
             if (tm) CUDA_TRY(cudaEventRecord(ctx->ev_kin[0], ctx->side), "cudaEventRecord");
             launch_kin_coef(ctx->c64.p, ctx->fac.p, ctx->vel64.p, ctx->ref64.p, F, rd, ctx->kin.p,
                             ctx->kquad.p, ctx->side);
@@ -883,7 +1023,7 @@ static int run_frame(bart_ctx *ctx, double t0, int32_t path, void *adc, int32_t 
                           ctx->counters.p + 3, ctx->status.p, s);
         launch_compact(ctx->state.p, F, rd, ctx->blk_cnt.p, ctx->vis_idx.p, ctx->vis_cnt.p, s);
         launches += 1 + 3;
-        if (B > 1) {
+        if (B > 1 && !(band && !stats)) {
             launch_scene_lists(ctx->vis_idx.p, ctx->vis_cnt.p, F, O, ctx->d_foff.p, B, ctx->vstart.p,
                                ctx->vcnt.p, s);
             launches += 1;
@@ -960,33 +1100,6 @@ static int run_frame(bart_ctx *ctx, double t0, int32_t path, void *adc, int32_t 
         if (tm) CUDA_TRY(cudaEventRecord(ctx->ev[3], s), "cudaEventRecord");
         // 4. synthesis
         nv.next("bart synthesis");
-        SynthArgs a;
-        a.fac = ctx->fac.p;
-        a.tri64 = ctx->tri64.p;
-        a.c64 = ctx->c64.p;
-        a.vel64 = ctx->vel64.p;
-        a.vel32 = ctx->vel32.p;
-        a.ref64 = ctx->ref64.p;
-        a.ref32 = ctx->ref32.p;
-        a.fac_lo = ctx->fac_lo.p;
-        a.vis_idx = ctx->vis_idx.p;
-        a.vis_cnt = ctx->vis_cnt.p;
-        a.VO = B * O;
-        a.vstart = B > 1 ? ctx->vstart.p : nullptr;
-        a.vcnt = B > 1 ? ctx->vcnt.p : ctx->vis_cnt.p;
-        a.F = F;
-        a.kin = nullptr;
-        a.kquad = nullptr;
-        a.out = adc;
-        a.out_c64 = dtype == BART_C64;
-        a.counters = ctx->counters.p;
-        a.item_off = nullptr;
-        a.item_counter = nullptr;
-        a.partial = nullptr;
-        a.tiles_per_item = tpi;
-        a.max_items = 0;
-        a.layout_S = ctx->layout_S;
-        a.rd = rd;
         if (path == BART_PATH_MIXED) {
             a.partial = ctx->partial.p;
             a.item_off = ctx->item_off.p;
@@ -998,10 +1111,15 @@ static int run_frame(bart_ctx *ctx, double t0, int32_t path, void *adc, int32_t 
             a.nc = rd.N;
             CUDA_TRY(cudaStreamWaitEvent(s, ctx->join_ev, 0), "cudaStreamWaitEvent");
             if (tm) CUDA_TRY(cudaEventRecord(ctx->ev_syn[0], s), "cudaEventRecord");
-            launch_synth_mixed(a, s);
+            if (band) {
+                launch_synth_band(bt, a, s);
+                if (stats) launch_count_records(a, s);
+            } else {
+                launch_synth_mixed(a, s);
+            }
             if (tm) CUDA_TRY(cudaEventRecord(ctx->ev_syn[1], s), "cudaEventRecord");
             ctx->chunks = 1;
-            launches += 4;
+            launches += band ? (stats ? 8 : 7) : 4;
         } else if (path == BART_PATH_SPECTRAL) {
             a.kin = ctx->kin.p;
             a.kquad = ctx->kquad.p;

@@ -94,10 +94,10 @@ __device__ __forceinline__ float4 kin_finish(float xh, float xl, float R, float 
 
 // a row without a convergent expansion: FP64 square root at slot s (far
 // field: R + l / R)
-__device__ __forceinline__ float4 kin_fallback(const double *__restrict__ quad, int s, double Tc,
+__device__ __forceinline__ float4 kin_fallback(const double *__restrict__ quad, double s, double Tc,
                                                double f0c, double mu_f0)
 {
-    const double t = (double)s * Tc;
+    const double t = s * Tc;
     double R = sqrt(quad[0] + t * (quad[1] + t * quad[2]));
     R += (quad[3] + t * quad[4]) / R;
     const double x0u = R * f0c;
@@ -112,7 +112,7 @@ __device__ __forceinline__ float4 kin_fallback(const double *__restrict__ quad, 
 __device__ __forceinline__ void kin_eval2(const float4 *__restrict__ rt,
                                           const float4 *__restrict__ rr,
                                           const double *__restrict__ qt,
-                                          const double *__restrict__ qr, int s, float tau,
+                                          const double *__restrict__ qr, double s, float tau,
                                           double Tc, double f0c, double mu_f0, float mfh,
                                           float mfl, float4 &kt, float4 &kr)
 {
@@ -163,6 +163,8 @@ struct MixConsts {
 //   vertex (V): [0..2] ph0_v  [3..5] lo_v  [6..8] w_v  [9..11] step re
 //               [12..14] step im  [15] hi  [16] p2  [17..19] 2 cos(2 step)
 //               [20..22] 4 sin(2 step)
+//   pair (P, band rows): as V for the phasors m, a, c, but [6] P k_0 (times
+//               kappa sinc at each sample), [23] (k_0 D / 2)^2
 //   series (S): [0] ph0c [1] hi [2] loc [3] p2 [4] po [5] pl [6..13] cr [14..20] ci
 //   edge (E):   [0] ph0c [1] hi [2] loc [3] p2 [4+4e] po [5+4e] pl [6+4e] G [7+4e] K
 //               [16] sinc-series flags (int bits)
@@ -180,12 +182,18 @@ __device__ __forceinline__ float red1(float x) { return x - rintf(x); }
 struct MixRow {
     const float4 *kin_t, *kin_r;     // kinematics rows of the row's TX and RX
     const double *quad_t, *quad_r;   // their FP64 fallback data
-    int sl;                          // chirp slot
+    double sl;                       // chirp slot (not whole at a band node, see band.cuh)
     int ant_t, ant_r;                // antenna indices of the row's TX and RX
     float tau_s, tn;                 // slot offset from the expansion point; chirp start (s)
     float ptx[3], prx[3];            // antenna positions
+    // band rows only (see band.cuh): the reference phase taken off the record
+    // (ph0, hi, lo, p2 as in RecM) and the spacing of the row's samples
+    float4 ref;
+    float d;
+    float turn;                      // cycles added to each step
 };
 
+template <bool BAND = false>
 __device__ __forceinline__ int build_mixed_record(const SynthArgs &A, const MixConsts &K,
                                                   const MixRow &w, int k, float *R,
                                                   bool exact_u = false)
@@ -288,9 +296,15 @@ __device__ __forceinline__ int build_mixed_record(const SynthArgs &A, const MixC
     }
     float hi = kt.y + kr.y;
     hi = hi >= 1.f ? hi - 1.f : hi;
-    const float loc = (kt.z + kr.z) + K.f0c_fs * Ld - K.mu_c2fs * Lp * Ld;
-    const float p2 = K.half_f0c_fs2 * Ldd + K.mu_c_fs2 * Ld;
+    float loc = (kt.z + kr.z) + K.f0c_fs * Ld - K.mu_c2fs * Lp * Ld;
+    float p2 = K.half_f0c_fs2 * Ldd + K.mu_c_fs2 * Ld;
     const float ph0c = red1((kt.x + kr.x) - K.mu_2c2 * Lp * Lp);
+    if (BAND) {                  // hi - ref.hi is exact: multiples of 2^-14
+        hi = red1(hi - w.ref.y);
+        loc -= w.ref.z;
+        p2 -= w.ref.w;
+    }
+    const float dstep = BAND ? w.d : 1.f;     // samples per step of the recurrence
     // Large facets (f0 |u_v| / c beyond 64 cycles, |u| over ~0.25 m): the
     // FP32 offsets, directions and the product f0 u / c would put ~1e-4 rad
     // into the vertex phases, so u_v and the phases derived from it are
@@ -380,7 +394,7 @@ __device__ __forceinline__ int build_mixed_record(const SynthArgs &A, const MixC
                              fabsf(u[0] - u[2]));
     const float A2 = 2.f * fr.area * g;
     if (K.kmax * (umax - umin) < (float)kSeriesKD) {
-        R[0] = ph0c;
+        R[0] = BAND ? red1(ph0c - w.ref.x) : ph0c;
         R[1] = hi;
         R[2] = loc;
         R[3] = p2;
@@ -404,8 +418,8 @@ __device__ __forceinline__ int build_mixed_record(const SynthArgs &A, const MixC
         for (int i = 0; i < 7; ++i)
             R[14 + i] = ((i & 1) ? sc : -sc) * h[2 * i + 1] * (float)c_inv_fact[2 * i + 3];
         return kRecSeries;
-    } else if (K.kmax * dmin < (float)kEdgeKd) {
-        R[0] = ph0c;
+    } else if (!(BAND && exact_u) && K.kmax * dmin < (float)kEdgeKd) {
+        R[0] = BAND ? red1(ph0c - w.ref.x) : ph0c;
         R[1] = hi;
         R[2] = loc;
         R[3] = p2;
@@ -437,20 +451,63 @@ __device__ __forceinline__ int build_mixed_record(const SynthArgs &A, const MixC
     } else {
         R[15] = hi;
         R[16] = p2;
+        bool pair = false;
+        if (BAND && exact_u && K.kmax * dmin < (float)kPairKd) {
+            // pair form: the vertices a, b of the edge nearly normal to b_t,
+            // D = u_a - u_b, m their middle, c the third vertex.  The vertex
+            // form's two large terms taken together leave three phasors
+            //   F = G (e_a - e_c) + j P k sinc(k D / 2) e_m,
+            //   P = 2A / (u_b - u_c),  G = P / (u_a - u_c),
+            // with no cancelling weights (the other edges have k |du| >= 1/2)
+            pair = true;
+            float D = (u[0] - u[1]) + (ul[0] - ul[1]);
+            float ua = u[0], la = ul[0], ub_ = u[1], lb = ul[1], uc = u[2], lc = ul[2];
+            if (fabsf(u[1] - u[2]) == dmin) {
+                D = (u[1] - u[2]) + (ul[1] - ul[2]);
+                ua = u[1]; la = ul[1]; ub_ = u[2]; lb = ul[2]; uc = u[0]; lc = ul[0];
+            } else if (fabsf(u[0] - u[2]) == dmin) {
+                D = (u[0] - u[2]) + (ul[0] - ul[2]);
+                ub_ = u[2]; lb = ul[2]; uc = u[1]; lc = ul[1];
+            }
+            const float Pw = __fdividef(A2, (ub_ - uc) + (lb - lc));
+            const float G = __fdividef(Pw, (ua - uc) + (la - lc));
+            float um, lm;
+            two_sum(ua, -0.5f * D, um, lm);
+            u[0] = um; ul[0] = lm + la;
+            u[1] = ua; ul[1] = la;
+            u[2] = uc; ul[2] = lc;
+            R[6] = Pw * K.k0;
+            R[7] = G;
+            R[8] = -G;
+            const float x = 0.5f * K.k0 * D;
+            R[23] = x * x;
+        }
         // vertex steps = the centroid's step times e^{j x_v},
         // x_v = -2 pi mu/(fs c) u_v, from its Taylor series (error
         // below x^6/720 = 1.4e-9 for |x| < 0.1), else sincospi
         float sc_, cc_;
-        sincospif(2.f * red1(hi + loc), &sc_, &cc_);
+        sincospif(2.f * (BAND ? red1(fmaf(dstep, hi, dstep * loc)) + w.turn : red1(hi + loc)),
+                  &sc_, &cc_);
 #pragma unroll
         for (int v = 0; v < 3; ++v) {
             const float ua = u[v], ub_ = u[(v + 1) % 3], uc = u[(v + 2) % 3];
             R[v] = vphase(ph0c, ua, ul[v]);
+            if (BAND) R[v] = red1(R[v] - w.ref.x);
             const float lo = loc - K.muc * ua;
             R[3 + v] = lo;
-            R[6 + v] = __fdividef(-A2, (ua - ub_) * (ua - uc));
+            if (pair) {
+                if (v == 0) R[0] += R[0] < 0.25f ? 0.25f : -0.75f;      // the factor j
+            } else if (BAND && exact_u) {
+                // the vertex sum cancels, so its weights take the same u as its
+                // phases, residues included
+                const float lb = ul[(v + 1) % 3], lc = ul[(v + 2) % 3];
+                R[6 + v] = __fdividef(-A2, ((ua - ub_) + (ul[v] - lb)) * ((ua - uc) + (ul[v] - lc)));
+            } else {
+                R[6 + v] = __fdividef(-A2, (ua - ub_) * (ua - uc));
+            }
             float s_, c_;
-            const float x = -6.283185307179586f * K.muc * ua;
+            const float x = BAND ? -6.283185307179586f * (dstep * K.muc) * ua
+                                 : -6.283185307179586f * K.muc * ua;
             if (fabsf(x) < 0.1f) {
                 const float x2 = x * x;
                 const float cx = fmaf(x2, fmaf(x2, 1.f / 24.f, -0.5f), 1.f);
@@ -458,7 +515,8 @@ __device__ __forceinline__ int build_mixed_record(const SynthArgs &A, const MixC
                 c_ = fmaf(cc_, cx, -sc_ * sx);
                 s_ = fmaf(sc_, cx, cc_ * sx);
             } else {
-                sincospif(2.f * red1(hi + lo), &s_, &c_);
+                sincospif(2.f * (BAND ? red1(fmaf(dstep, hi, dstep * lo)) + w.turn : red1(hi + lo)),
+                          &s_, &c_);
             }
             R[9 + v] = c_;
             R[12 + v] = s_;
@@ -469,17 +527,20 @@ __device__ __forceinline__ int build_mixed_record(const SynthArgs &A, const MixC
                                               : fmaf(4.f * c_, c_, -2.f);
             R[20 + v] = 8.f * c_ * s_;                // 4 sin(2 step)
         }
+        if (pair) return kRecPair;
     }
     return kRecVertex;
 }
 
 // The term of a series- or edge-form record (see RecM) at fast-time sample
 // m: the facet integral's k-dependence evaluated per sample, times the
-// phasor of the record's phase (Eq. 13); unscaled (times C / k_m^2 later).
+// phasor of the record's phase (Eq. 13) and `turn` cycles; unscaled (times
+// C / k_m^2 later).
 __device__ __forceinline__ void series_edge_term(const float *R, bool series, float fm,
-                                                 const MixConsts &K, float &dr, float &di)
+                                                 const MixConsts &K, float &dr, float &di,
+                                                 float turn = 0.f)
 {
-    const float thc = fmaf(R[3], fm * fm, fmaf(R[2], fm, R[0] + red1(R[1] * fm)));
+    const float thc = fmaf(R[3], fm * fm, fmaf(R[2], fm, R[0] + red1(R[1] * fm))) + turn;
     const float kp = fmaf(fm, K.kap_step, 1.f);
     dr = 0.f;
     di = 0.f;

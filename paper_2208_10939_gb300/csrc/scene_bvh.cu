@@ -45,10 +45,12 @@ __global__ void build_facets_kernel(const MeshDesc *__restrict__ meshes,
                                     float *__restrict__ aabb, float *__restrict__ vel32,
                                     unsigned int *__restrict__ bounds,
                                     double *__restrict__ ref64, float *__restrict__ ref32,
-                                    float *__restrict__ fac_lo)
+                                    float *__restrict__ fac_lo, unsigned int *__restrict__ box)
 {
     const int64_t f = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     float cf[3] = {0.f, 0.f, 0.f};
+    int inst = -1;
+    unsigned int bx[7] = {0u, 0u, 0u, 0u, 0u, 0u, 0u};    // the facet's part of its box
     const bool valid = f < F;
     if (valid) {
         int lo = 0, hi = n_inst - 1;            // last instance with off <= f
@@ -67,6 +69,7 @@ __global__ void build_facets_kernel(const MeshDesc *__restrict__ meshes,
             for (int r = 0; r < 3; ++r)
                 v[3 * k + r] = world_coord(in.rot + 3 * r, x, y, z, in.pos[r], in.vel[r], t0);
         }
+        inst = lo;
         float vmax = 0.f;
         for (int i = 0; i < 9; ++i) {
             tri64[9 * f + i] = v[i];
@@ -101,6 +104,11 @@ __global__ void build_facets_kernel(const MeshDesc *__restrict__ meshes,
                 rec.dv[3 * k + r] = (float)d;
                 fac_lo[12 * f + 3 + 3 * k + r] = (float)(d - (double)rec.dv[3 * k + r]);
             }
+        float rad2 = 0.f;
+        for (int k = 0; k < 3; ++k)
+            rad2 = fmaxf(rad2, rec.dv[3 * k] * rec.dv[3 * k] + rec.dv[3 * k + 1] * rec.dv[3 * k + 1] +
+                                   rec.dv[3 * k + 2] * rec.dv[3 * k + 2]);
+        bx[6] = f2ord(rad2);
         const double inl = nl > 0.0 ? 1.0 / nl : 0.0;
         rec.n[0] = (float)(nx * inl);
         rec.n[1] = (float)(ny * inl);
@@ -119,6 +127,8 @@ __global__ void build_facets_kernel(const MeshDesc *__restrict__ meshes,
             mx = fmaxf(mx, fmaxf(fabsf((float)lo_), fabsf((float)hi_)));
             aabb[6 * f + r] = __double2float_rd(lo_);
             aabb[6 * f + 3 + r] = __double2float_ru(hi_);
+            bx[r] = ~f2ord(__double2float_rd(lo_));
+            bx[3 + r] = f2ord(__double2float_ru(hi_));
         }
         const float pad = 1e-4f + 4e-6f * mx;
         for (int r = 0; r < 3; ++r) {
@@ -135,6 +145,18 @@ __global__ void build_facets_kernel(const MeshDesc *__restrict__ meshes,
             }
             vel32[4 * lo + 3] = 0.f;
             ref32[4 * lo + 3] = 0.f;
+        }
+    }
+    // the instances' boxes: a warp of one instance reduces before its atomics
+    {
+        const int i0 = __shfl_sync(0xffffffffu, inst, 0);
+        if (__all_sync(0xffffffffu, inst == i0)) {
+            for (int r = 0; r < 7; ++r) {
+                const unsigned int m = __reduce_max_sync(0xffffffffu, bx[r]);
+                if ((threadIdx.x & 31) == 0 && i0 >= 0) atomicMax(box + 8 * (int64_t)i0 + r, m);
+            }
+        } else if (inst >= 0) {
+            for (int r = 0; r < 7; ++r) atomicMax(box + 8 * (int64_t)inst + r, bx[r]);
         }
     }
     // centroid bounds for the Morton grid
@@ -154,21 +176,22 @@ __global__ void build_facets_kernel(const MeshDesc *__restrict__ meshes,
 const void *build_facets_kernel_fn(int *t0_arg_index, int *n_args)
 {
     *t0_arg_index = 4;      // meshes, insts, n_inst, F, t0, tri64, tri32, c64, fac, aabb,
-    *n_args = 15;           // vel32, bounds, ref64, ref32, fac_lo
+    *n_args = 16;           // vel32, bounds, ref64, ref32, fac_lo, box
     return reinterpret_cast<const void *>(build_facets_kernel);
 }
 
 void launch_build_facets(const MeshDesc *meshes, const InstDev *insts, int n_inst, int64_t F,
                          double t0, double *tri64, float *tri32, double *c64, FacetRec *fac,
                          float *aabb, float *vel32, unsigned int *bounds, double *ref64,
-                         float *ref32, float *fac_lo, cudaStream_t s)
+                         float *ref32, float *fac_lo, unsigned int *box, cudaStream_t s)
 {
+    cudaMemsetAsync(box, 0, (size_t)n_inst * 8 * sizeof(unsigned int), s);
     cudaMemsetAsync(bounds, 0xff, 3 * sizeof(unsigned int), s);
     cudaMemsetAsync(bounds + 3, 0, 3 * sizeof(unsigned int), s);
     const int T = 256;
     const unsigned int G = (unsigned int)((F + T - 1) / T);
     build_facets_kernel<<<G, T, 0, s>>>(meshes, insts, n_inst, F, t0, tri64, tri32, c64, fac,
-                                        aabb, vel32, bounds, ref64, ref32, fac_lo);
+                                        aabb, vel32, bounds, ref64, ref32, fac_lo, box);
 }
 
 // -------------------------------------------------------------------------

@@ -43,6 +43,7 @@
 #include <algorithm>
 
 #include "bart_internal.cuh"
+#include "mixed_lane.cuh"
 #include "mixed_record.cuh"
 #include "record_fp64.cuh"
 
@@ -193,44 +194,6 @@ void launch_kin_coef(const double *c64, const FacetRec *fac, const double *vel64
 constexpr int kMixWarps = 2;         // 2-warp CTAs: 22 KB of shared memory at S = 16
 constexpr int kMixMinBlocks = 8;     // resident CTAs per SM: 16 warps, 128 registers a thread
 
-// Packed FP32 pairs (sm_100+ f32x2 arithmetic): two floats in one 64-bit
-// register pair, one instruction for both lanes of a pair.  The mixed
-// kernel keeps two consecutive samples of a lane in one pair.
-__device__ __forceinline__ uint64_t pk2(float lo, float hi)
-{
-    uint64_t r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-    return r;
-}
-__device__ __forceinline__ void upk2(uint64_t r, float &lo, float &hi)
-{
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(r));
-}
-__device__ __forceinline__ uint64_t ffma2(uint64_t a, uint64_t b, uint64_t c)
-{
-    uint64_t d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
-__device__ __forceinline__ uint64_t fmul2(uint64_t a, uint64_t b)
-{
-    uint64_t d;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-__device__ __forceinline__ uint64_t fadd2(uint64_t a, uint64_t b)
-{
-    uint64_t d;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-__device__ __forceinline__ uint64_t fsub2(uint64_t a, uint64_t b)
-{
-    uint64_t d;
-    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-
 // S: consecutive samples per lane; LPR: lanes per chirp row (RPW = 32/LPR
 // rows of the same channel share a warp, e.g. two 256-sample chirps at
 // S = 16).  A 32-record tile holds LPR facets x RPW chirps: lane l builds
@@ -360,104 +323,17 @@ synth_mixed_kernel(SynthArgs A, MixConsts K, int W)
             const int i = row * LPR + ii;
             if ((mv >> i) & 1u) {
                 // ------- vertex form: a three-term recurrence per vertex -------
-                // e^{j(phi + (s+2) a)} = 2 cos(a) e^{j(phi + (s+1) a)} - e^{j(phi + s a)}:
-                // on sample pairs (2k, 2k+1) with the two-sample angle, one FMA
-                // per pair and component.  Pair k is held times sg(k) = +1 for
-                // k mod 4 in {0, 1}, else -1, so that the recurrence needs no
-                // negated addend: held(k) = sg(k) sg(k-1) c2 held(k-1) + held(k-2).
-                // 128-bit broadcast loads of the record
-                const float4 *R4 = reinterpret_cast<const float4 *>(sRec[warp][i].f);
-                const float4 q0 = R4[0], q1 = R4[1], q2v = R4[2], q3 = R4[3], q4 = R4[4],
-                             q5 = R4[5];
-                const float ph0[3] = {q0.x, q0.y, q0.z};
-                const float lo[3] = {q0.w, q1.x, q1.y};
-                const float wv[3] = {q1.z, q1.w, q2v.x};
-                const float sre[3] = {q2v.y, q2v.z, q2v.w};
-                const float sim[3] = {q3.x, q3.y, q3.z};
-                const float c2x2[3] = {q4.y, q4.z, q4.w};     // 2 cos(2 step)
-                const float s2x4[3] = {q5.x, q5.y, q5.z};     // 4 sin(2 step)
-                const float hi = q3.w, p2 = q4.x;
-                // the vertices' common phase at the lane's first sample
-                const float tq = red1(hi * fm0) + p2 * fm0sq;
-                const float eps = p2 * eps_lane;
-    #pragma unroll
-                for (int v = 0; v < 3; ++v) {
-                    const float thv = red1(fmaf(lo[v], fm0, ph0[v] + tq));
-                    float zs, zc;
-                    __sincosf(6.283185307179586f * thv, &zs, &zc);
-                    zc *= wv[v];
-                    zs *= wv[v];
-                    // the lane's step (angle + eps) and its doubled cosines
-                    const float stc = fmaf(-eps, sim[v], sre[v]);
-                    const float sts = fmaf(eps, sre[v], sim[v]);
-                    const float a1 = 2.f * stc;
-                    const float a2 = fmaf(-eps, s2x4[v], c2x2[v]);
-                    // samples m0 + 1 (rotation), m0 + 2 and m0 + 3 (recurrence)
-                    const float zc1 = fmaf(zc, stc, -zs * sts), zs1 = fmaf(zc, sts, zs * stc);
-                    const float zc2 = fmaf(a1, zc1, -zc), zs2 = fmaf(a1, zs1, -zs);
-                    const float zc3 = fmaf(a1, zc2, -zc1), zs3 = fmaf(a1, zs2, -zs1);
-                    uint64_t XC = pk2(zc, zc1), XS = pk2(zs, zs1);       // held(k - 1)
-                    uint64_t YC = pk2(zc2, zc3), YS = pk2(zs2, zs3);     // held(k)
-                    const uint64_t A2 = pk2(a2, a2), NA2 = pk2(-a2, -a2);
-                    PR[0] = fadd2(PR[0], XC);
-                    PI[0] = fadd2(PI[0], XS);
-                    if (S2 > 1) {
-                        PR[1] = fadd2(PR[1], YC);
-                        PI[1] = fadd2(PI[1], YS);
-                    }
-    #pragma unroll
-                    for (int k = 2; k < S2; ++k) {
-                        const bool neg = (k & 2) != 0;                   // sg(k) = -1
-                        const uint64_t A = (((k - 1) & 2) != 0) != neg ? NA2 : A2;
-                        const uint64_t NC = ffma2(A, YC, XC), NS = ffma2(A, YS, XS);
-                        XC = YC;
-                        XS = YS;
-                        YC = NC;
-                        YS = NS;
-                        if (neg) {
-                            PR[k] = fsub2(PR[k], YC);
-                            PI[k] = fsub2(PI[k], YS);
-                        } else {
-                            PR[k] = fadd2(PR[k], YC);
-                            PI[k] = fadd2(PI[k], YS);
-                        }
-                    }
-                }
-        
+                vertex_form_lane<S>(sRec[warp][i].f, fm0, fm0sq, eps_lane, PR, PI);
             } else if ((ms >> i) & 1u) {
                 // ---------------- series / edge forms: per sample ----------------
-                const bool series = (mser >> i) & 1u;
-                const float *R = sRec[warp][i].f;
-    #pragma unroll
-                for (int j = 0; j < S; ++j) {
-                    float dr, di;
-                    series_edge_term(R, series, (float)(m0 + j), K, dr, di);
-                    // into sample j's half of its pair
-                    const uint64_t DR = (j & 1) ? pk2(0.f, dr) : pk2(dr, 0.f);
-                    const uint64_t DI = (j & 1) ? pk2(0.f, di) : pk2(di, 0.f);
-                    PR[j >> 1] = fadd2(PR[j >> 1], DR);
-                    PI[j >> 1] = fadd2(PI[j >> 1], DI);
-                }
-        
+                series_edge_lane<S>(sRec[warp][i].f, (mser >> i) & 1u, fm0, 1.f, 0.f, K, PR, PI);
             }
         }
         // ---------------- Kahan-compensated tile accumulation ----------------
 #pragma unroll
         for (int k = 0; k < S2; ++k) {
-            uint64_t sr = sAcc[warp][0][k][lane], si = sAcc[warp][1][k][lane];
-            uint64_t cr = sAcc[warp][2][k][lane], ci = sAcc[warp][3][k][lane];
-            uint64_t y = fsub2(PR[k], cr);
-            uint64_t t = fadd2(sr, y);
-            cr = fsub2(fsub2(t, sr), y);
-            sr = t;
-            y = fsub2(PI[k], ci);
-            t = fadd2(si, y);
-            ci = fsub2(fsub2(t, si), y);
-            si = t;
-            sAcc[warp][0][k][lane] = sr;
-            sAcc[warp][1][k][lane] = si;
-            sAcc[warp][2][k][lane] = cr;
-            sAcc[warp][3][k][lane] = ci;
+            kahan_pair(sAcc[warp][0][k][lane], sAcc[warp][2][k][lane], PR[k]);
+            kahan_pair(sAcc[warp][1][k][lane], sAcc[warp][3][k][lane], PI[k]);
             PR[k] = PI[k] = zero2;
         }
         __syncwarp();
