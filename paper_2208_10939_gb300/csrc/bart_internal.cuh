@@ -114,29 +114,20 @@ void launch_build_facets(const MeshDesc *meshes, const InstDev *insts, int n_ins
                          FacetRec *fac, float *aabb, float *vel32, unsigned int *bounds,
                          double *ref64, float *ref32, float *fac_lo, unsigned int *box,
                          cudaStream_t s);
-void launch_morton(const FacetRec *fac, int64_t F, const unsigned int *bounds,
-                   uint32_t *keys, int32_t *vals, cudaStream_t s);
-// Stable LSD radix sort of (key, value) pairs on the low `bits` bits.
-// Temp buffers sized by radix_sort_temp_words(n).
+// Temp words of the multi-launch radix sort, and float4 words of the leaf
+// levels, for n facets.
 int64_t radix_sort_temp_words(int64_t n);
-void radix_sort_pairs(uint32_t *keys, int32_t *vals, uint32_t *keys_tmp, int32_t *vals_tmp,
-                      uint32_t *temp, int64_t n, int bits, cudaStream_t s);
-void launch_lbvh_build(const uint32_t *keys, const int32_t *vals, int64_t n,
-                       BvhNode *nodes, int32_t *parent, int32_t *leaf_parent,
-                       cudaStream_t s);
-// Batched scenes (facets [foff[b], foff[b+1]) form scene b, foff on the
-// device): Morton codes, a sort by (scene, code), and one hierarchy whose
-// scene subtrees are disjoint; root[b] receives scene b's root node (~facet
-// for a one-facet scene).  mkeys, skeys: F words of scratch.
-void launch_lbvh_batched(const FacetRec *fac, int64_t F, const unsigned int *bounds,
-                         const int64_t *foff, int B, uint32_t *keys, int32_t *vals,
-                         uint32_t *keys_tmp, int32_t *vals_tmp, uint32_t *temp, uint32_t *mkeys,
-                         uint32_t *skeys, BvhNode *nodes, int32_t *parent, int32_t *leaf_parent,
-                         int32_t *root, cudaStream_t s);
-int lbvh_batched_launches(int B);
-void launch_lbvh_refit(const int32_t *vals, const float *aabb, int64_t n, BvhNode *nodes,
-                       const int32_t *parent, const int32_t *leaf_parent, int32_t *flags,
-                       cudaStream_t s);
+int64_t leaf_levels_words(int64_t n);
+// Morton codes, sort, hierarchy and boxes; returns the launches.  Batched
+// scenes (B > 1: facets [foff[b], foff[b+1]) form scene b, foff on the
+// device): sorted by (scene, code), one hierarchy whose scene subtrees are
+// disjoint, root[b] scene b's root node (~facet for a one-facet scene).
+// mkeys, skeys: F words of scratch for B > 1; ticket: one int, zero before
+// and after.
+int launch_lbvh(const FacetRec *fac, const float *aabb, int64_t F, const unsigned int *bounds,
+                const int64_t *foff, int B, uint32_t *keys, int32_t *vals, uint32_t *keys_tmp,
+                int32_t *vals_tmp, uint32_t *temp, uint32_t *mkeys, uint32_t *skeys, float4 *levels,
+                int *ticket, BvhNode *nodes, int32_t *root, cudaStream_t s);
 
 // ---- visibility (visibility.cu) ----
 // order: facet ids in the sequence the ray threads take them (Morton order), or NULL.

@@ -147,7 +147,8 @@ struct bart_ctx {
     DevBuf<uint32_t> keys, keys_tmp, sort_temp;
     DevBuf<int32_t> vals, vals_tmp;
     DevBuf<BvhNode> nodes;
-    DevBuf<int32_t> parent, leaf_parent, flags;
+    DevBuf<float4> levels;              // boxes of runs of the sorted leaves
+    DevBuf<int> ticket;                 // block counter of their kernel, zero between frames
     DevBuf<uint8_t> state;
     DevBuf<int32_t> blk_cnt, vis_idx, vis_cnt;
     DevBuf<float4> kin;                 // kinematics Taylor rows [A][F][9]
@@ -267,8 +268,8 @@ struct bart_ctx {
         bounds.release();
         ref64.release(); ref32.release();
         keys.release(); keys_tmp.release(); sort_temp.release(); vals.release();
-        vals_tmp.release(); nodes.release(); parent.release(); leaf_parent.release();
-        flags.release(); state.release(); blk_cnt.release(); vis_idx.release();
+        vals_tmp.release(); nodes.release(); levels.release(); ticket.release();
+        state.release(); blk_cnt.release(); vis_idx.release();
         box.release(); band_tab.release(); band_ws.release(); d_ioff.release(); d_sinst.release();
         band_coarse.release();
         vis_cnt.release(); kin.release(); kquad.release(); partial.release(); item_off.release();
@@ -393,11 +394,13 @@ int bart_create(bart_ctx **out, int device)
     int rc = c->counters.ensure(5, "counters");
     if (rc == BART_OK) rc = c->status.ensure(1, "status");
     if (rc == BART_OK) rc = c->bounds.ensure(6, "bounds");
+    if (rc == BART_OK) rc = c->ticket.ensure(1, "ticket");
     if (rc != BART_OK) {
         delete c;
         return rc;
     }
     cudaError_t e = cudaMemset(c->status.p, 0, sizeof(int));
+    if (e == cudaSuccess) e = cudaMemset(c->ticket.p, 0, sizeof(int));
     if (e != cudaSuccess) {
         delete c;
         return cuda_fail(e, "cudaMemset");
@@ -756,9 +759,7 @@ static int run_frame(bart_ctx *ctx, double t0, int32_t path, void *adc, int32_t 
     BART_TRY(ctx->vals_tmp.ensure(F, "sort values"));
     BART_TRY(ctx->sort_temp.ensure(radix_sort_temp_words(F), "sort histogram"));
     BART_TRY(ctx->nodes.ensure(F > 1 ? F - 1 : 1, "bvh nodes"));
-    BART_TRY(ctx->parent.ensure(F > 1 ? F - 1 : 1, "bvh parents"));
-    BART_TRY(ctx->leaf_parent.ensure(F, "bvh leaf parents"));
-    BART_TRY(ctx->flags.ensure(F > 1 ? F - 1 : 1, "bvh refit flags"));
+    BART_TRY(ctx->levels.ensure((size_t)leaf_levels_words(F), "bvh leaf levels"));
     BART_TRY(ctx->state.ensure((size_t)A * F, "visibility states"));
     BART_TRY(ctx->blk_cnt.ensure(compact_blk_words(F, O + A), "compaction counts"));
     BART_TRY(ctx->vis_idx.ensure((size_t)(O + A) * F, "lit facet lists"));
@@ -994,26 +995,15 @@ static int run_frame(bart_ctx *ctx, double t0, int32_t path, void *adc, int32_t 
         // 2. LBVH (batched scenes: one hierarchy with a subtree per scene)
         SceneSplit split;
         nv.next("bart bvh");
+        launches += launch_lbvh(ctx->fac.p, ctx->aabb.p, F, ctx->bounds.p, ctx->d_foff.p, B,
+                                ctx->keys.p, ctx->vals.p, ctx->keys_tmp.p, ctx->vals_tmp.p,
+                                ctx->sort_temp.p, ctx->mkeys.p, ctx->skeys.p, ctx->levels.p,
+                                ctx->ticket.p, ctx->nodes.p, ctx->d_root.p, s);
         if (B > 1) {
-            launch_lbvh_batched(ctx->fac.p, F, ctx->bounds.p, ctx->d_foff.p, B, ctx->keys.p,
-                                ctx->vals.p, ctx->keys_tmp.p, ctx->vals_tmp.p, ctx->sort_temp.p,
-                                ctx->mkeys.p, ctx->skeys.p, ctx->nodes.p, ctx->parent.p,
-                                ctx->leaf_parent.p, ctx->d_root.p, s);
-            launches += lbvh_batched_launches(B);
             split.B = B;
             split.foff = ctx->d_foff.p;
             split.root = ctx->d_root.p;
-        } else {
-            launch_morton(ctx->fac.p, F, ctx->bounds.p, ctx->keys.p, ctx->vals.p, s);
-            radix_sort_pairs(ctx->keys.p, ctx->vals.p, ctx->keys_tmp.p, ctx->vals_tmp.p,
-                             ctx->sort_temp.p, F, 30, s);
-            launch_lbvh_build(ctx->keys.p, ctx->vals.p, F, ctx->nodes.p, ctx->parent.p,
-                              ctx->leaf_parent.p, s);
-            launches += 1 + 3 * 4 + (F >= 2 ? 1 : 0);
         }
-        launch_lbvh_refit(ctx->vals.p, ctx->aabb.p, F, ctx->nodes.p, ctx->parent.p,
-                          ctx->leaf_parent.p, ctx->flags.p, s);
-        launches += F >= 2 ? 1 : 0;
         if (tm) CUDA_TRY(cudaEventRecord(ctx->ev[2], s), "cudaEventRecord");
         // 3. visibility + per-channel lit lists (+ their per-scene ranges)
         nv.next("bart visibility");
