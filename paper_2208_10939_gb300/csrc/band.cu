@@ -567,15 +567,19 @@ synth_band_kernel(SynthArgs A, MixConsts K, BandArgs b)
     {
         const float nf = b.nodes[chirps.node0 + node];
         const float slot = fmaf(nf, (float)A.rd.slots, A.rd.tdm ? (float)tx : 0.f);   // exact
-        w.sl = slot;
-        w.tau_s = slot - K.s_mid;
         w.tn = slot * K.tc;
-        w.kin_t = A.kin + (int64_t)tx * F * kKinRow;
-        w.kin_r = A.kin + (int64_t)(P + rx) * F * kKinRow;
-        w.quad_t = A.kquad + (int64_t)tx * F * kKinQuadWords;
-        w.quad_r = A.kquad + (int64_t)(P + rx) * F * kKinQuadWords;
         w.ant_t = tx;
         w.ant_r = P + rx;
+        const double t = (double)slot * A.rd.Tc;
+#pragma unroll
+        for (int r = 0; r < 3; ++r) {
+            const double vt = A.vel64[3 * inst + r] * t;
+            const double xt = A.rd.ant[tx][r] - vt, xr = A.rd.ant[P + rx][r] - vt;
+            w.ath[r] = (float)xt;
+            w.atl[r] = (float)(xt - (double)w.ath[r]);
+            w.arh[r] = (float)xr;
+            w.arl[r] = (float)(xr - (double)w.arh[r]);
+        }
         w.d = d;
         // with the reference off, the steps' angles lie about 0, where the
         // recurrence's rounding grows fastest (as the square of the steps);
@@ -583,11 +587,6 @@ synth_band_kernel(SynthArgs A, MixConsts K, BandArgs b)
         // turn; lanes start at whole turns, and band_reduce_kernel turns back
         w.turn = pl.rotate ? 0.125f : 0.f;
         w.ref = b.refn[(int64_t)it.v * b.sh.N + node];
-#pragma unroll
-        for (int r = 0; r < 3; ++r) {
-            w.ptx[r] = K.ant[tx][r];
-            w.prx[r] = K.ant[P + rx][r];
-        }
     }
     uint64_t PR[S2], PI[S2];
 #pragma unroll

@@ -830,6 +830,7 @@ static int run_frame(bart_ctx *ctx, double t0, int32_t path, void *adc, int32_t 
     BandArgs bt{};
     const bool mixed_rows = path == BART_PATH_MIXED || path == BART_PATH_SPECTRAL ||
                             path == kPathAdjointMixed;
+    const bool kin_rows = mixed_rows && (!band || stats);
     if (path == BART_PATH_SPECTRAL && ctx->spec_M != rd.M) {
         std::vector<float> tab(2 * (size_t)rd.M);
         spectral_tables(rd.M, tab.data());
@@ -842,8 +843,12 @@ static int run_frame(bart_ctx *ctx, double t0, int32_t path, void *adc, int32_t 
     if (mixed_rows) {
         // kinematics: Taylor rows of R(t) per antenna and facet (one launch,
         // evaluated per record inside the synthesis)
-        BART_TRY(ctx->kin.ensure((size_t)A * F * kKinRowWords, "kinematics rows"));
-        BART_TRY(ctx->kquad.ensure((size_t)A * F * kKinQuadWords, "kinematics quadratics"));
+        // (the band-limited path forms its paths itself; its record counts,
+        // on request, are of the rows' records)
+        if (kin_rows) {
+            BART_TRY(ctx->kin.ensure((size_t)A * F * kKinRowWords, "kinematics rows"));
+            BART_TRY(ctx->kquad.ensure((size_t)A * F * kKinQuadWords, "kinematics quadratics"));
+        }
         if (band) {
             if (ctx->band_sh.N != rd.N || ctx->band_sh.M != rd.M) {
                 BandShape sh;
@@ -987,8 +992,9 @@ static int run_frame(bart_ctx *ctx, double t0, int32_t path, void *adc, int32_t 
                 launches += 2;
             }
             if (tm) CUDA_TRY(cudaEventRecord(ctx->ev_kin[0], ctx->side), "cudaEventRecord");
-            launch_kin_coef(ctx->c64.p, ctx->fac.p, ctx->vel64.p, ctx->ref64.p, F, rd, ctx->kin.p,
-                            ctx->kquad.p, ctx->side);
+            if (kin_rows)
+                launch_kin_coef(ctx->c64.p, ctx->fac.p, ctx->vel64.p, ctx->ref64.p, F, rd, ctx->kin.p,
+                                ctx->kquad.p, ctx->side);
             if (tm) CUDA_TRY(cudaEventRecord(ctx->ev_kin[1], ctx->side), "cudaEventRecord");
             CUDA_TRY(cudaEventRecord(ctx->join_ev, ctx->side), "cudaEventRecord");
         }
@@ -1109,7 +1115,7 @@ static int run_frame(bart_ctx *ctx, double t0, int32_t path, void *adc, int32_t 
             }
             if (tm) CUDA_TRY(cudaEventRecord(ctx->ev_syn[1], s), "cudaEventRecord");
             ctx->chunks = 1;
-            launches += band ? (stats ? 8 : 7) : 4;
+            launches += band ? (stats ? 8 : 6) : 4;
         } else if (path == BART_PATH_SPECTRAL) {
             a.kin = ctx->kin.p;
             a.kquad = ctx->kquad.p;

@@ -47,7 +47,7 @@ __device__ __forceinline__ void two_sum(float a, float b, float &s, float &e)
 // its double-float residual h = 1 - |d|^2 r0^2 (|h| ~ 1e-7, so the step
 // leaves ~h^2), then d r
 __device__ __forceinline__ void df_unit(const float sh[3], const float sl[3], float uh[3],
-                                        float ul[3])
+                                        float ul[3], float *Rh = nullptr, float *Rl = nullptr)
 {
     float p[3], pe = 0.f, cross = 0.f;
 #pragma unroll
@@ -70,6 +70,12 @@ __device__ __forceinline__ void df_unit(const float sh[3], const float sl[3], fl
     for (int r = 0; r < 3; ++r) {
         uh[r] = __fmul_rn(sh[r], r0);
         ul[r] = __fmaf_rn(sh[r], r0, -uh[r]) + (sh[r] * rl + sl[r] * r0);
+    }
+    if (Rh) {            // and the length: q r0 and one Newton step on its residual
+        const float R0 = __fmul_rn(qh, r0);
+        const float c = 0.5f * r0 * (__fmaf_rn(-R0, R0, qh) + ql);
+        *Rh = __fadd_rn(R0, c);
+        *Rl = __fsub_rn(c, __fsub_rn(*Rh, R0));
     }
 }
 
@@ -186,8 +192,11 @@ struct MixRow {
     int ant_t, ant_r;                // antenna indices of the row's TX and RX
     float tau_s, tn;                 // slot offset from the expansion point; chirp start (s)
     float ptx[3], prx[3];            // antenna positions
-    // band rows only (see band.cuh): the reference phase taken off the record
-    // (ph0, hi, lo, p2 as in RecM) and the spacing of the row's samples
+    // band rows only (see band.cuh; they use neither the kinematics rows nor
+    // ptx, prx): antenna less v t_n as float pairs, v the instance's velocity;
+    // the reference phase taken off the record (ph0, hi, lo, p2 as in RecM);
+    // the spacing of the row's samples
+    float ath[3], atl[3], arh[3], arl[3];
     float4 ref;
     float d;
     float turn;                      // cycles added to each step
@@ -201,50 +210,97 @@ __device__ __forceinline__ int build_mixed_record(const SynthArgs &A, const MixC
     const FacetRec fr = A.fac[k];
     const float4 vv = reinterpret_cast<const float4 *>(A.vel32)[fr.inst];
     float4 kt, kr;
-    kin_eval2(w.kin_t + (int64_t)k * kKinRow, w.kin_r + (int64_t)k * kKinRow,
-              w.quad_t + kKinQuadWords * (int64_t)k, w.quad_r + kKinQuadWords * (int64_t)k,
-              w.sl, w.tau_s, A.rd.Tc, K.f0c_d, K.mu_f0_d, K.mfh, K.mfl, kt, kr);
-    // directions t, r and the amplitude's ranges: from the facet
-    // centroid, or (far field) from the instance origin, whose
-    // plane waves every facet of the instance sees
-    // The origin o(t_n) = o0 + v t_n is never formed in FP32: at tens of
-    // metres its rounding would repeat with the instance's per-chirp step
-    // v T_c (the same for every facet of the instance, so coherent across
-    // them: a Doppler spur).  Each direction is normalised from the
-    // constant B = p - o0 and the small D = -v t_n instead.
     float th[3], rh[3], Rt, Rr;
-    const float D[3] = {-vv.x * w.tn, -vv.y * w.tn, -vv.z * w.tn};
-    float o0[3];
-    if (A.rd.far_field) {
-        const float4 rf = reinterpret_cast<const float4 *>(A.ref32)[fr.inst];
-        o0[0] = rf.x; o0[1] = rf.y; o0[2] = rf.z;
+    float uth[3], utl[3], urh[3], url[3];    // band rows: unit vectors as float pairs
+    if constexpr (BAND) {
+        // paths and directions straight from a - c in double-float: as many
+        // operations as evaluating the Taylor rows, without their 288 bytes
+        // a record and the FP64 kernel that makes them (which took 3.1 ms
+        // beside an intersection frame's hierarchy and slowed it to 3.3 ms)
+        const float *cl = A.fac_lo + 12 * (int64_t)k;
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            float sh[3], sl[3], Rh, Rl;
+#pragma unroll
+            for (int r = 0; r < 3; ++r) {
+                float er;
+                two_sum(e == 0 ? w.ath[r] : w.arh[r], -fr.c[r], sh[r], er);
+                sl[r] = er + ((e == 0 ? w.atl[r] : w.arl[r]) - cl[r]);
+            }
+            df_unit(sh, sl, e == 0 ? uth : urh, e == 0 ? utl : url, &Rh, &Rl);
+            const float ph = __fmul_rn(Rh, K.f0c);
+            const float pl = __fmaf_rn(Rh, K.f0c, -ph) + (Rh * K.f0c_lo + Rl * K.f0c);
+            const float xh = __fadd_rn(ph, pl), xl = __fsub_rn(pl, __fsub_rn(xh, ph));
+            (e == 0 ? kt : kr) = kin_finish(xh, xl, Rh, K.mfh, K.mfl);
+        }
+        Rt = kt.w;
+        Rr = kr.w;
+        if (exact_u) {
+#pragma unroll
+            for (int r = 0; r < 3; ++r) {
+                th[r] = uth[r];
+                rh[r] = urh[r];
+            }
+        } else {                             // a static instance's: FP32, as below with D = 0
+            float Bt[3], Br[3];
+#pragma unroll
+            for (int r = 0; r < 3; ++r) {
+                Bt[r] = w.ath[r] - fr.c[r];
+                Br[r] = w.arh[r] - fr.c[r];
+            }
+            const float it = rsqrtf(Bt[0] * Bt[0] + Bt[1] * Bt[1] + Bt[2] * Bt[2]);
+            const float ir = rsqrtf(Br[0] * Br[0] + Br[1] * Br[1] + Br[2] * Br[2]);
+#pragma unroll
+            for (int r = 0; r < 3; ++r) {
+                th[r] = Bt[r] * it;
+                rh[r] = Br[r] * ir;
+            }
+        }
     } else {
-        o0[0] = fr.c[0]; o0[1] = fr.c[1]; o0[2] = fr.c[2];
-    }
-    {
-        float Bt[3], Br[3];
-#pragma unroll
-        for (int r = 0; r < 3; ++r) {
-            Bt[r] = w.ptx[r] - o0[r];
-            Br[r] = w.prx[r] - o0[r];
-        }
-        const float dd = D[0] * D[0] + D[1] * D[1] + D[2] * D[2];
-        const float qt = (Bt[0] * Bt[0] + Bt[1] * Bt[1] + Bt[2] * Bt[2]) +
-                         fmaf(2.f, Bt[0] * D[0] + Bt[1] * D[1] + Bt[2] * D[2], dd);
-        const float qr = (Br[0] * Br[0] + Br[1] * Br[1] + Br[2] * Br[2]) +
-                         fmaf(2.f, Br[0] * D[0] + Br[1] * D[1] + Br[2] * D[2], dd);
-        const float it = rsqrtf(qt), ir = rsqrtf(qr);
-#pragma unroll
-        for (int r = 0; r < 3; ++r) {
-            th[r] = fmaf(Bt[r], it, D[r] * it);
-            rh[r] = fmaf(Br[r], ir, D[r] * ir);
-        }
+        kin_eval2(w.kin_t + (int64_t)k * kKinRow, w.kin_r + (int64_t)k * kKinRow,
+                  w.quad_t + kKinQuadWords * (int64_t)k, w.quad_r + kKinQuadWords * (int64_t)k,
+                  w.sl, w.tau_s, A.rd.Tc, K.f0c_d, K.mu_f0_d, K.mfh, K.mfl, kt, kr);
+        // directions t, r and the amplitude's ranges: from the facet
+        // centroid, or (far field) from the instance origin, whose
+        // plane waves every facet of the instance sees
+        // The origin o(t_n) = o0 + v t_n is never formed in FP32: at tens of
+        // metres its rounding would repeat with the instance's per-chirp step
+        // v T_c (the same for every facet of the instance, so coherent across
+        // them: a Doppler spur).  Each direction is normalised from the
+        // constant B = p - o0 and the small D = -v t_n instead.
+        const float D[3] = {-vv.x * w.tn, -vv.y * w.tn, -vv.z * w.tn};
+        float o0[3];
         if (A.rd.far_field) {
-            Rt = qt * it;
-            Rr = qr * ir;
+            const float4 rf = reinterpret_cast<const float4 *>(A.ref32)[fr.inst];
+            o0[0] = rf.x; o0[1] = rf.y; o0[2] = rf.z;
         } else {
-            Rt = kt.w;
-            Rr = kr.w;
+            o0[0] = fr.c[0]; o0[1] = fr.c[1]; o0[2] = fr.c[2];
+        }
+        {
+            float Bt[3], Br[3];
+#pragma unroll
+            for (int r = 0; r < 3; ++r) {
+                Bt[r] = w.ptx[r] - o0[r];
+                Br[r] = w.prx[r] - o0[r];
+            }
+            const float dd = D[0] * D[0] + D[1] * D[1] + D[2] * D[2];
+            const float qt = (Bt[0] * Bt[0] + Bt[1] * Bt[1] + Bt[2] * Bt[2]) +
+                             fmaf(2.f, Bt[0] * D[0] + Bt[1] * D[1] + Bt[2] * D[2], dd);
+            const float qr = (Br[0] * Br[0] + Br[1] * Br[1] + Br[2] * Br[2]) +
+                             fmaf(2.f, Br[0] * D[0] + Br[1] * D[1] + Br[2] * D[2], dd);
+            const float it = rsqrtf(qt), ir = rsqrtf(qr);
+#pragma unroll
+            for (int r = 0; r < 3; ++r) {
+                th[r] = fmaf(Bt[r], it, D[r] * it);
+                rh[r] = fmaf(Br[r], ir, D[r] * ir);
+            }
+            if (A.rd.far_field) {
+                Rt = qt * it;
+                Rr = qr * ir;
+            } else {
+                Rt = kt.w;
+                Rr = kr.w;
+            }
         }
     }
     float b[3];
@@ -271,7 +327,7 @@ __device__ __forceinline__ int build_mixed_record(const SynthArgs &A, const MixC
     {
         float ut[3] = {th[0], th[1], th[2]}, ur[3] = {rh[0], rh[1], rh[2]};
         float Rtp = Rt, Rrp = Rr;
-        if (A.rd.delay_ref) {
+        if (!BAND && A.rd.delay_ref) {
             const float4 rf = reinterpret_cast<const float4 *>(A.ref32)[fr.inst];
             const float ox = fmaf(vv.x, w.tn, rf.x), oy = fmaf(vv.y, w.tn, rf.y),
                         oz = fmaf(vv.z, w.tn, rf.z);
@@ -321,45 +377,53 @@ __device__ __forceinline__ int build_mixed_record(const SynthArgs &A, const MixC
         exact_u || K.f0c * fmaxf(fmaxf(fabsf(u[0]), fabsf(u[1])), fabsf(u[2])) > 64.f;
     if (large) {
         const float *res = A.fac_lo + 12 * (int64_t)k;
-        // the origin of the directions at the chirp start: the centroid,
-        // or (far field) the instance origin
-        float oh[3], ol[3];
-        if (A.rd.far_field) {
-            const float4 rf = reinterpret_cast<const float4 *>(A.ref32)[fr.inst];
-            oh[0] = rf.x; oh[1] = rf.y; oh[2] = rf.z;
-#pragma unroll
-            for (int r = 0; r < 3; ++r)
-                ol[r] = (float)(A.ref64[3 * fr.inst + r] - (double)oh[r]);
-        } else {
-#pragma unroll
-            for (int r = 0; r < 3; ++r) {
-                oh[r] = fr.c[r];
-                ol[r] = res[r];
-            }
-        }
-        const float vel[3] = {vv.x, vv.y, vv.z};
         float bh[3] = {0.f, 0.f, 0.f}, bl[3] = {0.f, 0.f, 0.f};
-#pragma unroll
-        for (int e = 0; e < 2; ++e) {
-            const int ant = e == 0 ? w.ant_t : w.ant_r;
-            float sh[3], sl[3];
+        if constexpr (BAND) {
 #pragma unroll
             for (int r = 0; r < 3; ++r) {
-                // antenna - origin - v t_n, as sh + sl
-                float d1, e1, d2, e2;
-                two_sum(K.ant[ant][r], -oh[r], d1, e1);
-                two_sum(d1, -(vel[r] * w.tn), d2, e2);
-                sh[r] = d2;
-                sl[r] = (e1 + e2) + (K.ant_lo[ant][r] - ol[r]);
+                two_sum(uth[r], urh[r], bh[r], bl[r]);
+                bl[r] = utl[r] + url[r] + bl[r];
             }
-            float th_[3], tl_[3];
-            df_unit(sh, sl, th_, tl_);
+        } else {
+            // the origin of the directions at the chirp start: the centroid,
+            // or (far field) the instance origin
+            float oh[3], ol[3];
+            if (A.rd.far_field) {
+                const float4 rf = reinterpret_cast<const float4 *>(A.ref32)[fr.inst];
+                oh[0] = rf.x; oh[1] = rf.y; oh[2] = rf.z;
 #pragma unroll
-            for (int r = 0; r < 3; ++r) {
-                float s_, e_;
-                two_sum(bh[r], th_[r], s_, e_);
-                bh[r] = s_;
-                bl[r] = bl[r] + tl_[r] + e_;
+                for (int r = 0; r < 3; ++r)
+                    ol[r] = (float)(A.ref64[3 * fr.inst + r] - (double)oh[r]);
+            } else {
+#pragma unroll
+                for (int r = 0; r < 3; ++r) {
+                    oh[r] = fr.c[r];
+                    ol[r] = res[r];
+                }
+            }
+            const float vel[3] = {vv.x, vv.y, vv.z};
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const int ant = e == 0 ? w.ant_t : w.ant_r;
+                float sh[3], sl[3];
+#pragma unroll
+                for (int r = 0; r < 3; ++r) {
+                    // antenna - origin - v t_n, as sh + sl
+                    float d1, e1, d2, e2;
+                    two_sum(K.ant[ant][r], -oh[r], d1, e1);
+                    two_sum(d1, -(vel[r] * w.tn), d2, e2);
+                    sh[r] = d2;
+                    sl[r] = (e1 + e2) + (K.ant_lo[ant][r] - ol[r]);
+                }
+                float th_[3], tl_[3];
+                df_unit(sh, sl, th_, tl_);
+#pragma unroll
+                for (int r = 0; r < 3; ++r) {
+                    float s_, e_;
+                    two_sum(bh[r], th_[r], s_, e_);
+                    bh[r] = s_;
+                    bl[r] = bl[r] + tl_[r] + e_;
+                }
             }
         }
 #pragma unroll
