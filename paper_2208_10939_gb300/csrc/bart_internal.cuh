@@ -77,6 +77,13 @@ struct __align__(16) BvhNode {
 };
 static_assert(sizeof(BvhNode) == 64, "BvhNode layout");
 
+// Four-wide node of the visibility rays (see lbvh_widen_kernel): the slots'
+// box corners, the child code (as in BvhNode) in lo.w.
+struct __align__(16) WideNode {
+    float4 lo[4], hi[4];
+};
+static_assert(sizeof(WideNode) == 128, "WideNode layout");
+
 struct MeshDesc {
     const double *verts;
     const int32_t *tris;
@@ -100,7 +107,9 @@ constexpr int kStatusWaitTimeout = 2;   // a bounded device wait expired (see ba
 
 // ---- scene + BVH (scene_bvh.cu) ----
 // tri32: per facet 12 floats -- the world vertices rounded to FP32 and the
-// largest |coordinate| among them (for the visibility FP32 pre-test);
+// largest |coordinate| among them (for the double-bounce legs' FP32 pre-test;
+// may be NULL); trel: per facet 3 float4, the first vertex, the edges from it
+// and the vertex's residue (mt_rel_classify, for the visibility pre-test);
 // fac_lo: per facet 12 floats, the rounding residues of the FP32 centroid
 // and vertex offsets in FacetRec (c - (double)rec.c, dv - (double)rec.dv),
 // so that c and dv are available as double-float pairs
@@ -110,8 +119,8 @@ constexpr int kStatusWaitTimeout = 2;   // a bounded device wait expired (see ba
 // the world-facet kernel (its t0 argument is updated in replayed frame graphs)
 const void *build_facets_kernel_fn(int *t0_arg_index, int *n_args);
 void launch_build_facets(const MeshDesc *meshes, const InstDev *insts, int n_inst,
-                         int64_t F, double t0, double *tri64, float *tri32, double *c64,
-                         FacetRec *fac, float *aabb, float *vel32, unsigned int *bounds,
+                         int64_t F, double t0, double *tri64, float *tri32, float4 *trel,
+                         double *c64, FacetRec *fac, float *aabb, float *vel32, unsigned int *bounds,
                          double *ref64, float *ref32, float *fac_lo, unsigned int *box,
                          cudaStream_t s);
 // Temp words of the multi-launch radix sort, and float4 words of the leaf
@@ -127,7 +136,7 @@ int64_t leaf_levels_words(int64_t n);
 int launch_lbvh(const FacetRec *fac, const float *aabb, int64_t F, const unsigned int *bounds,
                 const int64_t *foff, int B, uint32_t *keys, int32_t *vals, uint32_t *keys_tmp,
                 int32_t *vals_tmp, uint32_t *temp, uint32_t *mkeys, uint32_t *skeys, float4 *levels,
-                int *ticket, BvhNode *nodes, int32_t *root, cudaStream_t s);
+                int *ticket, BvhNode *nodes, WideNode *wide, int32_t *root, cudaStream_t s);
 
 // ---- visibility (visibility.cu) ----
 // order: facet ids in the sequence the ray threads take them (Morton order), or NULL.
@@ -138,9 +147,9 @@ struct SceneSplit {
     const int64_t *foff = nullptr;
     const int32_t *root = nullptr;
 };
-void launch_visibility(const double *tri64, const float *tri32, const double *c64,
-                       const FacetRec *fac, const double *ref64, const BvhNode *nodes,
-                       const int32_t *order, int64_t F, const RadarDev &rd,
+void launch_visibility(const double *tri64, const float4 *trel, const double *c64,
+                       const FacetRec *fac, const float *fac_lo, const double *ref64,
+                       const WideNode *nodes, const int32_t *order, int64_t F, const RadarDev &rd,
                        const SceneSplit &sc, uint8_t *state, unsigned long long *n_graze,
                        int *status, cudaStream_t s);
 // lists 0..O-1: facets lit from both antennas of each channel; O..O+A-1: facets

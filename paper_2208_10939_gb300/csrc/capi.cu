@@ -137,7 +137,9 @@ struct bart_ctx {
     DevBuf<MeshDesc> d_meshes;
     DevBuf<InstDev> d_insts;
     DevBuf<double> tri64, c64, vel64;
-    DevBuf<float> tri32;
+    DevBuf<float> tri32;                // only with double bounce
+    DevBuf<float4> trel;
+    DevBuf<WideNode> wide;
     DevBuf<float> vel32, aabb;
     DevBuf<double> ref64;               // instance origins at t0 (delay reference points)
     DevBuf<float> ref32;
@@ -263,7 +265,7 @@ struct bart_ctx {
             m->rho.release();
             delete m;
         }
-        d_meshes.release(); d_insts.release(); tri64.release(); tri32.release(); c64.release();
+        d_meshes.release(); d_insts.release(); tri64.release(); tri32.release(); trel.release(); wide.release(); c64.release();
         vel64.release(); vel32.release(); aabb.release(); fac.release(); fac_lo.release();
         bounds.release();
         ref64.release(); ref32.release();
@@ -741,7 +743,8 @@ static int run_frame(bart_ctx *ctx, double t0, int32_t path, void *adc, int32_t 
     BART_TRY(ctx->d_meshes.ensure(md.size(), "mesh table"));
     BART_TRY(ctx->d_insts.ensure(I, "instance table"));
     BART_TRY(ctx->tri64.ensure(9 * F, "facet vertices"));
-    BART_TRY(ctx->tri32.ensure(12 * F, "facet vertices (f32)"));
+    if (ctx->radar.double_bounce) BART_TRY(ctx->tri32.ensure(12 * F, "facet vertices (f32)"));
+    BART_TRY(ctx->trel.ensure(3 * F, "facet edges"));
     BART_TRY(ctx->c64.ensure(3 * F, "facet centroids"));
     BART_TRY(ctx->vel64.ensure(3 * I, "instance velocities"));
     BART_TRY(ctx->vel32.ensure(4 * I, "instance velocities (f32)"));
@@ -759,6 +762,7 @@ static int run_frame(bart_ctx *ctx, double t0, int32_t path, void *adc, int32_t 
     BART_TRY(ctx->vals_tmp.ensure(F, "sort values"));
     BART_TRY(ctx->sort_temp.ensure(radix_sort_temp_words(F), "sort histogram"));
     BART_TRY(ctx->nodes.ensure(F > 1 ? F - 1 : 1, "bvh nodes"));
+    BART_TRY(ctx->wide.ensure(F > 1 ? F - 1 : 1, "bvh wide nodes"));
     BART_TRY(ctx->levels.ensure((size_t)leaf_levels_words(F), "bvh leaf levels"));
     BART_TRY(ctx->state.ensure((size_t)A * F, "visibility states"));
     BART_TRY(ctx->blk_cnt.ensure(compact_blk_words(F, O + A), "compaction counts"));
@@ -948,8 +952,8 @@ static int run_frame(bart_ctx *ctx, double t0, int32_t path, void *adc, int32_t 
         // 1. world facets at t0
         Stages nv;
         nv.next("bart facets");
-        launch_build_facets(ctx->d_meshes.p, ctx->d_insts.p, I, F, t0v, ctx->tri64.p, ctx->tri32.p,
-                            ctx->c64.p, ctx->fac.p, ctx->aabb.p, ctx->vel32.p, ctx->bounds.p,
+        launch_build_facets(ctx->d_meshes.p, ctx->d_insts.p, I, F, t0v, ctx->tri64.p,
+                            bounce ? ctx->tri32.p : nullptr, ctx->trel.p, ctx->c64.p, ctx->fac.p, ctx->aabb.p, ctx->vel32.p, ctx->bounds.p,
                             ctx->ref64.p, ctx->ref32.p, ctx->fac_lo.p, ctx->box.p, s);
         launches += 1;
         if (tm) CUDA_TRY(cudaEventRecord(ctx->ev[1], s), "cudaEventRecord");
@@ -1004,7 +1008,7 @@ static int run_frame(bart_ctx *ctx, double t0, int32_t path, void *adc, int32_t 
         launches += launch_lbvh(ctx->fac.p, ctx->aabb.p, F, ctx->bounds.p, ctx->d_foff.p, B,
                                 ctx->keys.p, ctx->vals.p, ctx->keys_tmp.p, ctx->vals_tmp.p,
                                 ctx->sort_temp.p, ctx->mkeys.p, ctx->skeys.p, ctx->levels.p,
-                                ctx->ticket.p, ctx->nodes.p, ctx->d_root.p, s);
+                                ctx->ticket.p, ctx->nodes.p, ctx->wide.p, ctx->d_root.p, s);
         if (B > 1) {
             split.B = B;
             split.foff = ctx->d_foff.p;
@@ -1013,8 +1017,8 @@ static int run_frame(bart_ctx *ctx, double t0, int32_t path, void *adc, int32_t 
         if (tm) CUDA_TRY(cudaEventRecord(ctx->ev[2], s), "cudaEventRecord");
         // 3. visibility + per-channel lit lists (+ their per-scene ranges)
         nv.next("bart visibility");
-        launch_visibility(ctx->tri64.p, ctx->tri32.p, ctx->c64.p, ctx->fac.p, ctx->ref64.p,
-                          ctx->nodes.p,
+        launch_visibility(ctx->tri64.p, ctx->trel.p, ctx->c64.p, ctx->fac.p, ctx->fac_lo.p, ctx->ref64.p,
+                          ctx->wide.p,
                           F >= 2 ? ctx->vals.p : nullptr, F, rd, split, ctx->state.p,
                           ctx->counters.p + 3, ctx->status.p, s);
         launch_compact(ctx->state.p, F, rd, ctx->blk_cnt.p, ctx->vis_idx.p, ctx->vis_cnt.p, s);

@@ -45,7 +45,7 @@ __device__ __forceinline__ double world_coord(const double *r, double x, double 
 __global__ void build_facets_kernel(const MeshDesc *__restrict__ meshes,
                                     const InstDev *__restrict__ insts, int n_inst, int64_t F,
                                     double t0, double *__restrict__ tri64,
-                                    float *__restrict__ tri32,
+                                    float *__restrict__ tri32, float4 *__restrict__ trel,
                                     double *__restrict__ c64, FacetRec *__restrict__ fac,
                                     float *__restrict__ aabb, float *__restrict__ vel32,
                                     unsigned int *__restrict__ bounds,
@@ -79,12 +79,14 @@ __global__ void build_facets_kernel(const MeshDesc *__restrict__ meshes,
         for (int i = 0; i < 9; ++i) {
             tri64[9 * f + i] = v[i];
             const float vf = (float)v[i];
-            tri32[12 * f + i] = vf;
+            if (tri32) tri32[12 * f + i] = vf;
             vmax = fmaxf(vmax, fabsf(vf));
         }
-        tri32[12 * f + 9] = vmax;
-        tri32[12 * f + 10] = 0.f;
-        tri32[12 * f + 11] = 0.f;
+        if (tri32) {
+            tri32[12 * f + 9] = vmax;
+            tri32[12 * f + 10] = 0.f;
+            tri32[12 * f + 11] = 0.f;
+        }
         double c[3];
         for (int r = 0; r < 3; ++r) {
             c[r] = __ddiv_rn(__dadd_rn(__dadd_rn(v[r], v[3 + r]), v[6 + r]), 3.0);
@@ -92,6 +94,11 @@ __global__ void build_facets_kernel(const MeshDesc *__restrict__ meshes,
         }
         const double e1[3] = {v[3] - v[0], v[4] - v[1], v[5] - v[2]};
         const double e2[3] = {v[6] - v[0], v[7] - v[1], v[8] - v[2]};
+        const float h0 = (float)v[0], h1 = (float)v[1], h2 = (float)v[2];
+        trel[3 * f] = make_float4(h0, h1, h2, (float)e1[0]);
+        trel[3 * f + 1] = make_float4((float)e1[1], (float)e1[2], (float)e2[0], (float)e2[1]);
+        trel[3 * f + 2] = make_float4((float)e2[2], (float)(v[0] - (double)h0),
+                                      (float)(v[1] - (double)h1), (float)(v[2] - (double)h2));
         const double nx = e1[1] * e2[2] - e1[2] * e2[1];
         const double ny = e1[2] * e2[0] - e1[0] * e2[2];
         const double nz = e1[0] * e2[1] - e1[1] * e2[0];
@@ -180,13 +187,14 @@ __global__ void build_facets_kernel(const MeshDesc *__restrict__ meshes,
 
 const void *build_facets_kernel_fn(int *t0_arg_index, int *n_args)
 {
-    *t0_arg_index = 4;      // meshes, insts, n_inst, F, t0, tri64, tri32, c64, fac, aabb,
-    *n_args = 16;           // vel32, bounds, ref64, ref32, fac_lo, box
+    *t0_arg_index = 4;      // meshes, insts, n_inst, F, t0, tri64, tri32, trel, c64, fac, aabb,
+    *n_args = 17;           // vel32, bounds, ref64, ref32, fac_lo, box
     return reinterpret_cast<const void *>(build_facets_kernel);
 }
 
 void launch_build_facets(const MeshDesc *meshes, const InstDev *insts, int n_inst, int64_t F,
-                         double t0, double *tri64, float *tri32, double *c64, FacetRec *fac,
+                         double t0, double *tri64, float *tri32, float4 *trel, double *c64,
+                         FacetRec *fac,
                          float *aabb, float *vel32, unsigned int *bounds, double *ref64,
                          float *ref32, float *fac_lo, unsigned int *box, cudaStream_t s)
 {
@@ -198,7 +206,7 @@ void launch_build_facets(const MeshDesc *meshes, const InstDev *insts, int n_ins
     // a block: 19 us for 200 facets, 22 us for 20k)
     const int T = 64;
     const unsigned int G = (unsigned int)((F + T - 1) / T);
-    build_facets_kernel<<<G, T, 0, s>>>(meshes, insts, n_inst, F, t0, tri64, tri32, c64, fac,
+    build_facets_kernel<<<G, T, 0, s>>>(meshes, insts, n_inst, F, t0, tri64, tri32, trel, c64, fac,
                                         aabb, vel32, bounds, ref64, ref32, fac_lo, box);
 }
 
@@ -766,6 +774,40 @@ __global__ void lbvh_build_kernel(const uint32_t *__restrict__ keys,
     }
 }
 
+// Four-wide nodes for the visibility rays: wide node i holds the children of
+// binary node i's children (a leaf child stands for itself), so that a ray
+// makes half the dependent loads on its way down, each of four boxes.  Empty
+// slots have a point box out of any ray's reach.
+__global__ void lbvh_widen_kernel(const BvhNode *__restrict__ nodes, int64_t n,
+                                  WideNode *__restrict__ wide)
+{
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n - 1) return;
+    const BvhNode nd = nodes[i];
+    WideNode w;
+    int c = 0;
+    auto put = [&](const float *a, const float *b, int code) {
+        w.lo[c] = make_float4(a[0], a[1], a[2], __int_as_float(code));
+        w.hi[c++] = make_float4(b[0], b[1], b[2], 0.f);
+    };
+    auto side = [&](const float *a, const float *b, int code) {
+        if (code < 0) {
+            put(a, b, code);
+        } else {
+            const BvhNode m = nodes[code];
+            put(m.lmin, m.lmax, m.left);
+            put(m.rmin, m.rmax, m.right);
+        }
+    };
+    side(nd.lmin, nd.lmax, nd.left);
+    side(nd.rmin, nd.rmax, nd.right);
+    while (c < 4) {
+        const float far[3] = {1e30f, 1e30f, 1e30f};
+        put(far, far, 0);
+    }
+    wide[i] = w;
+}
+
 // scene of each sorted leaf: facets [foff[b], foff[b+1]) belong to scene b
 __global__ void scene_keys_kernel(const int32_t *__restrict__ vals, int64_t n,
                                   const int64_t *__restrict__ foff, int B,
@@ -794,7 +836,7 @@ __global__ void scene_root_init_kernel(const int64_t *__restrict__ foff, int B,
 int launch_lbvh(const FacetRec *fac, const float *aabb, int64_t F, const unsigned int *bounds,
                 const int64_t *foff, int B, uint32_t *keys, int32_t *vals, uint32_t *keys_tmp,
                 int32_t *vals_tmp, uint32_t *temp, uint32_t *mkeys, uint32_t *skeys, float4 *levels,
-                int *ticket, BvhNode *nodes, int32_t *root, cudaStream_t s)
+                int *ticket, BvhNode *nodes, WideNode *wide, int32_t *root, cudaStream_t s)
 {
     const int T = 256;
     const unsigned int G = (unsigned int)((F + T - 1) / T);
@@ -822,7 +864,8 @@ int launch_lbvh(const FacetRec *fac, const float *aabb, int64_t F, const unsigne
         vals, aabb, F, levels, ticket);
     lbvh_build_kernel<<<(unsigned int)((F - 1 + T - 1) / T), T, 0, s>>>(
         keys, B > 1 ? skeys : nullptr, vals, F, levels, nodes, root);
-    return launches + 2;
+    lbvh_widen_kernel<<<(unsigned int)((F - 1 + 127) / 128), 128, 0, s>>>(nodes, F, wide);
+    return launches + 3;
 }
 
 }  // namespace bart
