@@ -63,17 +63,42 @@ struct AntGroups {
 constexpr int kVisThreads = 128, kVisPairs = kVisThreads;    // at most, a block
 constexpr int kVisQuads = kVisThreads / 4;
 
+struct VisArgs {
+    const double *tri64;
+    const float4 *trel;
+    const double *c64;
+    const FacetRec *fac;
+    const float *fac_lo;
+    const double *ref64;
+    const WideNode *nodes;
+    const int32_t *order;
+    int64_t F;
+    RadarDev rd;
+    AntGroups ag;
+    SceneSplit sc;
+    int pairs;
+    uint8_t *state;
+    unsigned long long *n_graze;
+    int *status;
+};
+
 template <bool BUNDLE, bool FAR>
-__global__ void __launch_bounds__(kVisThreads)
-visibility_kernel(const double *__restrict__ tri64, const float4 *__restrict__ trel,
-                  const double *__restrict__ c64, const FacetRec *__restrict__ fac,
-                  const float *__restrict__ fac_lo, const double *__restrict__ ref64,
-                  const WideNode *__restrict__ nodes,
-                  const int32_t *__restrict__ order, int64_t F, RadarDev rd, AntGroups ag,
-                  SceneSplit sc, int pairs, uint8_t *__restrict__ state,
-                  unsigned long long *n_graze, int *status)
+__device__ __forceinline__ void visibility_pairs(const VisArgs &v)
 {
     constexpr float u24 = 5.9604645e-8f;
+    const double *__restrict__ tri64 = v.tri64, *__restrict__ c64 = v.c64, *__restrict__ ref64 = v.ref64;
+    const float4 *__restrict__ trel = v.trel;
+    const FacetRec *__restrict__ fac = v.fac;
+    const float *__restrict__ fac_lo = v.fac_lo;
+    const WideNode *__restrict__ nodes = v.nodes;
+    const int32_t *__restrict__ order = v.order;
+    uint8_t *__restrict__ state = v.state;
+    const int64_t F = v.F;
+    const RadarDev &rd = v.rd;
+    const AntGroups &ag = v.ag;
+    const SceneSplit &sc = v.sc;
+    const int pairs = v.pairs;
+    int *status = v.status;
     __shared__ int s_k[kVisPairs];
     __shared__ uint16_t s_live[kVisPairs], s_rev[kVisPairs], s_graze[kVisPairs];
     __shared__ int s_cnt[kVisThreads / 32], s_next;
@@ -386,7 +411,21 @@ visibility_kernel(const double *__restrict__ tri64, const float4 *__restrict__ t
         __syncwarp();
     }
     const int gz = __reduce_add_sync(0xffffffffu, n_graze_q);
-    if (lane == 0 && gz) atomicAdd(n_graze, (unsigned long long)gz);
+    if (lane == 0 && gz) atomicAdd(v.n_graze, (unsigned long long)gz);
+}
+
+__global__ void __launch_bounds__(kVisThreads) visibility_kernel(const __grid_constant__ VisArgs v)
+{
+    visibility_pairs<true, false>(v);
+}
+// one antenna a group: plain slabs
+__global__ void __launch_bounds__(kVisThreads) visibility_single_kernel(const __grid_constant__ VisArgs v)
+{
+    visibility_pairs<false, false>(v);
+}
+__global__ void __launch_bounds__(kVisThreads) visibility_far_kernel(const __grid_constant__ VisArgs v)
+{
+    visibility_pairs<true, true>(v);
 }
 
 // Antennas of a group: all TX or all RX of up to 16 where that leaves 32k
@@ -441,11 +480,11 @@ void launch_visibility(const double *tri64, const float4 *trel, const double *c6
     const int64_t all = F * ag.n_groups;
     const int pairs = all <= 16 * 1024 ? 32 : all <= 112 * 1024 ? 64 : kVisPairs;
     const dim3 grid((unsigned int)((F + pairs - 1) / pairs), (unsigned int)ag.n_groups);
-    const bool bundle = ag.n_groups < rd.A, far = rd.far_field != 0;
-    auto *const kernel = bundle ? (far ? visibility_kernel<true, true> : visibility_kernel<true, false>)
-                                : (far ? visibility_kernel<false, true> : visibility_kernel<false, false>);
-    kernel<<<grid, kVisThreads, 0, s>>>(tri64, trel, c64, fac, fac_lo, ref64, nodes, order, F, rd, ag,
-                                        sc, pairs, state, n_graze, status);
+    const VisArgs v{tri64, trel, c64, fac, fac_lo, ref64, nodes, order, F,
+                    rd, ag, sc, pairs, state, n_graze, status};
+    if (rd.far_field) visibility_far_kernel<<<grid, kVisThreads, 0, s>>>(v);
+    else if (ag.n_groups < rd.A) visibility_kernel<<<grid, kVisThreads, 0, s>>>(v);
+    else visibility_single_kernel<<<grid, kVisThreads, 0, s>>>(v);
 }
 
 // -------------------------------------------------------------------------
