@@ -49,7 +49,9 @@ extern "C" {
 #define BART_PATH_SPECTRAL 2 /* the mixed path's records, each chirp row summed by the
                                 inverse-FFT route (Sec. 3.2): facet lines spread onto a
                                 uniform beat-frequency grid of 2M cells, one inverse FFT
-                                per row (a type-1 non-uniform FFT); needs M = 2^a 3^b */
+                                per row (a type-1 non-uniform FFT); needs M = 2^a 3^b; frames
+                                that the band-limited evaluation (csrc/band.cuh)
+                                takes are summed by it on both paths */
 
 /* complex sample types of an ADC cube (interleaved re, im) */
 #define BART_C128 0          /* complex double */
@@ -399,7 +401,7 @@ typedef struct bart_tune {
 
 /* Time the mixed-path synthesis of the current scene at t0 for each
  * candidate layout (samples per lane 16 and, where M allows, 32 and 8; tiles per
- * item 8 ... 512), each run once to warm up and then `reps` times (best
+ * item 8 ... 512, and for 16 also 0, the default), each run once to warm up and then `reps` times (best
  * time kept, CUDA events around the synthesis launches), and keep the
  * fastest layout for later frames (as bart_set_synth_layout).  adc: device
  * output of the shape bart_simulate_frame writes (overwritten).  Blocks

@@ -669,9 +669,9 @@ constexpr int kPathAdjointMixed = 101;
 //    160 0.87 / 1.24), or
 //  - the per-instance coarse cubes could exceed 16 GB.
 // A short frame gains too (one sedan, 1 chirp: 0.21 / 0.15 ms).
-static bool use_band(const bart_ctx *ctx, const RadarDev &rd, int64_t F, int I)
+static bool use_band(const bart_ctx *ctx, const RadarDev &rd, int32_t path, int64_t F, int I)
 {
-    return ctx->layout_S == 0 && !rd.far_field && !rd.delay_ref && rd.N <= 1024 &&
+    return (ctx->layout_S == 0 || path == BART_PATH_SPECTRAL) && !rd.far_field && !rd.delay_ref && rd.N <= 1024 &&
            F >= 8 * (int64_t)I * std::min(I, 32) && (int64_t)I * rd.O <= 65535 &&
            (int64_t)I * rd.O * rd.N * rd.M <= ((int64_t)1 << 31);
 }
@@ -830,12 +830,12 @@ static int run_frame(bart_ctx *ctx, double t0, int32_t path, void *adc, int32_t 
                         ? ctx->tpi_override
                         : synth_tiles_per_item(*std::max_element(scene_F.begin(), scene_F.end()));
     int64_t max_items = 0;
-    const bool band = path == BART_PATH_MIXED && use_band(ctx, rd, F, I);
+    const bool band = (path == BART_PATH_MIXED || path == BART_PATH_SPECTRAL) && use_band(ctx, rd, path, F, I);
     BandArgs bt{};
     const bool mixed_rows = path == BART_PATH_MIXED || path == BART_PATH_SPECTRAL ||
                             path == kPathAdjointMixed;
     const bool kin_rows = mixed_rows && (!band || stats);
-    if (path == BART_PATH_SPECTRAL && ctx->spec_M != rd.M) {
+    if (path == BART_PATH_SPECTRAL && !band && ctx->spec_M != rd.M) {
         std::vector<float> tab(2 * (size_t)rd.M);
         spectral_tables(rd.M, tab.data());
         BART_TRY(ctx->spec_tab.ensure(tab.size(), "spectral kernel tables"));
@@ -1100,7 +1100,7 @@ static int run_frame(bart_ctx *ctx, double t0, int32_t path, void *adc, int32_t 
         if (tm) CUDA_TRY(cudaEventRecord(ctx->ev[3], s), "cudaEventRecord");
         // 4. synthesis
         nv.next("bart synthesis");
-        if (path == BART_PATH_MIXED) {
+        if (path == BART_PATH_MIXED || (path == BART_PATH_SPECTRAL && band)) {
             a.partial = ctx->partial.p;
             a.item_off = ctx->item_off.p;
             a.item_counter = ctx->item_counter.p;
@@ -1371,12 +1371,13 @@ int bart_autotune(bart_ctx *ctx, double t0, void *adc, int32_t dtype, int32_t re
     std::vector<int> Ss = {0};
     if (synth_layout_samples(ctx->radar.M, 32) == 32) Ss.push_back(32);
     if (synth_layout_samples(ctx->radar.M, 8) == 8) Ss.push_back(8);
-    const int tpis[] = {8, 16, 32, 64, 128, 256, 512};
+    const int tpis[] = {0, 8, 16, 32, 64, 128, 256, 512};    // 0: the default, for 16 samples
     int rc = BART_OK;
     float best = 0.f;
     for (int S : Ss) {
         for (int tpi : tpis) {
             if (out->n_trials >= BART_TUNE_MAX) break;
+            if (tpi == 0 && S != 0) continue;
             ctx->layout_S = S;
             ctx->tpi_override = tpi;
             float ms_best = 0.f;

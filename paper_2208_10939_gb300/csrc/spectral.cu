@@ -25,6 +25,11 @@
 // spreading each warp evaluates queued records with its lanes over the
 // samples.  Work per record ~ W grid cells instead of M samples.
 //
+// This kernel takes the frames that the band-limited evaluation (band.cuh)
+// does not -- other delay forms, very long frames, many tiny instances -- since
+// the same transform's gain comes cheaper there: an intersection frame of 16
+// channels (64 x 512, 300k facets) took 19.7 ms here and takes 1.4 ms there.
+//
 // One CTA per chirp row.  The row's record list is cut into 64 blocks that
 // the warps take from a shared counter; a warp's lanes take consecutive runs
 // of a block (neighbouring facets sit at neighbouring beat frequencies, so
