@@ -2,20 +2,24 @@
 //
 //  1. RDM with the complex cube kept: Y[o][r][d'] (rdm.cu).
 //  2. cfar_kernel: cell-averaging CFAR.  A block owns TR whole range rows
-//     (TR * N <= 1024 cells, TR | M), so the cyclic Doppler neighbourhood of every
-//     cell is inside the block.  Vertical partial sums first, per column:
+//     (TR | M, TR * N <= 256 cells or one row), so the cyclic Doppler
+//     neighbourhood of every cell is inside the block.  Vertical partial sums first, per column:
 //       vout[r][c] = sum_{gr < |u| <= hr} P[r+u][c]   (rows outside the guard)
 //       vmid[r][c] = sum_{|u| <= gr}       P[r+u][c]   (rows of the guard)
 //     then per cell the training sum
 //       T = sum_{|k| <= hd} vout[r][c+k] + sum_{gd < |k| <= hd} vmid[r][c+k],
 //     every term a training cell, no cancellation.  FP64 sums of the FP32
 //     RDM; detection when (double)P > alpha * (T / n_train).
+//     The FP64 sums bound it (52 conversions and additions a cell at a 64th of
+//     the FP32 rate), so the blocks are small enough to be on every
+//     multiprocessor: 128 of 256 cells on a 256 x 128 map, 11 us, against 27
+//     with 32 of 1024 cells.
 //  3. emit_kernel: ordered compaction of the flags into row-major cell
-//     indices (per-block counts, block-local scan).
-//  4. steer_kernel: steering table E[o][i] = exp(+j 2 pi a_o s_i) with
-//     a_o = x_o / lambda_c, s_i = -1 + 2 i / bins; the phase 2 a_o s_i is
-//     formed and reduced mod 2 in FP64, the sine/cosine taken in the FFT's
-//     precision.
+//     indices (per-block counts summed by the whole block, block-local scan).
+//  4. steering table E[o][i] = exp(+j 2 pi a_o s_i) with a_o = x_o / lambda_c,
+//     s_i = -1 + 2 i / bins, by blocks of the CFAR's launch after the map's (it
+//     needs nothing of the map); the phase 2 a_o s_i is formed and reduced mod
+//     2 in FP64, the sine/cosine taken in the FFT's precision.
 //  5. angle_kernel: per detection, S_i = |sum_o E[o][i] Y_o|^2 over the
 //     grid, first maximum -> azimuth; range and rate from the bins.
 #include <cuda_runtime.h>
@@ -35,23 +39,54 @@ __device__ __forceinline__ void sincospi_p(float x, float *s, float *c) { sincos
 __device__ __forceinline__ void sincospi_p(double x, double *s, double *c) { sincospi(x, s, c); }
 
 constexpr int kCfarThreads = 256;
-constexpr int kCfarCells = 1024;      // cells per CFAR block (TR * N)
+constexpr int kCfarCells = 1024;      // the longest row (N)
 constexpr int kAngleThreads = 256;
 constexpr int kAngleBlocks = 4 * 152;
+constexpr int kSteerBlocks = 4 * 152;
 
 // whole range rows per CFAR block: the largest power of two TR with
-// TR N <= kCfarCells that divides M
+// TR N <= kCfarThreads that divides M, at least one
 int rows_per_block(int M, int N)
 {
     int tr = 1;
-    while (2 * tr * N <= kCfarCells && M % (2 * tr) == 0) tr *= 2;
+    while (2 * tr * N <= kCfarThreads && M % (2 * tr) == 0) tr *= 2;
     return tr;
 }
 
-__global__ void __launch_bounds__(kCfarThreads)
-cfar_kernel(const float *__restrict__ P, int M, int N, int TR, DetectDev dd,
-            uint8_t *__restrict__ flag, int32_t *__restrict__ blk_cnt)
+// steering table entries block, block + blocks, ... of kCfarThreads each
+template <typename T>
+__device__ __forceinline__ void steer(const RadarDev &rd, double lam_c, int bins, int block,
+                                      int blocks, typename Cx<T>::type *__restrict__ E)
 {
+    const int64_t n = (int64_t)rd.O * bins;
+    for (int64_t i = (int64_t)block * kCfarThreads + threadIdx.x; i < n;
+         i += (int64_t)blocks * kCfarThreads) {
+        const int o = (int)(i / bins), b = (int)(i % bins);
+        const int p = o / rd.Q, q = o % rd.Q;
+        const double a = (rd.ant[p][0] + rd.ant[rd.P + q][0]) / lam_c;
+        const double sv = -1.0 + 2.0 * (double)b / (double)bins;
+        double t = 2.0 * a * sv;            // phase / pi
+        t -= 2.0 * rint(0.5 * t);           // into [-1, 1]
+        T s, c;
+        sincospi_p((T)t, &s, &c);
+        typename Cx<T>::type e;
+        e.x = c;
+        e.y = s;
+        E[i] = e;
+    }
+}
+
+// blocks 0 .. nblk - 1: the map; the others: the steering table
+template <typename T>
+__global__ void __launch_bounds__(kCfarThreads)
+cfar_kernel(const float *__restrict__ P, int M, int N, int TR, int nblk, DetectDev dd,
+            uint8_t *__restrict__ flag, int32_t *__restrict__ blk_cnt, RadarDev rd,
+            typename Cx<T>::type *__restrict__ E)
+{
+    if (blockIdx.x >= nblk) {
+        steer<T>(rd, dd.lam_c, dd.bins, blockIdx.x - nblk, gridDim.x - nblk, E);
+        return;
+    }
     __shared__ double vout[kCfarCells];
     __shared__ double vmid[kCfarCells];
     const int r0 = blockIdx.x * TR;
@@ -133,14 +168,13 @@ __global__ void __launch_bounds__(kCfarThreads)
 emit_kernel(const uint8_t *__restrict__ flag, const int32_t *__restrict__ blk_cnt, int nblk,
             int cells, int32_t *__restrict__ list, int32_t *__restrict__ count)
 {
-    __shared__ int off_s;
-    if (threadIdx.x == 0) {
-        int off = 0;
-        for (int b = 0; b < blockIdx.x; ++b) off += blk_cnt[b];
-        off_s = off;
-        if (blockIdx.x == nblk - 1) *count = off + blk_cnt[blockIdx.x];
-    }
-    __syncthreads();
+    const bool last = blockIdx.x == nblk - 1;
+    if (blk_cnt[blockIdx.x] == 0 && !last) return;
+    // detections of the earlier blocks
+    int before = 0, off = 0;
+    for (int b = threadIdx.x; b < blockIdx.x; b += blockDim.x) before += blk_cnt[b];
+    block_exclusive_scan(before, &off);
+    if (last && threadIdx.x == 0) *count = off + blk_cnt[blockIdx.x];
     if (blk_cnt[blockIdx.x] == 0) return;
     const int per = (cells + blockDim.x - 1) / blockDim.x;   // consecutive cells per thread
     const int64_t base = (int64_t)blockIdx.x * cells;
@@ -149,34 +183,12 @@ emit_kernel(const uint8_t *__restrict__ flag, const int32_t *__restrict__ blk_cn
     for (int k = 0; k < per; ++k)
         if (c0 + k < cells) mine += flag[base + c0 + k];
     int total = 0;
-    int at = off_s + block_exclusive_scan(mine, &total);
+    int at = off + block_exclusive_scan(mine, &total);
     for (int k = 0; k < per && mine; ++k)
         if (c0 + k < cells && flag[base + c0 + k]) {
             list[at++] = (int32_t)(base + c0 + k);
             --mine;
         }
-}
-
-template <typename T>
-__global__ void steer_kernel(RadarDev rd, double lam_c, int bins,
-                             typename Cx<T>::type *__restrict__ E)
-{
-    const int64_t n = (int64_t)rd.O * bins;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const int o = (int)(i / bins), b = (int)(i % bins);
-        const int p = o / rd.Q, q = o % rd.Q;
-        const double a = (rd.ant[p][0] + rd.ant[rd.P + q][0]) / lam_c;
-        const double sv = -1.0 + 2.0 * (double)b / (double)bins;
-        double t = 2.0 * a * sv;            // phase / pi
-        t -= 2.0 * rint(0.5 * t);           // into [-1, 1]
-        T s, c;
-        sincospi_p((T)t, &s, &c);
-        typename Cx<T>::type e;
-        e.x = c;
-        e.y = s;
-        E[i] = e;
-    }
 }
 
 template <typename T>
@@ -281,32 +293,33 @@ void detect_carve(void *ws, const RadarDev &rd, int dtype, int bins, DetectBufs 
 }
 
 template <typename T>
-static void run_angle(const RadarDev &rd, const DetectDev &dd, const DetectBufs &b,
-                      const float *rdm, bart_point *points, int max_points, cudaStream_t s)
+static void run_points(const RadarDev &rd, const DetectDev &dd, const DetectBufs &b,
+                       bart_point *points, int max_points, cudaStream_t s)
 {
     using C = typename Cx<T>::type;
-    const int64_t ne = (int64_t)rd.O * dd.bins;
-    const int sb = (int)((ne + 255) / 256 < 4 * 152 ? (ne + 255) / 256 : 4 * 152);
-    steer_kernel<T><<<sb, 256, 0, s>>>(rd, dd.lam_c, dd.bins, reinterpret_cast<C *>(b.steer));
+    const int TR = rows_per_block(rd.M, rd.N);
+    const int nblk = rd.M / TR;
+    const int64_t ne = ((int64_t)rd.O * dd.bins + kCfarThreads - 1) / kCfarThreads;
+    const int sb = (int)(ne < kSteerBlocks ? ne : kSteerBlocks);
+    C *E = reinterpret_cast<C *>(b.steer);
+    cfar_kernel<T><<<nblk + sb, kCfarThreads, 0, s>>>(b.rdm, rd.M, rd.N, TR, nblk, dd, b.flag,
+                                                      b.blk_cnt, rd, E);
+    emit_kernel<<<nblk, kCfarThreads, 0, s>>>(b.flag, b.blk_cnt, nblk, TR * rd.N, b.list,
+                                             b.count);
     if (max_points <= 0) return;
     const size_t smem = (size_t)rd.O * sizeof(C);
     angle_kernel<T><<<kAngleBlocks, kAngleThreads, smem, s>>>(
-        reinterpret_cast<const C *>(b.cube), reinterpret_cast<const C *>(b.steer), rdm, b.list,
-        b.count, max_points, rd.O, rd.M, rd.N, dd, points);
+        reinterpret_cast<const C *>(b.cube), E, b.rdm, b.list, b.count, max_points, rd.O, rd.M,
+        rd.N, dd, points);
 }
 
 int launch_detect(const void *adc, int dtype, const RadarDev &rd, const DetectDev &dd,
                   const DetectBufs &b, bart_point *points, int max_points, cudaStream_t s)
 {
     launch_rdm_cube(adc, dtype, rd, b.X, b.cube, b.rdm, s);
-    const int TR = rows_per_block(rd.M, rd.N);
-    const int nblk = rd.M / TR;
-    cfar_kernel<<<nblk, kCfarThreads, 0, s>>>(b.rdm, rd.M, rd.N, TR, dd, b.flag, b.blk_cnt);
-    emit_kernel<<<nblk, kCfarThreads, 0, s>>>(b.flag, b.blk_cnt, nblk, TR * rd.N, b.list,
-                                             b.count);
-    if (dtype == BART_C64) run_angle<float>(rd, dd, b, b.rdm, points, max_points, s);
-    else run_angle<double>(rd, dd, b, b.rdm, points, max_points, s);
-    return 3 + 3 + (max_points > 0 ? 1 : 0);
+    if (dtype == BART_C64) run_points<float>(rd, dd, b, points, max_points, s);
+    else run_points<double>(rd, dd, b, points, max_points, s);
+    return 3 + 2 + (max_points > 0 ? 1 : 0);
 }
 
 }  // namespace bart
