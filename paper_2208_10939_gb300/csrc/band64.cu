@@ -1,0 +1,716 @@
+// Band-limited FP64 echo synthesis (see band64.cuh): tables, plan, reference
+// phases, work items, node sums, interpolation.
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+#include <algorithm>
+
+#include "band64.cuh"
+#include "band_plan.cuh"
+#include "record_fp64.cuh"
+
+namespace bart {
+
+// -------------------------------------------------------------------------
+// layouts (host)
+// -------------------------------------------------------------------------
+void band64_shape(int N, int M, Band64Shape &sh)
+{
+    // nodes and the phase they carry: 4 sum_{k >= K-1} |J_k(a)| = 1e-13
+    static const struct { int K; float a; } chirps[] = {
+        {8, 0.077f}, {10, 0.255f}, {12, 0.569f}, {14, 1.01f}, {16, 1.59f}, {20, 3.05f},
+        {24, 4.86f}, {28, 6.92f}, {32, 9.19f}, {40, 14.1f}, {48, 19.6f}, {64, 31.3f},
+        {80, 43.8f}, {128, 83.7f}};
+    static const struct { int K; float a; } samples[] = {
+        {32, 9.19f}, {64, 31.3f}, {96, 56.8f}, {128, 83.7f}, {160, 111.f}, {192, 139.f},
+        {224, 168.f}, {256, 197.f}, {320, 256.f}, {384, 316.f}, {448, 376.f}, {512, 437.f},
+        {640, 558.f}, {768, 681.f}};
+    sh = Band64Shape{};
+    sh.N = N;
+    sh.M = M;
+    int x = 0;
+    int64_t w = 0;
+    auto chirp = [&](int K, float a, bool table) {
+        const int l = sh.n_n++;
+        sh.kn[l] = K;
+        sh.an[l] = a;
+        sh.xn[l] = x;
+        sh.wn[l] = w;
+        x += K;
+        if (table) w += (int64_t)K * N;
+    };
+    chirp(N, 1e30f, false);
+    chirp(1, 0.f, false);
+    for (auto &c : chirps)
+        if (5 * c.K <= 4 * N && sh.n_n < kB64N) chirp(c.K, c.a, true);
+    x = 0;
+    w = 0;
+    auto sample = [&](int K, float a, bool table) {
+        const int l = sh.n_m++;
+        sh.km[l] = K;
+        sh.am[l] = a;
+        sh.xm[l] = x;
+        sh.wm[l] = w;
+        x += K;
+        if (table) w += (int64_t)K * M;
+    };
+    sample(M, 1e30f, false);
+    for (auto &c : samples)
+        if (5 * c.K <= 4 * M && sh.n_m < kB64M) sample(c.K, c.a, true);
+}
+
+Band64Sizes band64_sizes(const Band64Shape &sh)
+{
+    Band64Sizes z{};
+    for (int l = 0; l < sh.n_n; ++l) {
+        z.xn += sh.kn[l];
+        if (l > 1) z.wn += (int64_t)sh.kn[l] * sh.N;
+    }
+    for (int l = 0; l < sh.n_m; ++l) {
+        z.xm += sh.km[l];
+        if (l > 0) z.wm += (int64_t)sh.km[l] * sh.M;
+    }
+    return z;
+}
+
+void band64_tables(double *tab, Band64Args &b)
+{
+    const Band64Sizes z = band64_sizes(b.sh);
+    b.turn = reinterpret_cast<double2 *>(tab);
+    b.xn = tab + 512;
+    b.xm = b.xn + z.xn;
+    b.wn = b.xm + z.xm;
+    b.wm = b.wn + z.wn;
+}
+
+namespace {
+
+// -------------------------------------------------------------------------
+// tables: the Chebyshev nodes of [0, len - 1] and their barycentric weights at
+// the whole positions (a warp a position); block (0, 0) also the sines
+// -------------------------------------------------------------------------
+__device__ __forceinline__ double cheb_node(int j, int K, int len)
+{
+    return 0.5 * (len - 1) * (1.0 - cospi((j + 0.5) / K));
+}
+
+__global__ void __launch_bounds__(256) band64_table_kernel(Band64Shape sh, double *__restrict__ xn,
+                                                           double *__restrict__ xm,
+                                                           double *__restrict__ wn,
+                                                           double *__restrict__ wm,
+                                                           double2 *__restrict__ turn)
+{
+    const bool chirps = (int)blockIdx.x < sh.n_n;
+    const int l = chirps ? blockIdx.x : blockIdx.x - sh.n_n;
+    const int K = chirps ? sh.kn[l] : sh.km[l], len = chirps ? sh.N : sh.M;
+    const bool whole = l == 0 || (chirps && l == 1);
+    double *x = chirps ? xn + sh.xn[l] : xm + sh.xm[l];
+    if (blockIdx.x == 0 && blockIdx.y == 0) {
+        double s, c;
+        sincospi(threadIdx.x / 128.0, &s, &c);
+        turn[threadIdx.x] = make_double2(c, s);
+    }
+    if (blockIdx.y == 0)
+        for (int j = threadIdx.x; j < K; j += blockDim.x) x[j] = whole ? j : cheb_node(j, K, len);
+    if (whole) return;
+    const int lane = threadIdx.x & 31;
+    for (int n = blockIdx.y * 8 + (threadIdx.x >> 5); n < len; n += gridDim.y * 8) {
+        double sum = 0.0;
+        int hit = -1;
+        for (int j = lane; j < K; j += 32) {
+            const double d = n - cheb_node(j, K, len);
+            if (d == 0.0) hit = j;
+            else sum += (j & 1 ? -1.0 : 1.0) * sinpi((j + 0.5) / K) / d;
+        }
+        for (int off = 16; off > 0; off >>= 1) {
+            sum += __shfl_xor_sync(0xffffffffu, sum, off);
+            hit = max(hit, __shfl_xor_sync(0xffffffffu, hit, off));
+        }
+        for (int j = lane; j < K; j += 32) {
+            const double d = n - cheb_node(j, K, len);
+            const double v = hit >= 0 ? (j == hit ? 1.0 : 0.0)
+                                      : (j & 1 ? -1.0 : 1.0) * sinpi((j + 0.5) / K) / (d * sum);
+            if (chirps) wn[sh.wn[l] + (int64_t)n * K + j] = v;
+            else wm[sh.wm[l] + (int64_t)j * len + n] = v;
+        }
+    }
+}
+
+// -------------------------------------------------------------------------
+// plan and reference phases
+// -------------------------------------------------------------------------
+__global__ void band64_plan_kernel(Band64Args b, RadarDev rd, MixConsts K,
+                                   const float *__restrict__ vel32, const FacetRec *__restrict__ fac)
+{
+    const int i = blockIdx.x;
+    const BandBounds q = band_bounds(b.box, i, rd, K, vel32);
+    if (threadIdx.x != 0) return;
+    Band64Plan pl;
+    for (int r = 0; r < 3; ++r) pl.c[r] = q.c[r];
+    pl.in = pl.im = 0;
+    pl.rotate = q.ok;
+    const float span = 3.1415927f * q.beta * (float)(b.sh.M - 1);
+    if (q.ok)
+        for (int l = 1; l < b.sh.n_m && pl.im == 0; ++l)
+            if (span <= b.sh.am[l]) pl.im = l;
+    // a facet lit from both sides has a kink where its obliquity changes sign:
+    // every chirp is kept
+    const bool smooth = b.ioff[i] < b.ioff[i + 1] && !fac[b.ioff[i]].two_sided;
+    if (q.speed == 0.f) {
+        pl.in = 1;
+    } else if (q.ok && smooth) {
+        for (int l = 2; l < b.sh.n_n && pl.in == 0; ++l)
+            if (q.turn <= b.sh.an[l]) pl.in = l;
+    }
+    b.plan[i] = pl;
+}
+
+__device__ __forceinline__ double two_sum(double a, double b, double &e)
+{
+    const double s = a + b, t = s - a;
+    e = (a - (s - t)) + (b - t);
+    return s;
+}
+
+// The reference phase of (instance, channel) in a chirp that starts at tn, as
+// a quadratic in the time from the middle of its samples, cycles: the box
+// centre's path, its constant in double-double (its rounding is the whole
+// instance's), reduced mod 1.
+__device__ __forceinline__ double4 band64_ref(const RadarDev &rd, const float *c,
+                                              const double *__restrict__ v, int p, int q, double tn)
+{
+    const double tc = 0.5 * (rd.M - 1) / rd.fs, t = rd.intra ? tn + tc : tn;
+    const double v2 = v[0] * v[0] + v[1] * v[1] + v[2] * v[2];
+    double Lh = 0.0, Ll = 0.0, L1 = 0.0, L2 = 0.0;
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+        const double *pa = rd.ant[e == 0 ? p : rd.P + q];
+        double qh = 0.0, ql = 0.0, sv = 0.0, er;
+        for (int r = 0; r < 3; ++r) {
+            double sl;
+            const double s = two_sum(pa[r] - (double)c[r], -v[r] * t, sl);
+            const double pr = s * s;
+            ql += fma(s, s, -pr) + 2.0 * s * sl;
+            qh = two_sum(qh, pr, er);
+            ql += er;
+            sv += s * v[r];
+        }
+        const double R = sqrt(qh);
+        const double lo = 0.5 * (fma(-R, R, qh) + ql) / R;
+        const double rr = -sv / R;
+        Lh = two_sum(Lh, R, er);
+        Ll += er + lo;
+        L1 += rr;
+        L2 += 0.5 * (v2 - rr * rr) / R;
+    }
+    if (!rd.intra) L1 = L2 = 0.0;
+    const double F = (rd.f0 + rd.slope * tc) / kC0, mc = rd.slope / kC0;
+    const double m2 = rd.slope / (2.0 * kC0 * kC0);
+    const double ph = F * Lh, phe = fma(F, Lh, -ph);
+    const double p0 = (ph - rint(ph)) + (phe + F * Ll) - m2 * Lh * Lh;
+    return make_double4(p0 - rint(p0), F * L1 + mc * Lh - 2.0 * m2 * Lh * L1,
+                        F * L2 + mc * L1 - m2 * (L1 * L1 + 2.0 * Lh * L2), 0.0);
+}
+
+__device__ __forceinline__ double chirp_start(const RadarDev &rd, double n, int tx)
+{
+    return (n * rd.slots + (rd.tdm ? tx : 0)) * rd.Tc;
+}
+
+__global__ void __launch_bounds__(128)
+band64_ref_kernel(Band64Args b, RadarDev rd, const double *__restrict__ vel64)
+{
+    const int v = blockIdx.y, i = v / b.O, o = v % b.O;
+    const Band64Plan pl = b.plan[i];
+    const int N = b.sh.N, nj = b.sh.kn[pl.in];
+    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    const bool node = e >= N;                     // chirps first, then nodes
+    const int k = node ? e - N : e;
+    if (k >= (node ? nj : N)) return;
+    double4 r = make_double4(0.0, 0.0, 0.0, 0.0);
+    if (pl.rotate) {
+        const int p = o / rd.Q, q = o % rd.Q;
+        const double n = node ? b.xn[b.sh.xn[pl.in] + k] : (double)k;
+        r = band64_ref(rd, pl.c, vel64 + 3 * i, p, q, chirp_start(rd, n, p));
+    }
+    (node ? b.refn : b.ref)[(int64_t)v * N + k] = r;
+}
+
+// -------------------------------------------------------------------------
+// list parts and work items
+// -------------------------------------------------------------------------
+__global__ void band64_lists_kernel(Band64Args b, const int32_t *__restrict__ vis_idx,
+                                    const int32_t *__restrict__ vis_cnt, int64_t F)
+{
+    const int lane = threadIdx.x & 31;
+    const int v = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    if (v >= b.I * b.O) return;
+    const int i = v / b.O, o = v % b.O;
+    const int32_t *list = vis_idx + (int64_t)o * F;
+    const int lo = warp_lower_bound(list, vis_cnt[o], b.ioff[i], lane);
+    const int n = warp_lower_bound(list + lo, vis_cnt[o] - lo, b.ioff[i + 1], lane);
+    if (lane == 0) {
+        b.vstart[v] = lo;
+        b.vcnt[v] = n;
+    }
+}
+
+constexpr int kSeg = 64;             // nodes of a work item
+
+// parts of an (instance, channel)'s facets, by its own list and layout alone:
+// the sums do not depend on what else is in the call
+__device__ __forceinline__ int band64_chunks(const Band64Shape &sh, const Band64Plan &pl, int cnt)
+{
+    const int64_t room = (int64_t)kB64Room * sh.N * sh.M / ((int64_t)sh.kn[pl.in] * sh.km[pl.im]);
+    return (int)max((int64_t)1, min(room, (int64_t)min(kB64Chunks, (cnt + 127) / 128)));
+}
+
+__device__ __forceinline__ int band64_item_count(const Band64Shape &sh, const Band64Plan &pl, int cnt)
+{
+    return cnt == 0 ? 0 : sh.kn[pl.in] * ((sh.km[pl.im] + kSeg - 1) / kSeg) *
+                              band64_chunks(sh, pl, cnt);
+}
+
+// item prefix (one block)
+__global__ void __launch_bounds__(1024) band64_items_kernel(Band64Args b)
+{
+    __shared__ int s_w[32], s_run;
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int V = b.I * b.O;
+    if (t == 0) {
+        s_run = 0;
+        *b.ticket = 0;
+    }
+    __syncthreads();
+    for (int v0 = 0; v0 < V; v0 += 1024) {
+        const int v = v0 + t;
+        const int items = v < V ? band64_item_count(b.sh, b.plan[v / b.O], b.vcnt[v]) : 0;
+        int x = items;
+        for (int off = 1; off < 32; off <<= 1) {
+            const int u = __shfl_up_sync(0xffffffffu, x, off);
+            if (lane >= off) x += u;
+        }
+        if (lane == 31) s_w[warp] = x;
+        __syncthreads();
+        int before = s_run, all = 0;
+        for (int k = 0; k < 32; ++k) {
+            if (k < warp) before += s_w[k];
+            all += s_w[k];
+        }
+        if (v < V) b.item0[v] = before + x - items;
+        __syncthreads();
+        if (t == 0) s_run += all;
+        __syncthreads();
+    }
+    if (t == 0) b.item0[V] = s_run;
+}
+
+// -------------------------------------------------------------------------
+// phasors and records
+// -------------------------------------------------------------------------
+
+// exp(j 2 pi x): the nearest 256th of a turn from the table, the rest (at most
+// 0.0123 rad) by the sine's and cosine's own series (next terms 8e-18, 1e-20).
+// 14 FP64 operations.
+__device__ __forceinline__ void turn_exp(double x, const double2 *turn, double &c, double &s)
+{
+    const double big = 6755399441055744.0;            // 1.5 2^52: rounds to whole numbers
+    const double t = fma(x, 256.0, big);
+    const double2 w = turn[__double2loint(t) & 255];
+    const double r = fma(t - big, -1.0 / 256.0, x), r2 = r * r;
+    const double p = 2.0 * kPi, p2 = p * p;
+    const double es = r * fma(r2, fma(r2, p * p2 * p2 / 120.0, -p * p2 / 6.0), p);
+    const double ec = fma(r2, fma(r2, fma(r2, -p2 * p2 * p2 / 720.0, p2 * p2 / 24.0), -p2 / 2.0), 1.0);
+    c = fma(w.x, ec, -w.y * es);
+    s = fma(w.x, es, w.y * ec);
+}
+
+__device__ __forceinline__ double frac1(double x)      // x - rint(x)
+{
+    const double big = 6755399441055744.0;
+    return x - ((x + big) - big);
+}
+
+// path length over a chirp: sqrt(q(t)) of both legs as a quartic in the time
+// from the middle of the samples where |q(t) / q(tc) - 1| stays below 1e-3
+// (next term 7/256 1e-15), else evaluated as it stands
+struct Rec64 {
+    double L[5];                     // the quartic, or qt0 qt1 q2 qr0 qr1
+    double d[16];
+    int kind, flags;
+    int quartic, pad;
+};
+
+struct Node64 {                      // a node's constants
+    double t, tau, fmc, kp, rp;
+};
+
+__device__ __forceinline__ Node64 band64_node(const RadarDev &rd, double x, const double4 &ref)
+{
+    Node64 n;
+    n.t = x / rd.fs;
+    n.tau = (x - 0.5 * (rd.M - 1)) / rd.fs;
+    const double fm = rd.f0 + rd.slope * n.t;
+    n.fmc = fm / kC0;
+    n.kp = fm / rd.f0;
+    n.rp = frac1(fma(n.tau, fma(n.tau, ref.z, ref.y), ref.x));
+    return n;
+}
+
+__device__ __forceinline__ void band64_record(const SynthArgs &A, int64_t k, double tn,
+                                              const double *ptx, const double *prx, double k0,
+                                              double kmax, Rec64 &R)
+{
+    const int inst = A.fac[k].inst;
+    double tri[9], c0[3], rec[kRecEntries];
+    for (int i = 0; i < 9; ++i) tri[i] = A.tri64[9 * k + i];
+    for (int r = 0; r < 3; ++r) c0[r] = A.c64[3 * k + r];
+    int flags = 0;
+    R.kind = build_record<double>(tri, c0, A.vel64 + 3 * inst, tn, ptx, prx, (double)A.fac[k].rho,
+                                  A.rd.intra, k0, kmax, kDelayFacet, nullptr, A.fac[k].two_sided,
+                                  rec, &flags);
+    R.flags = flags;
+    for (int i = 0; i < 16; ++i) R.d[i] = rec[kRecD + i];
+    const double h = 0.5 * (A.rd.M - 1) / A.rd.fs, q2 = rec[2];
+    const double q1t = rec[1] + 2.0 * q2 * h, q1r = rec[4] + 2.0 * q2 * h;
+    const double Qt = rec[0] + h * (rec[1] + h * q2), Qr = rec[3] + h * (rec[4] + h * q2);
+    R.quartic = Qt > 0.0 && Qr > 0.0 && h * (fabs(q1t) + h * q2) < 1e-3 * Qt &&
+                h * (fabs(q1r) + h * q2) < 1e-3 * Qr;
+    if (!R.quartic) {
+        for (int i = 0; i < 5; ++i) R.L[i] = rec[i];
+        return;
+    }
+    // sqrt(Q + q1 tau + q2 tau^2) = sum l_k tau^k: 2 l0 l1 = q1, 2 l0 l2 + l1^2 = q2,
+    // l0 l3 + l1 l2 = 0, 2 l0 l4 + 2 l1 l3 + l2^2 = 0
+    const double st = sqrt(Qt), sr = sqrt(Qr), ht = 0.5 / st, hr = 0.5 / sr;
+    const double t1 = q1t * ht, r1 = q1r * hr;
+    const double t2 = (q2 - t1 * t1) * ht, r2 = (q2 - r1 * r1) * hr;
+    const double t3 = -2.0 * t1 * t2 * ht, r3 = -2.0 * r1 * r2 * hr;
+    R.L[0] = st + sr;
+    R.L[1] = t1 + r1;
+    R.L[2] = t2 + r2;
+    R.L[3] = t3 + r3;
+    R.L[4] = -(2.0 * t1 * t3 + t2 * t2) * ht - (2.0 * r1 * r3 + r2 * r2) * hr;
+}
+
+__device__ __forceinline__ double band64_path(const Rec64 &R, const Node64 &n)
+{
+    if (R.quartic)
+        return fma(n.tau, fma(n.tau, fma(n.tau, fma(n.tau, R.L[4], R.L[3]), R.L[2]), R.L[1]), R.L[0]);
+    return sqrt(R.L[0] + n.t * (R.L[1] + n.t * R.L[2])) + sqrt(R.L[3] + n.t * (R.L[4] + n.t * R.L[2]));
+}
+
+// the record's term at a node, its reference phase taken off, added to (re, im)
+__device__ __forceinline__ void band64_eval(const Rec64 &R, const Node64 &n, double mu_2c2,
+                                            const double2 *turn, double &re, double &im)
+{
+    const double L = band64_path(R, n);
+    const double th = frac1(L * fma(-mu_2c2, L, n.fmc)) - n.rp;
+    double c, s;
+    if (R.kind == kRecVertex) {
+#pragma unroll
+        for (int v = 0; v < 3; ++v) {
+            turn_exp(fma(-n.fmc, R.d[v], th), turn, c, s);
+            re = fma(R.d[3 + v], c, re);
+            im = fma(R.d[3 + v], s, im);
+        }
+    } else if (R.kind == kRecSeries) {
+        turn_exp(fma(-n.fmc, R.d[0], th), turn, c, s);
+        const double k2 = n.kp * n.kp;
+        double a = R.d[8], bb = R.d[15];
+#pragma unroll
+        for (int q = 6; q >= 0; --q) a = fma(a, k2, R.d[1 + q]);
+#pragma unroll
+        for (int q = 5; q >= 0; --q) bb = fma(bb, k2, R.d[9 + q]);
+        const double pr = a * k2, pi = bb * k2 * n.kp;
+        re += c * pr - s * pi;
+        im += c * pi + s * pr;
+    } else {
+        for (int e = 0; e < 3; ++e) {
+            turn_exp(fma(-n.fmc, R.d[3 * e], th), turn, c, s);
+            const double x = n.kp * R.d[3 * e + 1];
+            double sn;
+            if (R.flags & (1 << e)) {
+                const double x2 = x * x;
+                sn = 1.0 + x2 * (-1.0 / 6 + x2 * (1.0 / 120 + x2 * (-1.0 / 5040 +
+                     x2 * (1.0 / 362880 + x2 * (-1.0 / 39916800)))));
+            } else {
+                sn = sin(x) / x;
+            }
+            const double coef = n.kp * R.d[3 * e + 2] * sn;
+            re -= coef * s;
+            im += coef * c;
+        }
+    }
+}
+
+// -------------------------------------------------------------------------
+// node sums.  Work item = (instance, channel, chirp node, 64 sample nodes,
+// part of the facets), handed out by a ticket: the FP64 pipe is shared by all
+// blocks of a multiprocessor, so an equal count of items a multiprocessor is
+// an equal load.  A warp takes a quarter of the part: a lane builds a
+// facet's record, then the records go round with two nodes a lane; the four
+// warps' sums are added in order.
+// -------------------------------------------------------------------------
+constexpr int kB64Warps = 4;
+
+__device__ __forceinline__ int band64_find(const int32_t *__restrict__ item0, int V, int item)
+{
+    int lo = 0, hi = V - 1;                       // last v with item0[v] <= item
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (item0[mid] <= item) lo = mid;
+        else hi = mid - 1;
+    }
+    return lo;
+}
+
+__global__ void __launch_bounds__(kB64Warps * 32)
+synth_band64_kernel(SynthArgs A, Band64Args b)
+{
+    __shared__ Rec64 s_rec[kB64Warps][32];
+    __shared__ double2 s_turn[256];
+    __shared__ double2 s_sum[kB64Warps - 1][kSeg];
+    __shared__ int s_item;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    for (int i = threadIdx.x; i < 256; i += blockDim.x) s_turn[i] = b.turn[i];
+    const RadarDev &rd = A.rd;
+    const int V = b.I * b.O, total = b.item0[V];
+    const double c = kC0;
+    const double k0 = 2.0 * kPi * rd.f0 / c;
+    const double kmax = 2.0 * kPi * (rd.f0 + rd.slope * (rd.M - 1) / rd.fs) / c;
+    const double mu_2c2 = rd.slope / (2.0 * c * c);
+    for (;;) {
+        __syncthreads();
+        if (threadIdx.x == 0) s_item = atomicAdd(b.ticket, 1);
+        __syncthreads();
+        if (s_item >= total) return;
+        const int v = band64_find(b.item0, V, s_item);
+        const int i = v / b.O, o = v % b.O, cnt = b.vcnt[v];
+        const Band64Plan pl = b.plan[i];
+        const int nj = b.sh.kn[pl.in], Km = b.sh.km[pl.im], segs = (Km + kSeg - 1) / kSeg;
+        const int C = band64_chunks(b.sh, pl, cnt);
+        int at = s_item - b.item0[v];
+        const int chunk = at % C;
+        at /= C;
+        const int seg = at % segs, j = at / segs;
+        const int tx = o / rd.Q, rx = o % rd.Q;
+        const double tn = chirp_start(rd, b.xn[b.sh.xn[pl.in] + j], tx);
+        const double *ptx = rd.ant[tx], *prx = rd.ant[rd.P + rx];
+        const double4 ref = b.refn[(int64_t)v * b.sh.N + j];
+        const int s0 = seg * kSeg + lane;
+        const bool two = seg * kSeg + 32 < Km;    // Km is a multiple of 32
+        const double *xm = b.xm + b.sh.xm[pl.im];
+        const Node64 n0 = band64_node(rd, xm[s0], ref);
+        const Node64 n1 = band64_node(rd, xm[two ? s0 + 32 : s0], ref);
+        double re0 = 0.0, im0 = 0.0, re1 = 0.0, im1 = 0.0;
+        const int32_t *list = A.vis_idx + (int64_t)o * A.F + b.vstart[v];
+        const int part = chunk * kB64Warps + warp;
+        const int beg = (int)((int64_t)cnt * part / (C * kB64Warps));
+        const int end = (int)((int64_t)cnt * (part + 1) / (C * kB64Warps));
+        for (int base = beg; base < end; base += 32) {
+            const int m = min(32, end - base);
+            __syncwarp();
+            if (lane < m)
+                band64_record(A, list[base + lane], tn, ptx, prx, k0, kmax, s_rec[warp][lane]);
+            __syncwarp();
+            for (int k = 0; k < m; ++k) {
+                const Rec64 &R = s_rec[warp][k];
+                band64_eval(R, n0, mu_2c2, s_turn, re0, im0);
+                if (two) band64_eval(R, n1, mu_2c2, s_turn, re1, im1);
+            }
+        }
+        if (warp > 0) {
+            s_sum[warp - 1][lane] = make_double2(re0, im0);
+            s_sum[warp - 1][lane + 32] = make_double2(re1, im1);
+        }
+        __syncthreads();
+        if (warp == 0) {
+            for (int k = 0; k < kB64Warps - 1; ++k) {
+                re0 += s_sum[k][lane].x;
+                im0 += s_sum[k][lane].y;
+                re1 += s_sum[k][lane + 32].x;
+                im1 += s_sum[k][lane + 32].y;
+            }
+            double2 *out = b.coarse + (int64_t)v * kB64Room * b.sh.N * b.sh.M +
+                           ((int64_t)chunk * nj + j) * Km;
+            out[s0] = make_double2(re0, im0);
+            if (two) out[s0 + 32] = make_double2(re1, im1);
+        }
+    }
+}
+
+// the parts' sums into the first, in order
+__global__ void __launch_bounds__(256) band64_reduce_kernel(Band64Args b)
+{
+    const int v = blockIdx.x, cnt = b.vcnt[v];
+    if (cnt == 0) return;
+    const Band64Plan pl = b.plan[v / b.O];
+    const int C = band64_chunks(b.sh, pl, cnt);
+    if (C == 1) return;
+    const int n = b.sh.kn[pl.in] * b.sh.km[pl.im];
+    double2 *x = b.coarse + (int64_t)v * kB64Room * b.sh.N * b.sh.M;
+    for (int e = blockIdx.y * 256 + threadIdx.x; e < n; e += gridDim.y * 256) {
+        double2 a = x[e];
+        for (int k = 1; k < C; ++k) {
+            const double2 q = x[(int64_t)k * n + e];
+            a.x += q.x;
+            a.y += q.y;
+        }
+        x[e] = a;
+    }
+}
+
+// -------------------------------------------------------------------------
+// interpolation: a block makes 64 chirps x 16 samples of a channel, instance
+// by instance: first along the samples (its 16 samples of every chirp node, in
+// shared memory), then along the chirps, turned by the reference
+// -------------------------------------------------------------------------
+constexpr int kExpN = 64, kExpM = 16;
+
+__global__ void __launch_bounds__(256)
+band64_expand_kernel(Band64Args b, RadarDev rd, void *__restrict__ out, int out_c64)
+{
+    __shared__ double2 s_d[kB64MaxNodes][kExpM];
+    __shared__ double2 s_turn[256];
+    s_turn[threadIdx.x] = b.turn[threadIdx.x];
+    const int N = b.sh.N, M = b.sh.M;
+    const int mt = M / kExpM;                     // M is a multiple of 32
+    const int m0 = (int)(blockIdx.x % mt) * kExpM, n0 = (int)(blockIdx.x / mt) * kExpN;
+    const int o = blockIdx.y, scene = blockIdx.z;
+    const int mm = threadIdx.x & (kExpM - 1), nn = threadIdx.x / kExpM, m = m0 + mm;
+    const double tau = (m - 0.5 * (rd.M - 1)) / rd.fs;
+    double2 acc[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) acc[k] = make_double2(0.0, 0.0);
+    for (int i = b.scene_inst[scene]; i < b.scene_inst[scene + 1]; ++i) {
+        const int v = i * b.O + o;
+        if (b.vcnt[v] == 0) continue;
+        const Band64Plan pl = b.plan[i];
+        const int nj = b.sh.kn[pl.in], Km = b.sh.km[pl.im];
+        const double2 *x = b.coarse + (int64_t)v * kB64Room * N * M;
+        // rows: the chirp nodes, or (every chirp kept) the block's chirps
+        const int j0 = pl.in == 0 ? n0 : 0, rows = pl.in == 0 ? min(kExpN, N - n0) : nj;
+        __syncthreads();
+        for (int j = nn; j < rows; j += 256 / kExpM) {
+            const double2 *row = x + (int64_t)(j0 + j) * Km;
+            double2 d = make_double2(0.0, 0.0);
+            if (pl.im == 0) {
+                d = row[m];
+            } else {
+                const double *w = b.wm + b.sh.wm[pl.im] + m;
+#pragma unroll 8
+                for (int s = 0; s < Km; ++s) {
+                    const double ws = w[(int64_t)s * M];
+                    const double2 cs = row[s];
+                    d.x = fma(ws, cs.x, d.x);
+                    d.y = fma(ws, cs.y, d.y);
+                }
+            }
+            s_d[j][mm] = d;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int n = n0 + nn + k * (256 / kExpM);
+            if (n >= N) break;
+            double2 z = make_double2(0.0, 0.0);
+            if (pl.in == 0) {
+                z = s_d[n - n0][mm];
+            } else if (pl.in == 1) {
+                z = s_d[0][mm];
+            } else {
+                const double *w = b.wn + b.sh.wn[pl.in] + (int64_t)n * nj;
+                for (int j = 0; j < nj; ++j) {
+                    const double wj = w[j];
+                    const double2 d = s_d[j][mm];
+                    z.x = fma(wj, d.x, z.x);
+                    z.y = fma(wj, d.y, z.y);
+                }
+            }
+            if (pl.rotate) {
+                const double4 r = b.ref[(int64_t)v * N + n];
+                double c, s;
+                turn_exp(frac1(fma(tau, fma(tau, r.z, r.y), r.x)), s_turn, c, s);
+                z = make_double2(z.x * c - z.y * s, z.x * s + z.y * c);
+            }
+            acc[k].x += z.x;
+            acc[k].y += z.y;
+        }
+    }
+    const double fm = rd.f0 + rd.slope * (double)m / rd.fs;
+    const double km = 2.0 * kPi * fm / kC0;
+    const double sc = 2.0 * sqrt(kPi) / pow(4.0 * kPi, 1.5) / (km * km);
+    const int64_t row = ((int64_t)scene * b.O + o) * N;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const int n = n0 + nn + k * (256 / kExpM);
+        if (n >= N) break;
+        const int64_t e = (row + n) * M + m;
+        if (out_c64)
+            static_cast<float2 *>(out)[e] = make_float2((float)(acc[k].x * sc), (float)(acc[k].y * sc));
+        else
+            static_cast<double2 *>(out)[e] = make_double2(acc[k].x * sc, acc[k].y * sc);
+    }
+}
+
+// per-form counts of every (facet, channel, chirp) record (stats)
+__global__ void __launch_bounds__(128) count_records64_kernel(SynthArgs A)
+{
+    const int n = blockIdx.x, vrow = blockIdx.y, o = vrow % A.rd.O;
+    const int tx = o / A.rd.Q, rx = o % A.rd.Q;
+    const double c = kC0, k0 = 2.0 * kPi * A.rd.f0 / c;
+    const double kmax = 2.0 * kPi * (A.rd.f0 + A.rd.slope * (A.rd.M - 1) / A.rd.fs) / c;
+    const int32_t *list = A.vis_idx + (int64_t)o * A.F + (A.vstart ? A.vstart[vrow] : 0);
+    unsigned int cnt[3] = {0, 0, 0};
+    for (int e = threadIdx.x; e < A.vcnt[vrow]; e += 128) {
+        Rec64 R;
+        band64_record(A, list[e], chirp_start(A.rd, n, tx), A.rd.ant[tx], A.rd.ant[A.rd.P + rx], k0,
+                      kmax, R);
+        ++cnt[R.kind == kRecVertex ? 0 : R.kind == kRecSeries ? 1 : 2];
+    }
+    for (int k = 0; k < 3; ++k) {
+        const unsigned int s = __reduce_add_sync(0xffffffffu, cnt[k]);
+        if ((threadIdx.x & 31) == 0 && s) atomicAdd(A.counters + k, (unsigned long long)s);
+    }
+}
+
+}  // namespace
+
+void launch_band64_tables(const Band64Args &b, cudaStream_t s)
+{
+    band64_table_kernel<<<dim3((unsigned int)(b.sh.n_n + b.sh.n_m), 16), 256, 0, s>>>(
+        b.sh, const_cast<double *>(b.xn), const_cast<double *>(b.xm), const_cast<double *>(b.wn),
+        const_cast<double *>(b.wm), const_cast<double2 *>(b.turn));
+}
+
+void launch_band64_plan(const Band64Args &b, const SynthArgs &a, cudaStream_t s)
+{
+    const MixConsts K = mix_consts(a.rd);
+    band64_plan_kernel<<<b.I, 32, 0, s>>>(b, a.rd, K, a.vel32, a.fac);
+    const dim3 g((unsigned int)((2 * b.sh.N + 127) / 128), (unsigned int)(b.I * b.O));
+    band64_ref_kernel<<<g, 128, 0, s>>>(b, a.rd, a.vel64);
+}
+
+void launch_synth_band64(const Band64Args &b, const SynthArgs &a, cudaStream_t s)
+{
+    const int V = b.I * b.O;
+    band64_lists_kernel<<<(V + 3) / 4, 128, 0, s>>>(b, a.vis_idx, a.vis_cnt, a.F);
+    band64_items_kernel<<<1, 1024, 0, s>>>(b);
+    int dev = 0, sms = 0, per_sm = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, synth_band64_kernel, kB64Warps * 32, 0);
+    synth_band64_kernel<<<std::max(1, sms) * std::max(1, per_sm), kB64Warps * 32, 0, s>>>(a, b);
+    band64_reduce_kernel<<<dim3((unsigned int)V, 4), 256, 0, s>>>(b);
+    const int tiles = (b.sh.M / kExpM) * ((b.sh.N + kExpN - 1) / kExpN);
+    band64_expand_kernel<<<dim3((unsigned int)tiles, (unsigned int)b.O, (unsigned int)b.B), 256, 0,
+                           s>>>(b, a.rd, a.out, a.out_c64);
+}
+
+void launch_count_records64(const SynthArgs &a, cudaStream_t s)
+{
+    count_records64_kernel<<<dim3((unsigned int)a.rd.N, (unsigned int)a.VO), 128, 0, s>>>(a);
+}
+
+}  // namespace bart

@@ -17,6 +17,7 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include "band.cuh"
+#include "band64.cuh"
 #include "bart_internal.cuh"
 #include "bounce.cuh"
 #include "bartsim.h"
@@ -167,6 +168,11 @@ struct bart_ctx {
     DevBuf<int64_t> d_ioff;             // facet offsets of the instances [I + 1]
     DevBuf<int32_t> d_sinst;            // first instance of each scene [B + 1]
     DevBuf<float2> band_coarse;
+    // the FP64 path's band-limited evaluation
+    Band64Shape band64_sh = {};
+    DevBuf<double> band64_tab;
+    DevBuf<unsigned char> band64_ws;
+    DevBuf<double2> band64_coarse;
     DevBuf<unsigned long long> counters;   // 0 vertex, 1 series, 2 edge, 3 grazing
     DevBuf<int> status;
     DevBuf<unsigned char> rdm_ws, adc_own;
@@ -273,7 +279,7 @@ struct bart_ctx {
         vals_tmp.release(); nodes.release(); levels.release(); ticket.release();
         state.release(); blk_cnt.release(); vis_idx.release();
         box.release(); band_tab.release(); band_ws.release(); d_ioff.release(); d_sinst.release();
-        band_coarse.release();
+        band_coarse.release(); band64_tab.release(); band64_ws.release(); band64_coarse.release();
         vis_cnt.release(); kin.release(); kquad.release(); partial.release(); item_off.release();
         item_counter.release(); counters.release(); status.release();
         rdm_ws.release(); adc_own.release(); rdm_own.release(); noise_scratch.release();
@@ -676,6 +682,19 @@ static bool use_band(const bart_ctx *ctx, const RadarDev &rd, int32_t path, int6
            (int64_t)I * rd.O * rd.N * rd.M <= ((int64_t)1 << 31);
 }
 
+// The FP64 path's two evaluations: band-limited (band64.cuh) unless the delay
+// form is not the facet's own, the frame is longer than its tables go, or its
+// scratch (kB64Room cubes an instance) would exceed 16 GB.  However small the
+// instances, interpolating one costs about what the direct sum spends on one
+// lit facet (100 FP64 operations a sample), so their size is no condition, and
+// a scene gives the same bits alone and in a batch.  A 5k-facet car on 12
+// channels of 32 x 256: 33.1 ms by the direct sum, 2.7 ms band-limited.
+static bool use_band64(const RadarDev &rd, int I)
+{
+    return !rd.far_field && !rd.delay_ref && rd.N <= 1024 && (int64_t)I * rd.O <= 65535 &&
+           (int64_t)I * rd.O * rd.N * rd.M <= ((int64_t)1 << 28);
+}
+
 // work items to aim for: six per resident warp, so that the last wave is short
 static int synth_band_target()
 {
@@ -929,10 +948,60 @@ static int run_frame(bart_ctx *ctx, double t0, int32_t path, void *adc, int32_t 
             BART_TRY(ensure_events(ctx->ev_syn, 2));
         }
     }
-    // the FP64 path splits each row's facet list over several warps when the
+    // FP64: band-limited where that applies and its scratch is to be had
+    bool band64 = path == BART_PATH_FP64 && use_band64(rd, I);
+    Band64Args b64{};
+    if (band64) {
+        const int64_t V = (int64_t)I * O;
+        if (ctx->band64_coarse.ensure((size_t)(V * kB64Room * rd.N * rd.M),
+                                      "band coarse samples") != BART_OK) {
+            g_err.clear();
+            band64 = false;
+        } else {
+            if (ctx->band64_sh.N != rd.N || ctx->band64_sh.M != rd.M) {
+                band64_shape(rd.N, rd.M, b64.sh);
+                const Band64Sizes z = band64_sizes(b64.sh);
+                ctx->band64_sh = Band64Shape{};
+                BART_TRY(ctx->band64_tab.ensure((size_t)(512 + z.xn + z.xm + z.wn + z.wm),
+                                                "band tables"));
+                band64_tables(ctx->band64_tab.p, b64);
+                launch_band64_tables(b64, s);
+                CUDA_TRY(cudaGetLastError(), "band table launch");
+                ctx->band64_sh = b64.sh;
+            }
+            b64.sh = ctx->band64_sh;
+            band64_tables(ctx->band64_tab.p, b64);
+            b64.I = I;
+            b64.B = B;
+            b64.O = O;
+            b64.box = ctx->box.p;
+            b64.scene_inst = ctx->d_sinst.p;
+            b64.ioff = ctx->d_ioff.p;
+            b64.coarse = ctx->band64_coarse.p;
+            auto carve = [&](unsigned char *p) -> size_t {
+                size_t n = 0;
+                auto take = [&](auto *&field, int64_t count) {
+                    using T = std::remove_reference_t<decltype(*field)>;
+                    field = reinterpret_cast<T *>(p + n);
+                    n += ((size_t)count * sizeof(T) + 31) / 32 * 32;
+                };
+                take(b64.ref, V * rd.N);
+                take(b64.refn, V * rd.N);
+                take(b64.plan, I);
+                take(b64.vstart, V);
+                take(b64.vcnt, V);
+                take(b64.item0, V + 1);
+                take(b64.ticket, 1);
+                return n;
+            };
+            BART_TRY(ctx->band64_ws.ensure(carve(nullptr), "band plans and items"));
+            carve(ctx->band64_ws.p);
+        }
+    }
+    // the FP64 direct sum splits each row's facet list over several warps when the
     // rows alone would not fill the GPU; their partial sums need scratch
     int fp64_chunks = 1;
-    if (path == BART_PATH_FP64) {
+    if (path == BART_PATH_FP64 && !band64) {
         fp64_chunks = synth_fp64_chunks(rd, B * O, F);
         if (fp64_chunks > 1)
             BART_TRY(ctx->partial.ensure((size_t)fp64_chunks * B * O * rd.N * rd.M * 2,
@@ -1023,7 +1092,7 @@ static int run_frame(bart_ctx *ctx, double t0, int32_t path, void *adc, int32_t 
                           ctx->counters.p + 3, ctx->status.p, s);
         launch_compact(ctx->state.p, F, rd, ctx->blk_cnt.p, ctx->vis_idx.p, ctx->vis_cnt.p, s);
         launches += 1 + 3;
-        if (B > 1 && !(band && !stats)) {
+        if (B > 1 && !((band || band64) && !stats)) {
             launch_scene_lists(ctx->vis_idx.p, ctx->vis_cnt.p, F, O, ctx->d_foff.p, B, ctx->vstart.p,
                                ctx->vcnt.p, s);
             launches += 1;
@@ -1152,9 +1221,16 @@ static int run_frame(bart_ctx *ctx, double t0, int32_t path, void *adc, int32_t 
             a.n0 = 0;
             a.nc = rd.N;
             a.partial = fp64_chunks > 1 ? ctx->partial.p : nullptr;
-            launch_synth_fp64(a, s);
+            if (band64) {
+                launch_band64_plan(b64, a, s);
+                launch_synth_band64(b64, a, s);
+                if (stats) launch_count_records64(a, s);
+                launches += stats ? 8 : 7;
+            } else {
+                launch_synth_fp64(a, s);
+                launches += fp64_chunks > 1 ? 2 : 1;
+            }
             ctx->chunks = 1;
-            launches += fp64_chunks > 1 ? 2 : 1;
         }
         // 5. the double-bounce echo, added into the cube (FP64 on every path)
         if (bounce && ctx->db_n > 0) {
