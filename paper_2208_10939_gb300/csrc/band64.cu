@@ -271,8 +271,17 @@ __device__ __forceinline__ int band64_item_count(const Band64Shape &sh, const Ba
                               band64_chunks(sh, pl, cnt);
 }
 
+// the adjoint's items: a chirp node and kAdjFacets facets each
+constexpr int kAdjFacets = 128;
+
+__device__ __forceinline__ int band64_adjoint_count(const Band64Shape &sh, const Band64Plan &pl,
+                                                    int cnt)
+{
+    return sh.kn[pl.in] * ((cnt + kAdjFacets - 1) / kAdjFacets);
+}
+
 // item prefix (one block)
-__global__ void __launch_bounds__(1024) band64_items_kernel(Band64Args b)
+__global__ void __launch_bounds__(1024) band64_items_kernel(Band64Args b, int adjoint)
 {
     __shared__ int s_w[32], s_run;
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
@@ -284,7 +293,9 @@ __global__ void __launch_bounds__(1024) band64_items_kernel(Band64Args b)
     __syncthreads();
     for (int v0 = 0; v0 < V; v0 += 1024) {
         const int v = v0 + t;
-        const int items = v < V ? band64_item_count(b.sh, b.plan[v / b.O], b.vcnt[v]) : 0;
+        const int items = v >= V ? 0
+                          : adjoint ? band64_adjoint_count(b.sh, b.plan[v / b.O], b.vcnt[v])
+                                    : band64_item_count(b.sh, b.plan[v / b.O], b.vcnt[v]);
         int x = items;
         for (int off = 1; off < 32; off <<= 1) {
             const int u = __shfl_up_sync(0xffffffffu, x, off);
@@ -675,6 +686,451 @@ __global__ void __launch_bounds__(128) count_records64_kernel(SynthArgs A)
     }
 }
 
+// -------------------------------------------------------------------------
+// adjoint: the transposes of the interpolation, then each facet's reverse
+// pass over its node terms.  With H[n][m] = conj(G) scale(m) exp(j 2 pi ref),
+// the loss varies as Re sum_{j,s} Hc[j][s] dC[j][s],
+//   Hc[j][s] = sum_n Wn[n][j] sum_m Wm[m][s] H[n][m].
+// -------------------------------------------------------------------------
+
+// Y[j][m] = sum_n Wn[n][j] H[n][m], 16 samples of an (instance, channel) a block
+__global__ void __launch_bounds__(256)
+band64_gather_kernel(Band64Args b, RadarDev rd, const void *__restrict__ grad, int grad_c64)
+{
+    constexpr int R = 256 / kExpM;                // rows at once
+    __shared__ double2 s_h[R][kExpM];
+    __shared__ double2 s_turn[256];
+    s_turn[threadIdx.x] = b.turn[threadIdx.x];
+    __syncthreads();
+    const int v = blockIdx.y, i = v / b.O, o = v % b.O;
+    if (b.vcnt[v] == 0) return;
+    const Band64Plan pl = b.plan[i];
+    const int N = b.sh.N, M = b.sh.M, nj = b.sh.kn[pl.in];
+    const int mm = threadIdx.x & (kExpM - 1), nn = threadIdx.x / kExpM;
+    const int m = blockIdx.x * kExpM + mm;
+    int scene = 0;
+    while (b.scene_inst[scene + 1] <= i) ++scene;
+    const double fm = rd.f0 + rd.slope * (double)m / rd.fs, km = 2.0 * kPi * fm / kC0;
+    const double sc = 2.0 * sqrt(kPi) / pow(4.0 * kPi, 1.5) / (km * km);
+    const double tau = (m - 0.5 * (rd.M - 1)) / rd.fs;
+    const int64_t row = ((int64_t)scene * b.O + o) * N;
+    double2 *Y = b.coarse + (int64_t)v * kB64Room * N * M;
+    const auto h_at = [&](int n) -> double2 {
+        double2 g;
+        if (grad_c64) {
+            const float2 f = static_cast<const float2 *>(grad)[(row + n) * M + m];
+            g = make_double2(f.x, f.y);
+        } else {
+            g = static_cast<const double2 *>(grad)[(row + n) * M + m];
+        }
+        g = make_double2(g.x * sc, -g.y * sc);
+        if (!pl.rotate) return g;
+        const double4 r = b.ref[(int64_t)v * N + n];
+        double c, s;
+        turn_exp(frac1(fma(tau, fma(tau, r.z, r.y), r.x)), s_turn, c, s);
+        return make_double2(g.x * c - g.y * s, g.x * s + g.y * c);
+    };
+    if (pl.in == 0) {
+        for (int n = nn; n < N; n += R) Y[(int64_t)n * M + m] = h_at(n);
+        return;
+    }
+    const double *w = b.wn + b.sh.wn[pl.in];
+    for (int j0 = 0; j0 < nj; j0 += 2 * R) {
+        const int ja = j0 + nn, jb = ja + R;
+        double2 ya = make_double2(0.0, 0.0), yb = ya;
+        for (int n0 = 0; n0 < N; n0 += R) {
+            __syncthreads();
+            if (n0 + nn < N) s_h[nn][mm] = h_at(n0 + nn);
+            __syncthreads();
+            const int lim = min(R, N - n0);
+            for (int q = 0; q < lim; ++q) {
+                const double2 h = s_h[q][mm];
+                if (ja < nj) {
+                    const double wa = pl.in == 1 ? 1.0 : w[(int64_t)(n0 + q) * nj + ja];
+                    ya.x = fma(wa, h.x, ya.x);
+                    ya.y = fma(wa, h.y, ya.y);
+                }
+                if (jb < nj) {
+                    const double wb = w[(int64_t)(n0 + q) * nj + jb];
+                    yb.x = fma(wb, h.x, yb.x);
+                    yb.y = fma(wb, h.y, yb.y);
+                }
+            }
+        }
+        if (ja < nj) Y[(int64_t)ja * M + m] = ya;
+        if (jb < nj) Y[(int64_t)jb * M + m] = yb;
+    }
+}
+
+// Hc[j][s] = sum_m Wm[m][s] Y[j][m], a node a thread
+__global__ void __launch_bounds__(128) band64_gather_samples_kernel(Band64Args b)
+{
+    const int v = blockIdx.y;
+    if (b.vcnt[v] == 0) return;
+    const Band64Plan pl = b.plan[v / b.O];
+    const int M = b.sh.M, nj = b.sh.kn[pl.in], Km = b.sh.km[pl.im];
+    const double2 *Y = b.coarse + (int64_t)v * kB64Room * b.sh.N * M;
+    double2 *H = b.coarse + ((int64_t)v * kB64Room + 1) * b.sh.N * M;
+    for (int e = blockIdx.x * 128 + threadIdx.x; e < nj * Km; e += gridDim.x * 128) {
+        const int j = e / Km, s = e - j * Km;
+        const double2 *y = Y + (int64_t)j * M;
+        double2 h = make_double2(0.0, 0.0);
+        if (pl.im == 0) {
+            h = y[s];
+        } else {
+            const double *w = b.wm + b.sh.wm[pl.im] + (int64_t)s * M;
+#pragma unroll 8
+            for (int m = 0; m < M; ++m) {
+                h.x = fma(w[m], y[m].x, h.x);
+                h.y = fma(w[m], y[m].y, h.y);
+            }
+        }
+        H[e] = h;
+    }
+}
+
+struct V3 {
+    double x, y, z;
+};
+__device__ __forceinline__ V3 v3(double x, double y, double z) { return V3{x, y, z}; }
+__device__ __forceinline__ V3 v3(const double *p) { return V3{p[0], p[1], p[2]}; }
+__device__ __forceinline__ V3 operator+(V3 a, V3 b) { return V3{a.x + b.x, a.y + b.y, a.z + b.z}; }
+__device__ __forceinline__ V3 operator-(V3 a, V3 b) { return V3{a.x - b.x, a.y - b.y, a.z - b.z}; }
+__device__ __forceinline__ V3 operator*(double s, V3 a) { return V3{s * a.x, s * a.y, s * a.z}; }
+__device__ __forceinline__ double dot(V3 a, V3 b) { return fma(a.x, b.x, fma(a.y, b.y, a.z * b.z)); }
+__device__ __forceinline__ V3 cross(V3 a, V3 b)
+{
+    return V3{a.y * b.z - a.z * b.y, a.z * b.x - a.x * b.z, a.x * b.y - a.y * b.x};
+}
+
+// Reverse pass of build_record (facet delay form): gp[10] = sum over the record's
+// entries of bar[entry] d entry / d (vertex coordinates, reflectivity); bq: bars of
+// qt0, qt1, qr0, qr1; bd: of d[0..15].  The centroid is the vertices' mean.
+__device__ __forceinline__ void record_reverse(const double *tri, const double *c0, const double *vel,
+                                               double tn, const double *ptx, const double *prx,
+                                               double rho, int intra, double k0, int two_sided,
+                                               int kind, const double *bq, const double *bd,
+                                               double *gp)
+{
+    const V3 c = v3(c0), vv = v3(vel);
+    V3 dv[3], bdv[3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        dv[i] = v3(tri + 3 * i) - c;
+        bdv[i] = v3(0.0, 0.0, 0.0);
+    }
+    const V3 cc = c + tn * vv;
+    const V3 e1 = dv[1] - dv[0], e2 = dv[2] - dv[0], nr = cross(e1, e2);
+    const double nl = sqrt(dot(nr, nr)), inl = 1.0 / nl, area = 0.5 * nl;
+    const V3 n = inl * nr;
+    const V3 dt = v3(ptx) - cc, dr = v3(prx) - cc;
+    const double it = 1.0 / sqrt(dot(dt, dt)), ir = 1.0 / sqrt(dot(dr, dr));
+    const V3 b = it * dt + ir * dr;
+    const double bn = dot(b, n), sg = two_sided && bn < 0.0 ? -0.5 : 0.5;
+    const double ok = sg * bn, g = rho * ok * it * ir;
+    const V3 bt = b - bn * n;
+    double u[3], bu[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+    for (int i = 0; i < 3; ++i) u[i] = dot(bt, dv[i]);
+    const double A2 = 2.0 * area * g;
+    double bA2 = 0.0, bg = 0.0;
+    V3 bbt = v3(0.0, 0.0, 0.0), bnv = v3(0.0, 0.0, 0.0);
+    if (kind == kRecVertex) {
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            const int i1 = (i + 1) % 3, i2 = (i + 2) % 3;
+            const double p = 1.0 / (u[i] - u[i1]), q = 1.0 / (u[i] - u[i2]);
+            const double f = -p * q, t = bd[3 + i] * A2 * f;
+            bA2 += bd[3 + i] * f;
+            bu[i] += bd[i] - t * (p + q);
+            bu[i1] += t * p;
+            bu[i2] += t * q;
+        }
+    } else if (kind == kRecSeries) {
+        const double ub = (u[0] + u[1] + u[2]) / 3.0;
+        const double y0 = k0 * (u[0] - ub), y1 = k0 * (u[1] - ub), y2 = k0 * (u[2] - ub);
+        const double s2 = y0 * y1 + y0 * y2 + y1 * y2, s3 = y0 * y1 * y2;
+        double h[15], bh[15];
+        h[0] = 1.0;
+        h[1] = 0.0;
+        h[2] = -s2;
+        for (int p = 3; p < 15; ++p) h[p] = -s2 * h[p - 2] + s3 * h[p - 3];
+        const double sc = A2 * k0 * k0;
+        double bsc = 0.0, b2 = 0.0, b3 = 0.0;
+        for (int i = 0; i < 8; ++i) {
+            const double w = ((i & 1) ? -1.0 : 1.0) * c_inv_fact[2 * i + 2] * bd[1 + i];
+            bh[2 * i] = sc * w;
+            bsc += h[2 * i] * w;
+        }
+        for (int i = 0; i < 7; ++i) {
+            const double w = ((i & 1) ? 1.0 : -1.0) * c_inv_fact[2 * i + 3] * bd[9 + i];
+            bh[2 * i + 1] = sc * w;
+            bsc += h[2 * i + 1] * w;
+        }
+        for (int p = 14; p >= 3; --p) {
+            b2 -= bh[p] * h[p - 2];
+            bh[p - 2] -= s2 * bh[p];
+            b3 += bh[p] * h[p - 3];
+            bh[p - 3] += s3 * bh[p];
+        }
+        b2 -= bh[2];
+        bA2 = bsc * k0 * k0;
+        const double by0 = b2 * (y1 + y2) + b3 * y1 * y2, by1 = b2 * (y0 + y2) + b3 * y0 * y2,
+                     by2 = b2 * (y0 + y1) + b3 * y0 * y1;
+        const double m = (bd[0] - k0 * (by0 + by1 + by2)) / 3.0;
+        bu[0] = k0 * by0 + m;
+        bu[1] = k0 * by1 + m;
+        bu[2] = k0 * by2 + m;
+    } else {
+        const double ib2 = 1.0 / dot(bt, bt), kg = k0 * g * ib2;
+        const V3 nxb = cross(n, bt);
+        V3 bx = v3(0.0, 0.0, 0.0);
+        double bb2 = 0.0;
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            const int i1 = (i + 1) % 3;
+            const V3 e = dv[i1] - dv[i];
+            const double x = dot(e, nxb), w = bd[3 * i + 2], t = 0.5 * k0 * bd[3 * i + 1];
+            bu[i] += 0.5 * bd[3 * i] - t;
+            bu[i1] += 0.5 * bd[3 * i] + t;
+            bg += w * k0 * x * ib2;
+            bb2 -= w * kg * x * ib2;
+            const V3 be = (w * kg) * nxb;
+            bdv[i1] = bdv[i1] + be;
+            bdv[i] = bdv[i] - be;
+            bx = bx + (w * kg) * e;
+        }
+        bnv = cross(bt, bx);
+        bbt = cross(bx, n) + (2.0 * bb2) * bt;
+    }
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        bbt = bbt + bu[i] * dv[i];
+        bdv[i] = bdv[i] + bu[i] * bt;
+    }
+    const double barea = 2.0 * g * bA2;
+    bg += 2.0 * area * bA2;
+    V3 bb = bbt;
+    const double bbn = -dot(bbt, n) + sg * bg * rho * it * ir;   // through bt and the obliquity
+    bnv = bnv - bn * bbt + bbn * b;
+    bb = bb + bbn * n;
+    const double bRt = -bg * g * it - dot(bb, dt) * it * it;
+    const double bRr = -bg * g * ir - dot(bb, dr) * ir * ir;
+    V3 bdt = it * bb + (2.0 * bq[0] + bRt * it) * dt;
+    V3 bdr = ir * bb + (2.0 * bq[2] + bRr * ir) * dr;
+    if (intra) {
+        bdt = bdt - (2.0 * bq[1]) * vv;
+        bdr = bdr - (2.0 * bq[3]) * vv;
+    }
+    const V3 bnr = inl * (bnv - dot(n, bnv) * n) + (0.5 * barea) * n;
+    const V3 be1 = cross(e2, bnr), be2 = cross(bnr, e1);
+    bdv[1] = bdv[1] + be1;
+    bdv[2] = bdv[2] + be2;
+    bdv[0] = bdv[0] - be1 - be2;
+    const V3 bc = (1.0 / 3.0) * (v3(0.0, 0.0, 0.0) - bdt - bdr - bdv[0] - bdv[1] - bdv[2]);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        gp[3 * i] = bdv[i].x + bc.x;
+        gp[3 * i + 1] = bdv[i].y + bc.y;
+        gp[3 * i + 2] = bdv[i].z + bc.z;
+    }
+    gp[9] = bg * ok * it * ir;
+}
+
+// Work item = (instance, channel, chirp node, 128 facets), a facet a lane: the
+// nodes' constants go round through shared memory, so that a lane's sums need
+// no exchange, and its reverse pass follows in registers.  The FP64 pipe
+// bounds it (some 95 operations a node).
+__global__ void __launch_bounds__(kAdjFacets)
+adjoint_band64_kernel(SynthArgs A, Band64Args b, double *__restrict__ gfac)
+{
+    constexpr int kInv = 21;                      // entries of a lane's column
+    __shared__ double s_r[kInv + 10][kAdjFacets]; // d[16], L[5], 1 / (2 leg) quartics
+    __shared__ double2 s_turn[256];
+    __shared__ Node64 s_node[kSeg];
+    __shared__ double2 s_h[kSeg];
+    __shared__ int s_item;
+    const int t = threadIdx.x;
+    for (int i = t; i < 256; i += blockDim.x) s_turn[i] = b.turn[i];
+    const RadarDev &rd = A.rd;
+    const int V = b.I * b.O, total = b.item0[V];
+    const double c = kC0;
+    const double k0 = 2.0 * kPi * rd.f0 / c;
+    const double kmax = 2.0 * kPi * (rd.f0 + rd.slope * (rd.M - 1) / rd.fs) / c;
+    const double mu_2c2 = rd.slope / (2.0 * c * c);
+    for (;;) {
+        __syncthreads();
+        if (t == 0) s_item = atomicAdd(b.ticket, 1);
+        __syncthreads();
+        if (s_item >= total) return;
+        const int v = band64_find(b.item0, V, s_item);
+        const int i = v / b.O, o = v % b.O, cnt = b.vcnt[v];
+        const Band64Plan pl = b.plan[i];
+        const int Km = b.sh.km[pl.im], parts = (cnt + kAdjFacets - 1) / kAdjFacets;
+        const int at = s_item - b.item0[v], j = at / parts;
+        const int e = (at - j * parts) * kAdjFacets + t;
+        const bool valid = e < cnt;
+        const int tx = o / rd.Q, rx = o % rd.Q;
+        const double tn = chirp_start(rd, b.xn[b.sh.xn[pl.in] + j], tx);
+        const double *ptx = rd.ant[tx], *prx = rd.ant[rd.P + rx];
+        const double4 ref = b.refn[(int64_t)v * b.sh.N + j];
+        const double2 *H = b.coarse + ((int64_t)v * kB64Room + 1) * b.sh.N * b.sh.M + (int64_t)j * Km;
+        const int64_t k = valid ? A.vis_idx[(int64_t)o * A.F + b.vstart[v] + e] : 0;
+        int kind = -1, flags = 0, quartic = 0;
+        if (valid) {
+            Rec64 R;
+            band64_record(A, k, tn, ptx, prx, k0, kmax, R);
+            kind = R.kind;
+            flags = R.flags;
+            quartic = R.quartic;
+            for (int q = 0; q < 16; ++q) s_r[q][t] = R.d[q];
+            for (int q = 0; q < 5; ++q) s_r[16 + q][t] = R.L[q];
+            if (quartic) {
+                // 1 / (2 sqrt(Q + q1 tau + q2 tau^2)) = h (1 + u)^(-1/2) to tau^4,
+                // u = a tau + a2 tau^2
+                const int inst = A.fac[k].inst;
+                const double *vel = A.vel64 + 3 * inst;
+                const double hc = rd.intra ? 0.5 * (rd.M - 1) / rd.fs : 0.0;
+                const double q2 = rd.intra ? vel[0] * vel[0] + vel[1] * vel[1] + vel[2] * vel[2] : 0.0;
+                for (int leg = 0; leg < 2; ++leg) {
+                    const double *pa = leg ? prx : ptx;
+                    double Q = 0.0, q1 = 0.0;
+                    for (int r = 0; r < 3; ++r) {
+                        const double x = pa[r] - (A.c64[3 * k + r] + vel[r] * (tn + hc));
+                        Q += x * x;
+                        q1 -= 2.0 * x * vel[r];
+                    }
+                    const double iQ = 1.0 / Q, a = rd.intra ? q1 * iQ : 0.0, a2 = q2 * iQ;
+                    const double h = 0.5 * sqrt(iQ), aa = a * a;
+                    double *w = &s_r[kInv + 5 * leg][t];
+                    w[0] = h;
+                    w[kAdjFacets] = -0.5 * a * h;
+                    w[2 * kAdjFacets] = h * (0.375 * aa - 0.5 * a2);
+                    w[3 * kAdjFacets] = h * a * (0.75 * a2 - 0.3125 * aa);
+                    w[4 * kAdjFacets] = h * (0.375 * a2 * a2 - 0.9375 * aa * a2 + 0.2734375 * aa * aa);
+                }
+            }
+        }
+        double bd[16], bq[4];
+#pragma unroll
+        for (int q = 0; q < 16; ++q) bd[q] = 0.0;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) bq[q] = 0.0;
+        const auto D = [&](int q) { return s_r[q][t]; };
+        for (int s0 = 0; s0 < Km; s0 += kSeg) {
+            __syncthreads();
+            const int ns = min(kSeg, Km - s0);
+            for (int s = t; s < ns; s += blockDim.x) {
+                s_node[s] = band64_node(rd, b.xm[b.sh.xm[pl.im] + s0 + s], ref);
+                s_h[s] = H[s0 + s];
+            }
+            __syncthreads();
+            if (!valid) continue;
+            for (int s = 0; s < ns; ++s) {
+                const Node64 &nd = s_node[s];
+                const double gr = s_h[s].x, gi = s_h[s].y, tau = nd.tau;
+                double L, it, ir;
+                if (quartic) {
+                    L = fma(tau, fma(tau, fma(tau, fma(tau, D(20), D(19)), D(18)), D(17)), D(16));
+                    it = fma(tau, fma(tau, fma(tau, fma(tau, D(25), D(24)), D(23)), D(22)), D(21));
+                    ir = fma(tau, fma(tau, fma(tau, fma(tau, D(30), D(29)), D(28)), D(27)), D(26));
+                } else {
+                    const double st = sqrt(D(16) + nd.t * (D(17) + nd.t * D(18)));
+                    const double sr = sqrt(D(19) + nd.t * (D(20) + nd.t * D(18)));
+                    L = st + sr;
+                    it = 0.5 / st;
+                    ir = 0.5 / sr;
+                }
+                const double fmc = nd.fmc, kp = nd.kp;
+                const double th = frac1(L * fma(-mu_2c2, L, fmc)) - nd.rp;
+                double ath = 0.0, cs, sn;             // d / d phase, over -2 pi
+                if (kind == kRecVertex) {
+#pragma unroll
+                    for (int q = 0; q < 3; ++q) {
+                        turn_exp(fma(-fmc, D(q), th), s_turn, cs, sn);
+                        const double zr = gr * cs - gi * sn, zi = D(3 + q) * (gr * sn + gi * cs);
+                        bd[3 + q] += zr;
+                        bd[q] = fma(fmc, zi, bd[q]);
+                        ath += zi;
+                    }
+                } else if (kind == kRecSeries) {
+                    turn_exp(fma(-fmc, D(0), th), s_turn, cs, sn);
+                    const double zr = gr * cs - gi * sn, zi = gr * sn + gi * cs;
+                    const double k2 = kp * kp;
+                    double a = D(8), bb = D(15);
+#pragma unroll
+                    for (int q = 6; q >= 0; --q) a = fma(a, k2, D(1 + q));
+#pragma unroll
+                    for (int q = 5; q >= 0; --q) bb = fma(bb, k2, D(9 + q));
+                    double pw = k2;
+#pragma unroll
+                    for (int q = 0; q < 8; ++q) {
+                        bd[1 + q] = fma(zr, pw, bd[1 + q]);
+                        if (q < 7) bd[9 + q] = fma(-zi * kp, pw, bd[9 + q]);
+                        pw *= k2;
+                    }
+                    ath = zr * (bb * k2 * kp) + zi * (a * k2);
+                    bd[0] = fma(fmc, ath, bd[0]);
+                } else {
+#pragma unroll
+                    for (int q = 0; q < 3; ++q) {
+                        turn_exp(fma(-fmc, D(3 * q), th), s_turn, cs, sn);
+                        const double zr = gr * cs - gi * sn, zi = gr * sn + gi * cs;
+                        const double x = kp * D(3 * q + 1);
+                        double f, fp;                 // sin x / x and its derivative
+                        if (flags & (1 << q)) {
+                            const double x2 = x * x;
+                            f = 1.0 + x2 * (-1.0 / 6 + x2 * (1.0 / 120 + x2 * (-1.0 / 5040 +
+                                x2 * (1.0 / 362880 + x2 * (-1.0 / 39916800)))));
+                            fp = x * (-1.0 / 3 + x2 * (1.0 / 30 + x2 * (-1.0 / 840 +
+                                 x2 * (1.0 / 45360 + x2 * (-1.0 / 3991680)))));
+                        } else {
+                            double sx, cx;
+                            sincos(x, &sx, &cx);
+                            const double ix = 1.0 / x;
+                            f = sx * ix;
+                            fp = (cx - f) * ix;
+                        }
+                        const double w = kp * D(3 * q + 2), coef = w * f;
+                        bd[3 * q + 2] = fma(-zi * kp, f, bd[3 * q + 2]);
+                        bd[3 * q + 1] = fma(-zi * w, fp * kp, bd[3 * q + 1]);
+                        bd[3 * q] = fma(coef * fmc, zr, bd[3 * q]);
+                        ath = fma(coef, zr, ath);
+                    }
+                }
+                // phase -> path length -> the legs' squared-range coefficients
+                const double aL = ath * fma(-2.0 * mu_2c2, L, fmc);
+                const double wt = aL * it, wr = aL * ir;
+                bq[0] += wt;
+                bq[1] = fma(wt, nd.t, bq[1]);
+                bq[2] += wr;
+                bq[3] = fma(wr, nd.t, bq[3]);
+            }
+        }
+        if (!valid) continue;
+        const double p2 = 2.0 * kPi;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) bq[q] *= -p2;
+        if (kind == kRecVertex) {
+#pragma unroll
+            for (int q = 0; q < 3; ++q) bd[q] *= p2;
+        } else if (kind == kRecSeries) {
+            bd[0] *= p2;
+        } else {
+#pragma unroll
+            for (int q = 0; q < 3; ++q) bd[3 * q] *= p2;
+        }
+        double tri[9], c0[3], gp[10];
+        const int inst = A.fac[k].inst;
+        for (int q = 0; q < 9; ++q) tri[q] = A.tri64[9 * k + q];
+        for (int r = 0; r < 3; ++r) c0[r] = A.c64[3 * k + r];
+        record_reverse(tri, c0, A.vel64 + 3 * inst, tn, ptx, prx, (double)A.fac[k].rho, rd.intra, k0,
+                       A.fac[k].two_sided, kind, bq, bd, gp);
+#pragma unroll
+        for (int p = 0; p < 10; ++p) atomicAdd(gfac + 10 * k + p, gp[p]);
+    }
+}
+
 }  // namespace
 
 void launch_band64_tables(const Band64Args &b, cudaStream_t s)
@@ -696,7 +1152,7 @@ void launch_synth_band64(const Band64Args &b, const SynthArgs &a, cudaStream_t s
 {
     const int V = b.I * b.O;
     band64_lists_kernel<<<(V + 3) / 4, 128, 0, s>>>(b, a.vis_idx, a.vis_cnt, a.F);
-    band64_items_kernel<<<1, 1024, 0, s>>>(b);
+    band64_items_kernel<<<1, 1024, 0, s>>>(b, 0);
     int dev = 0, sms = 0, per_sm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -706,6 +1162,23 @@ void launch_synth_band64(const Band64Args &b, const SynthArgs &a, cudaStream_t s
     const int tiles = (b.sh.M / kExpM) * ((b.sh.N + kExpN - 1) / kExpN);
     band64_expand_kernel<<<dim3((unsigned int)tiles, (unsigned int)b.O, (unsigned int)b.B), 256, 0,
                            s>>>(b, a.rd, a.out, a.out_c64);
+}
+
+void launch_adjoint_band64(const Band64Args &b, const SynthArgs &a, const void *grad, int grad_c64,
+                           double *gfac, cudaStream_t s)
+{
+    const int V = b.I * b.O;
+    cudaMemsetAsync(gfac, 0, (size_t)a.F * 10 * sizeof(double), s);
+    band64_lists_kernel<<<(V + 3) / 4, 128, 0, s>>>(b, a.vis_idx, a.vis_cnt, a.F);
+    band64_items_kernel<<<1, 1024, 0, s>>>(b, 1);
+    band64_gather_kernel<<<dim3((unsigned int)(b.sh.M / kExpM), (unsigned int)V), 256, 0, s>>>(
+        b, a.rd, grad, grad_c64);
+    band64_gather_samples_kernel<<<dim3(8, (unsigned int)V), 128, 0, s>>>(b);
+    int dev = 0, sms = 0, per_sm = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, adjoint_band64_kernel, kAdjFacets, 0);
+    adjoint_band64_kernel<<<std::max(1, sms) * std::max(1, per_sm), kAdjFacets, 0, s>>>(a, b, gfac);
 }
 
 void launch_count_records64(const SynthArgs &a, cudaStream_t s)

@@ -11,7 +11,10 @@
 // the whole instance shares, stays below a facet's.
 //
 // The direct sum is bound by the FP64 pipe (a 64th of the FP32 rate, 86 % busy):
-// its time goes with the samples it evaluates.  A 5k-facet car on 12 channels
+// its time goes with the samples it evaluates.  So it is with the adjoint, whose
+// facet sums over samples become sums over nodes once the cube's gradient has
+// gone through the interpolation's transpose (a 1.5k-facet car, 8 channels of 32
+// x 128: 7.95 ms, now 0.84 and 0.06 for the transpose).  A 5k-facet car on 12 channels
 // of 32 x 256 needs 12 x 64 of them and takes 2.7 ms against 33.1.
 #pragma once
 
@@ -71,6 +74,10 @@ void launch_band64_tables(const Band64Args &b, cudaStream_t s);
 void launch_band64_plan(const Band64Args &b, const SynthArgs &a, cudaStream_t s);
 // after the lists: items, node sums, expansion
 void launch_synth_band64(const Band64Args &b, const SynthArgs &a, cudaStream_t s);
+// after the lists: facet gradients gfac [F][10] of the loss whose gradient of the
+// cube is grad (the cube's order)
+void launch_adjoint_band64(const Band64Args &b, const SynthArgs &a, const void *grad, int grad_c64,
+                           double *gfac, cudaStream_t s);
 // per-form record counts of the whole frame (stats)
 void launch_count_records64(const SynthArgs &a, cudaStream_t s);
 

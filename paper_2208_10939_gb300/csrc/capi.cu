@@ -949,7 +949,7 @@ static int run_frame(bart_ctx *ctx, double t0, int32_t path, void *adc, int32_t 
         }
     }
     // FP64: band-limited where that applies and its scratch is to be had
-    bool band64 = path == BART_PATH_FP64 && use_band64(rd, I);
+    bool band64 = (path == BART_PATH_FP64 || path == kPathAdjoint) && use_band64(rd, I);
     Band64Args b64{};
     if (band64) {
         const int64_t V = (int64_t)I * O;
@@ -1208,7 +1208,11 @@ static int run_frame(bart_ctx *ctx, double t0, int32_t path, void *adc, int32_t 
                 a.kquad = ctx->kquad.p;
                 CUDA_TRY(cudaStreamWaitEvent(s, ctx->join_ev, 0), "cudaStreamWaitEvent");
             }
-            if (path == kPathAdjoint)
+            if (path == kPathAdjoint && band64) {
+                launch_band64_plan(b64, a, s);
+                launch_adjoint_band64(b64, a, ctx->adj_grad, ctx->adj_grad_c64, ctx->gfac.p, s);
+                launches += 6;
+            } else if (path == kPathAdjoint)
                 launch_adjoint_fp64(a, ctx->adj_grad, ctx->adj_grad_c64, ctx->gfac.p, s);
             else
                 launch_adjoint_mixed(a, ctx->adj_grad, ctx->adj_grad_c64, ctx->gfac.p, s);

@@ -1,5 +1,5 @@
-"""The band-limited evaluation of the FP64 path (csrc/band64.cuh) against the
-oracle at sampled entries: the ends of its chirp and sample layouts, one chirp,
+"""The band-limited evaluation of the FP64 path (csrc/band64.cuh) and of its
+adjoint, the path against the oracle at sampled entries: the ends of its chirp and sample layouts, one chirp,
 static and moving instances, time-division MIMO, no motion within a chirp, a mesh
 lit from both sides (every chirp kept), targets too near or too fast for the
 tables, few and many facets.
@@ -10,9 +10,11 @@ for the direct sum; a wrong node, weight or reference shows at 1e-3.
 """
 import numpy as np
 import pytest
+import torch
 
 import oracle
 import paper_2208_10939_gb300 as pkg
+from paper_2208_10939_gb300 import autograd as bag
 import scenegen as sg
 
 pytestmark = pytest.mark.gpu
@@ -70,3 +72,59 @@ def test_near_plate(sim, y):
                                                          np.array([0.0, 3.0, 0.0]))],
                   sg.make_radar(64, 12, 1, 2, 5.12e6, 30e12, 2.0, centre=(0.0, 0.0, 0.0)))
     check(sim, sc)
+
+
+def _plate(n, size, vel, two_sided=False):
+    m = sg.plate(size, size, n)
+    m.two_sided = two_sided
+    a = 0.3
+    rot = np.array([[np.cos(a), -np.sin(a), 0.0], [np.sin(a), np.cos(a), 0.0], [0.0, 0.0, 1.0]])
+    return sg.Scene([m], [sg.Instance(0, np.array([0.4, 9.0, 0.2]), rot, np.array(vel))],
+                    sg.make_radar(96, 14, 1, 3, 5.12e6, 20e12, 2.0, centre=(0.0, 0.0, 0.0)))
+
+
+def _car(speed, N, tdm=False, intra=True):
+    sc = sg.car_scene(seed=6, ntri=500, M=128, N=N, P=2, Q=1, slant=22.0)
+    sc.instances[0].vel = np.array([0.6 * speed, -0.8 * speed, 0.0])
+    sc.radar.tdm = tdm
+    sc.radar.intra_chirp_motion = intra
+    return sc
+
+
+# vertex, edge and series forms; static, all layouts, every chirp kept, every sample kept
+ADJOINT = {"car": lambda: _car(9.0, 40), "static": lambda: _car(0.0, 9, tdm=True),
+           "fast": lambda: _car(300.0, 12), "stepped": lambda: _car(9.0, 33, True, False),
+           "edges": lambda: _plate(2, 0.6, [0.0, 2.0, 0.0]),
+           "series": lambda: _plate(60, 0.02, [1.0, -3.0, 0.0]),
+           "two_sided": lambda: _plate(4, 0.5, [0.5, 2.0, 0.0], True)}
+
+
+@pytest.mark.parametrize("name", list(ADJOINT))
+def test_adjoint(sim, name):
+    """The cube is linear in the reflectivities: sum rho dL/drho = L, to the
+    rounding of the paths.  A shift of all vertices against central
+    differences of the cube: step 1e-6 m, (2 k h)^2 / 6 = 2e-6 of the largest
+    derivative the loss can have, 2 k |W| |x|."""
+    sc = ADJOINT[name]()
+    es = bag.EchoScene(sim, sc)
+    verts = es.vertex_tensor(sc, "cuda").requires_grad_(True)
+    rho = torch.from_numpy(sc.meshes[0].rho.copy()).cuda().requires_grad_(True)
+    adc = bag.echo(verts, rho, es)
+    rng = np.random.default_rng(3)
+    W = torch.from_numpy(rng.normal(size=adc.shape) + 1j * rng.normal(size=adc.shape)).cuda()
+    loss = (W.conj() * adc).real.sum()
+    loss.backward()
+    scale = float(W.norm() * adc.detach().norm())
+    lin = float((rho.detach().double() * rho.grad.double()).sum())
+    # (the reflectivities' gradient is returned in their own float32)
+    assert abs(lin - float(loss)) <= 1e-9 * scale + 2.0 ** -24 * float(
+        (rho.detach() * rho.grad).abs().double().sum())
+    h = 1e-6
+    k = 2.0 * np.pi * (sc.radar.f0 + sc.radar.slope * sc.radar.M / sc.radar.fs) / 299792458.0
+    for d in ([0.0, 1.0, 0.0], [0.6, 0.0, 0.8]):
+        step = torch.tensor(d, dtype=torch.float64, device="cuda")
+        with torch.no_grad():
+            up = (W.conj() * bag.echo(verts + h * step, rho, es)).real.sum()
+            dn = (W.conj() * bag.echo(verts - h * step, rho, es)).real.sum()
+        fd = float(up - dn) / (2.0 * h)
+        assert abs(fd - float((verts.grad * step).sum())) <= 5e-6 * 2.0 * k * scale
