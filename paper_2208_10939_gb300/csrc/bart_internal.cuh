@@ -126,6 +126,9 @@ void launch_build_facets(const MeshDesc *meshes, const InstDev *insts, int n_ins
 // Temp words of the multi-launch radix sort, and float4 words of the leaf
 // levels, for n facets.
 int64_t radix_sort_temp_words(int64_t n);
+// stable sort of 32-bit keys by their low `bits`, values along; result in keys / vals
+void radix_sort_pairs(uint32_t *keys, int32_t *vals, uint32_t *keys_tmp, int32_t *vals_tmp,
+                      uint32_t *temp, int64_t n, int bits, cudaStream_t s);
 int64_t leaf_levels_words(int64_t n);
 // Morton codes, sort, hierarchy and boxes; returns the launches.  Batched
 // scenes (B > 1: facets [foff[b], foff[b+1]) form scene b, foff on the

@@ -42,6 +42,7 @@
 #include <algorithm>
 #include <climits>
 
+#include "band.cuh"
 #include "bart_internal.cuh"
 #include "bounce.cuh"
 #include "geom64.cuh"
@@ -793,7 +794,7 @@ __device__ __forceinline__ void centre_phase(double th0, double th1, double u, c
 
 // RecV of a full FP64 record: each leg's path sqrt(q0 + q1 t + q2 t^2)
 // expanded to second order, the centres and amplitudes rounded to FP32
-__device__ __forceinline__ void rec64_to_v(const RecB &R, const PhaseK &K, RecV &V)
+__device__ __forceinline__ void rec64_to_v(const RecB &R, const PhaseK &K, double xref, RecV &V)
 {
     double L0 = 0.0, L1 = 0.0, L2 = 0.0;
     const double *qs[2] = {R.qt, R.qr};
@@ -808,6 +809,8 @@ __device__ __forceinline__ void rec64_to_v(const RecB &R, const PhaseK &K, RecV 
     }
     double th0, th1, th2;
     path_phase(L0, L1, L2, K, th0, th1, th2);
+    th0 -= K.f0c * xref;
+    th1 -= K.mucfs * xref;
     V.C = (float)th2;
     V.kind = R.kind;
     V.flags = R.flags;
@@ -980,12 +983,13 @@ __device__ __forceinline__ float inv_fact_f(int n)
 // which the form switches and the weights' pair differences come too;
 // directions, obliquity and every form's amplitudes in FP32
 // (record_fp64.cuh's forms).  Returns false when a row has
-// no expansion (the record then takes the full FP64 build).
+// no expansion (the record then takes the full FP64 build).  xref: path taken
+// off (the reference of a rate group, else 0).
 __device__ __forceinline__ bool lean_record(const BounceRow &Rt, const BounceRow &Rr,
                                             const BounceGeo &G, float wrho, int two_sided,
                                             double tau, float tn, const RadarDev &rd,
                                             const PhaseK &K, float k0, float kmax,
-                                            float chord0, RecV &V)
+                                            float chord0, double xref, RecV &V)
 {
     if (Rt.a[0] < 0.0 || Rr.a[0] < 0.0) return false;
     double t0, s0;
@@ -1018,6 +1022,8 @@ __device__ __forceinline__ bool lean_record(const BounceRow &Rt, const BounceRow
     double th0, th1, th2;
     path_phase(t0 + s0, rd.intra ? (double)(t1 + s1) : 0.0,
                rd.intra ? (double)(0.5f * (t2 + s2)) : 0.0, K, th0, th1, th2);
+    th0 -= K.f0c * xref;
+    th1 -= K.mucfs * xref;
     double ud[3];                    // u_v in FP64 for the phases
 #pragma unroll
     for (int v = 0; v < 3; ++v) {
@@ -1101,36 +1107,72 @@ __device__ __forceinline__ bool lean_record(const BounceRow &Rt, const BounceRow
 // by every lane over its S samples from an FP32 start phasor and its chord
 // step (the curvature C (S - 1)^2 / 4 cycles, below 1e-5, is left out),
 // the amplitudes of the series and edge forms per sample; batch sums in
-// FP32 added to FP64 totals.
-template <int S>
+// FP32 added to FP64 totals.  GROUPED: the rows are the chirp nodes of the rate
+// groups (see BounceGroup), the sums go to their node rows unscaled.
+template <int S, bool GROUPED>
 __global__ void __launch_bounds__(kDbWarps * 32, kDbF32Blocks)
 bounce_synth_f32_kernel(const BounceFacet *__restrict__ vf, const int64_t *__restrict__ txoff,
                         const FacetRec *__restrict__ fac, const double *__restrict__ vel64,
                         const uint8_t *__restrict__ state, int64_t F, RadarDev rd, int W,
                         void *out, int out_c64, unsigned long long *records,
                         const BounceRow *__restrict__ rows, const BounceGeo *__restrict__ geo,
-                        double tc, int NCH, double2 *__restrict__ partial)
+                        double tc, int NCH, double2 *__restrict__ partial, BounceGroups gr)
 {
     __shared__ RecV sV[kDbWarps][32];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t gw = (int64_t)blockIdx.x * kDbWarps + warp;
     const int N = rd.N;
-    if (gw >= (int64_t)rd.O * N * W * NCH) return;
-    const int chunk = (int)(gw % NCH);
-    const int seg = (int)(gw / NCH % W);
-    const int64_t unit = gw / ((int64_t)NCH * W);
-    const int o = (int)(unit / N), n = (int)(unit % N);
-    const int p = o / rd.Q, q = o % rd.Q;
+    int chunk, seg, p, q, n = 0;
+    double slot, xref = 0.0;                 // chirp; reference path of the group
+    int64_t v0, v1, prow;                    // virtual facets; output row
+    const int32_t *perm = nullptr;
+    if constexpr (GROUPED) {
+        if (gw >= gr.items) return;
+        int lo = 0, hi = gr.groups - 1;      // last group with item0 <= gw
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (gr.group[mid].item0 <= gw) lo = mid;
+            else hi = mid - 1;
+        }
+        const BounceGroup g = gr.group[lo];
+        int at = (int)(gw - g.item0);
+        chunk = at % g.chunks;
+        at /= g.chunks;
+        seg = at % W;
+        at /= W;
+        q = at % rd.Q;
+        n = at / rd.Q;                       // node
+        p = g.p;
+        const float node = g.lay == 0 ? (float)n : gr.nodes[g.node0 + n];
+        slot = (double)node * rd.slots + (rd.tdm ? p : 0);
+        xref = (double)g.rc * (slot * rd.Tc - tc);
+        perm = gr.perm + g.beg;
+        v0 = (int64_t)g.cnt * chunk / g.chunks;
+        v1 = (int64_t)g.cnt * (chunk + 1) / g.chunks;
+        prow = g.row0 + (int64_t)(n * rd.Q + q) * g.chunks + chunk;
+    } else {
+        if (gw >= (int64_t)rd.O * N * W * NCH) return;
+        chunk = (int)(gw % NCH);
+        seg = (int)(gw / NCH % W);
+        const int64_t unit = gw / ((int64_t)NCH * W);
+        const int o = (int)(unit / N);
+        n = (int)(unit % N);
+        p = o / rd.Q;
+        q = o % rd.Q;
+        slot = (double)((int64_t)n * rd.slots + (rd.tdm ? p : 0));
+        // this warp's chunk of the virtual facets of TX p
+        const int64_t vt0 = txoff[p], nv = txoff[p + 1] - vt0;
+        v0 = vt0 + nv * chunk / NCH;
+        v1 = vt0 + nv * (chunk + 1) / NCH;
+        prow = (int64_t)chunk * rd.O * N + (int64_t)o * N + n;
+    }
     const int m0 = (seg * 32 + lane) * S;
     const double c = kC0, f0 = rd.f0, mu = rd.slope, fs = rd.fs;
     const double f_max = f0 + mu * (rd.M - 1) / fs;
     const double k0 = 2.0 * kPi * f0 / c, kmax = 2.0 * kPi * f_max / c;
-    const double tn = (double)((int64_t)n * rd.slots + (rd.tdm ? p : 0)) * rd.Tc;
+    const double tn = slot * rd.Tc;
     const double *prx = rd.ant[rd.P + q];
     const uint8_t *st_r = state + (int64_t)(rd.P + q) * F;
-    // this warp's chunk of the virtual facets of TX p
-    const int64_t vt0 = txoff[p], nv = txoff[p + 1] - vt0;
-    const int64_t v0 = vt0 + nv * chunk / NCH, v1 = vt0 + nv * (chunk + 1) / NCH;
     const float fm0 = (float)m0, fm0sq = fm0 * fm0;
     const PhaseK PK = phase_consts(rd);
 
@@ -1142,9 +1184,10 @@ bounce_synth_f32_kernel(const BounceFacet *__restrict__ vf, const int64_t *__res
     for (int j = 0; j < S; ++j) accr[j] = acci[j] = 0.0;
     unsigned long long nrec = 0;
     for (int64_t base = v0; base < v1; base += 32) {
-        const int64_t v = base + lane;
+        const int64_t at = base + lane;
         bool valid = false;
-        if (v < v1) {
+        if (at < v1) {
+            const int64_t v = GROUPED ? perm[at] : at;
             const BounceFacet &B = vf[v];
             valid = st_r[B.b] == (B.side > 0 ? BART_VIS_LIT : BART_VIS_LIT_REV);
             if (valid) {
@@ -1152,12 +1195,12 @@ bounce_synth_f32_kernel(const BounceFacet *__restrict__ vf, const int64_t *__res
                 const bool lean = lean_record(rows[v * L], rows[v * L + 1 + q], geo[v],
                                               (float)B.w, fac[B.b].two_sided, tn - tc,
                                               (float)tn, rd, PK, k0f, kmaxf, (float)(S - 1),
-                                              sV[warp][lane]);
+                                              xref, sV[warp][lane]);
                 if (!lean) {
                     RecB R64;
                     build_rec64(B, vel64 + 3 * fac[B.b].inst, tn, prx, rd, k0, kmax,
                                 fac[B.b].two_sided, R64);
-                    rec64_to_v(R64, PK, sV[warp][lane]);
+                    rec64_to_v(R64, PK, xref, sV[warp][lane]);
                     chord_steps(sV[warp][lane], (float)(S - 1));
                 }
             }
@@ -1255,17 +1298,23 @@ bounce_synth_f32_kernel(const BounceFacet *__restrict__ vf, const int64_t *__res
         }
         __syncwarp();
     }
+    if constexpr (GROUPED) {
+        if (lane == 0 && seg == 0 && n == 0 && records) atomicAdd(records, nrec * N);
+        double2 *y = partial + prow * rd.M + m0;
+#pragma unroll
+        for (int j = 0; j < S; ++j) y[j] = make_double2(accr[j], acci[j]);
+        return;
+    }
     if (lane == 0 && seg == 0 && records) atomicAdd(records, nrec);
     const double camp = 2.0 * sqrt(kPi) / pow(4.0 * kPi, 1.5);
-    const int64_t row = ((int64_t)o * N + n) * rd.M + m0;
+    const int64_t row = ((int64_t)(p * rd.Q + q) * N + n) * rd.M + m0;
 #pragma unroll
     for (int j = 0; j < S; ++j) {
         const double fm = f0 + mu * (double)(m0 + j) / fs;
         const double km = 2.0 * kPi * fm / c;
         const double sc = camp / (km * km);
         if (NCH > 1) {         // this chunk's scaled partial sums, added in order later
-            partial[(int64_t)chunk * rd.O * N * rd.M + row + j] =
-                make_double2(accr[j] * sc, acci[j] * sc);
+            partial[prow * rd.M + m0 + j] = make_double2(accr[j] * sc, acci[j] * sc);
         } else if (out_c64) {
             float2 &y = reinterpret_cast<float2 *>(out)[row + j];
             y.x += (float)(accr[j] * sc);
@@ -1298,6 +1347,263 @@ __global__ void bounce_reduce_kernel(const double2 *__restrict__ partial, int64_
         double2 &y = reinterpret_cast<double2 *>(out)[i];
         y.x += re;
         y.y += im;
+    }
+}
+
+// -------------------------------------------------------------------------
+// Rate groups (BounceGroup in bounce.cuh): virtual facets of one TX whose paths
+// lengthen at nearly the same rate.
+// -------------------------------------------------------------------------
+constexpr int kDbRateBins = 2048;            // per TX; the last: rows without expansion
+constexpr int kDbKeys = kDbMaxTx * kDbRateBins;
+static_assert(kDbKeys <= 65536 && kDbKeys % 1024 == 0, "16-bit keys, a run of them per thread");
+constexpr int kDbChunk = 256;                // virtual facets of a work item
+
+// key, and the largest phase turn of the key's facets over half the frame
+// after their group's reference: every vertex's path of every RX
+__global__ void __launch_bounds__(128)
+bounce_key_kernel(const BounceFacet *__restrict__ vf, int64_t V, const BounceRow *__restrict__ rows,
+                  RadarDev rd, double h, float width, float kmax, uint32_t *__restrict__ keys,
+                  int32_t *__restrict__ perm, int32_t *__restrict__ cnt,
+                  unsigned int *__restrict__ turn)
+{
+    const int64_t v = (int64_t)blockIdx.x * 128 + threadIdx.x;
+    if (v >= V) return;
+    const BounceRow *R = rows + v * (1 + rd.Q);
+    const float rate = R[0].af[1] + R[1].af[1];
+    int bin = kDbRateBins - 1;
+    bool ok = isfinite(rate);
+    for (int l = 0; l <= rd.Q; ++l) ok = ok && R[l].a[0] >= 0.0;
+    float a = 3e38f;
+    if (ok) {
+        bin = (int)fminf(fmaxf(floorf(rate / width) + 1023.f, 0.f), (float)(kDbRateBins - 2));
+        const float rc = ((float)(bin - 1023) + 0.5f) * width, hf = (float)h;
+        const float mu_c2 = (float)(rd.slope / (kC0 * kC0));
+        a = 0.f;
+        for (int l = 1; l <= rd.Q; ++l) {
+            float bend = 0.f, hp = hf * hf;
+            for (int j = 2; j <= kDbDeg; ++j) {
+                bend += (fabsf(R[0].af[j]) + fabsf(R[l].af[j])) * hp;
+                hp *= hf;
+            }
+            const float r = R[0].af[1] + R[l].af[1];
+            float off = 0.f;
+            for (int c = 0; c < 3; ++c) {
+                float o = fabsf(r - (float)(R[0].pu[c][1] + R[l].pu[c][1]) - rc) * hf;
+                o += (float)(fabs(R[0].pu[c][2] + R[l].pu[c][2]) * h * h +
+                             fabs(R[0].pu[c][3] + R[l].pu[c][3]) * h * h * h);
+                off = fmaxf(off, o);
+            }
+            a = fmaxf(a, kmax * (off + bend) +
+                             6.2831853f * mu_c2 * (R[0].af[0] + R[l].af[0]) * fabsf(r) * hf);
+        }
+        a *= 1.02f;
+    }
+    const uint32_t key = (uint32_t)vf[v].p * kDbRateBins + bin;
+    keys[v] = key;
+    perm[v] = (int32_t)v;
+    atomicAdd(cnt + key, 1);
+    atomicMax(turn + key, __float_as_uint(a));
+}
+
+// exclusive scan over 1024 threads
+__device__ __forceinline__ long long scan1024(long long v, long long &total)
+{
+    __shared__ long long s_w[33];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    long long x = v;
+    for (int o = 1; o < 32; o <<= 1) {
+        const long long y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) s_w[warp] = x;
+    __syncthreads();
+    long long b = 0, t = 0;
+    for (int k = 0; k < 32; ++k) {
+        if (k < warp) b += s_w[k];
+        t += s_w[k];
+    }
+    total = t;
+    __syncthreads();
+    return b + x - v;
+}
+
+__device__ __forceinline__ BounceGroup bounce_group(const BandShape &sh, int key, int cnt, float turn,
+                                                    float width)
+{
+    BounceGroup g;
+    g.cnt = cnt;
+    g.p = key / kDbRateBins;
+    const int bin = key % kDbRateBins;
+    g.rc = bin == kDbRateBins - 1 ? 0.f : ((float)(bin - 1023) + 0.5f) * width;
+    g.lay = 0;
+    for (int l = 2; l < sh.n_n && g.lay == 0; ++l)
+        if (turn <= sh.n[l].amax) g.lay = l;
+    g.nj = g.lay == 0 ? sh.N : sh.n[g.lay].nj;
+    g.node0 = sh.n[g.lay].node0;
+    g.w0 = sh.n[g.lay].w0;
+    g.chunks = (cnt + kDbChunk - 1) / kDbChunk;
+    return g;
+}
+
+// one block: the groups in key order with their first facet, item, partial row
+// and node row; tot: groups, items, partial rows, node rows, records
+__global__ void __launch_bounds__(1024)
+bounce_plan_kernel(BandShape sh, int Q, int W, float width, const int32_t *__restrict__ cnt,
+                   const unsigned int *__restrict__ turn, BounceGroup *__restrict__ group,
+                   int64_t *__restrict__ tot)
+{
+    constexpr int kPer = kDbKeys / 1024;
+    const int k0 = threadIdx.x * kPer;
+    long long s[6] = {0, 0, 0, 0, 0, 0};     // facets, groups, items, rows, nodes, records
+    const auto add = [&](const BounceGroup &g) {
+        s[0] += g.cnt;
+        s[1] += 1;
+        s[2] += (long long)g.nj * Q * W * g.chunks;
+        s[3] += (long long)g.nj * Q * g.chunks;
+        s[4] += (long long)g.nj * Q;
+        s[5] += (long long)g.nj * g.cnt;
+    };
+    for (int k = k0; k < k0 + kPer; ++k)
+        if (cnt[k] > 0) add(bounce_group(sh, k, cnt[k], __uint_as_float(turn[k]), width));
+    long long total[6];
+    for (int i = 0; i < 6; ++i) s[i] = scan1024(s[i], total[i]);
+    for (int k = k0; k < k0 + kPer; ++k)
+        if (cnt[k] > 0) {
+            BounceGroup g = bounce_group(sh, k, cnt[k], __uint_as_float(turn[k]), width);
+            g.beg = (int32_t)s[0];
+            g.item0 = s[2];
+            g.row0 = s[3];
+            g.node_row0 = s[4];
+            group[s[1]] = g;
+            add(g);
+        }
+    if (threadIdx.x == 0)
+        for (int i = 0; i < 5; ++i) tot[i] = total[i + 1];
+}
+
+// the items' sums of each node row (in order) as FP32; y: the groups' reference
+// phase at each chirp, (constant, per sample) cycles
+__global__ void __launch_bounds__(256)
+bounce_node_kernel(BounceGroups gr, RadarDev rd, double tc, const double2 *__restrict__ partial,
+                   float2 *__restrict__ node, float2 *__restrict__ ref)
+{
+    const BounceGroup g = gr.group[blockIdx.x];
+    const int M = rd.M, rows = g.nj * rd.Q;
+    for (int r = blockIdx.y; r < rows; r += gridDim.y) {
+        const double2 *x = partial + (g.row0 + (int64_t)r * g.chunks) * M;
+        float2 *d = node + (g.node_row0 + r) * M;
+        for (int m = threadIdx.x; m < M; m += 256) {
+            double2 a = x[m];
+            for (int k = 1; k < g.chunks; ++k) {
+                const double2 b = x[(int64_t)k * M + m];
+                a.x += b.x;
+                a.y += b.y;
+            }
+            d[m] = make_float2((float)a.x, (float)a.y);
+        }
+    }
+    if (blockIdx.y == 0) {
+        const PhaseK K = phase_consts(rd);
+        for (int n = threadIdx.x; n < rd.N; n += 256) {
+            const double t = ((double)n * rd.slots + (rd.tdm ? g.p : 0)) * rd.Tc;
+            const double x = (double)g.rc * (t - tc);
+            ref[(int64_t)blockIdx.x * rd.N + n] =
+                make_float2((float)red1d(K.f0c * x), (float)(K.mucfs * x));
+        }
+    }
+}
+
+// x[n][m] += scale sum_groups exp(j 2 pi ref) sum_j Wn[n][j] node[j][m]: a block
+// makes 32 chirps of 64 samples of a channel; 16 node rows at a time in shared
+// memory; the groups' terms in compensated FP32 sums
+constexpr int kDbExN = 32, kDbExM = 64, kDbExJ = 16;
+
+__device__ __forceinline__ void kahan(float v, float &sum, float &c)
+{
+    const float y = v - c, t = sum + y;
+    c = (t - sum) - y;
+    sum = t;
+}
+
+__global__ void __launch_bounds__(256)
+bounce_expand_kernel(BounceGroups gr, RadarDev rd, const float2 *__restrict__ node,
+                     const float2 *__restrict__ ref, void *__restrict__ out, int out_c64)
+{
+    constexpr int kRows = 256 / kDbExM, kPer = kDbExN / kRows;
+    __shared__ float2 s_d[kDbExJ][kDbExM];
+    const int M = rd.M, N = rd.N, mt = (M + kDbExM - 1) / kDbExM;
+    const int mm = threadIdx.x % kDbExM, nn = threadIdx.x / kDbExM;
+    const int m = (int)(blockIdx.x % mt) * kDbExM + mm, n0 = (int)(blockIdx.x / mt) * kDbExN + nn;
+    const int o = blockIdx.y, p = o / rd.Q, q = o % rd.Q;
+    const bool in = m < M;
+    float re[kPer], im[kPer], cr[kPer], ci[kPer];
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) re[k] = im[k] = cr[k] = ci[k] = 0.f;
+    for (int gi = 0; gi < gr.groups; ++gi) {
+        const BounceGroup g = gr.group[gi];
+        if (g.p != p) continue;
+        float zr[kPer], zi[kPer];
+#pragma unroll
+        for (int k = 0; k < kPer; ++k) zr[k] = zi[k] = 0.f;
+        if (g.lay == 0) {
+#pragma unroll
+            for (int k = 0; k < kPer; ++k) {
+                const int n = n0 + k * kRows;
+                if (n < N && in) {
+                    const float2 d = node[(g.node_row0 + (int64_t)n * rd.Q + q) * M + m];
+                    zr[k] = d.x;
+                    zi[k] = d.y;
+                }
+            }
+        } else {
+            for (int j0 = 0; j0 < g.nj; j0 += kDbExJ) {
+                const int nj = min(kDbExJ, g.nj - j0);
+                __syncthreads();
+                for (int j = nn; j < nj; j += kRows)
+                    s_d[j][mm] = in ? node[(g.node_row0 + (int64_t)(j0 + j) * rd.Q + q) * M + m]
+                                    : make_float2(0.f, 0.f);
+                __syncthreads();
+                const float *w = gr.wn + g.w0 + j0;
+                for (int j = 0; j < nj; ++j) {
+                    const float2 d = s_d[j][mm];
+#pragma unroll
+                    for (int k = 0; k < kPer; ++k) {
+                        const int n = min(n0 + k * kRows, N - 1);
+                        const float wj = w[(int64_t)n * g.nj + j];
+                        zr[k] = fmaf(wj, d.x, zr[k]);
+                        zi[k] = fmaf(wj, d.y, zi[k]);
+                    }
+                }
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < kPer; ++k) {
+            const float2 r = ref[(int64_t)gi * N + min(n0 + k * kRows, N - 1)];
+            float s, c;
+            sincospif(2.f * red1f(fmaf(r.y, (float)m, r.x)), &s, &c);
+            kahan(zr[k] * c - zi[k] * s, re[k], cr[k]);
+            kahan(zr[k] * s + zi[k] * c, im[k], ci[k]);
+        }
+    }
+    if (!in) return;
+    const double fm = rd.f0 + rd.slope * (double)m / rd.fs;
+    const double km = 2.0 * kPi * fm / kC0;
+    const double sc = 2.0 * sqrt(kPi) / pow(4.0 * kPi, 1.5) / (km * km);
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+        const int n = n0 + k * kRows;
+        if (n >= N) break;
+        const int64_t e = ((int64_t)o * N + n) * M + m;
+        if (out_c64) {
+            float2 &y = static_cast<float2 *>(out)[e];
+            y.x += (float)((double)re[k] * sc);
+            y.y += (float)((double)im[k] * sc);
+        } else {
+            double2 &y = static_cast<double2 *>(out)[e];
+            y.x += (double)re[k] * sc;
+            y.y += (double)im[k] * sc;
+        }
     }
 }
 
@@ -1404,11 +1710,37 @@ int bounce_synth_chunks(const RadarDev &rd)
     return (int)std::max<int64_t>(1, std::min<int64_t>(16, (target + rows - 1) / rows));
 }
 
+bool bounce_groups_apply(const RadarDev &rd, const BandShape &sh)
+{
+    return sh.n_n > 2 && bounce_mid_time(rd) > 0.0;
+}
+
+int64_t bounce_group_keys() { return kDbKeys; }
+
+void launch_bounce_groups(const BounceFacet *vf, int64_t V, const void *rows, const RadarDev &rd,
+                          const BandShape &sh, uint32_t *keys, int32_t *perm, uint32_t *keys_tmp,
+                          int32_t *perm_tmp, uint32_t *sort_temp, int32_t *cnt, BounceGroup *group,
+                          int64_t *tot, cudaStream_t s)
+{
+    unsigned int *turn = reinterpret_cast<unsigned int *>(cnt) + kDbKeys;
+    cudaMemsetAsync(cnt, 0, (size_t)2 * kDbKeys * sizeof(int32_t), s);
+    const double h = bounce_mid_time(rd);
+    const double kmax = 2.0 * kPi * (rd.f0 + rd.slope * (rd.M - 1) / rd.fs) / kC0;
+    const float width = (float)(2.0 * kDbGroupTurn / (kmax * h));
+    bounce_key_kernel<<<(unsigned int)((V + 127) / 128), 128, 0, s>>>(
+        vf, V, static_cast<const BounceRow *>(rows), rd, h, width, (float)kmax, keys, perm, cnt, turn);
+    radix_sort_pairs(keys, perm, keys_tmp, perm_tmp, sort_temp, V, 16, s);
+    int S = 16;
+    while ((rd.M / 32) % S) S /= 2;
+    bounce_plan_kernel<<<1, 1024, 0, s>>>(sh, rd.Q, rd.M / (32 * S), width, cnt, turn, group, tot);
+}
+
 void launch_bounce_synth(const BounceFacet *vf, const int64_t *txoff, const FacetRec *fac,
                          const double *vel64, const uint8_t *state, int64_t F,
                          const RadarDev &rd, void *out, int out_c64, bool fp32_eval,
                          const void *rows, const void *geo, int NCH, double2 *partial,
-                         unsigned long long *records, cudaStream_t s)
+                         const BounceGroups *groups, unsigned long long *records,
+                         cudaStream_t s)
 {
     const int M = rd.M;                // a multiple of 32
     // samples per lane: the largest power of two up to 16 (FP32 evaluation)
@@ -1434,8 +1766,14 @@ void launch_bounce_synth(const BounceFacet *vf, const int64_t *txoff, const Face
     const BounceRow *R = static_cast<const BounceRow *>(rows);
     const BounceGeo *G = static_cast<const BounceGeo *>(geo);
     const double tc = bounce_mid_time(rd);
-    const unsigned int grid = (unsigned int)((warps * NCH + kDbWarps - 1) / kDbWarps);
-#define BART_DB_LAUNCH32(SS) bounce_synth_f32_kernel<SS><<<grid, blk, 0, s>>>(vf, txoff, fac, vel64, state, F, rd, W, out, out_c64, records, R, G, tc, NCH, partial)
+    const bool grouped = groups != nullptr;
+    const int64_t all = grouped ? groups->items : warps * NCH;
+    const unsigned int grid = (unsigned int)((all + kDbWarps - 1) / kDbWarps);
+    const BounceGroups gr = grouped ? *groups : BounceGroups{};
+#define BART_DB_LAUNCH32(SS) do { \
+        if (grouped) bounce_synth_f32_kernel<SS, true><<<grid, blk, 0, s>>>(vf, txoff, fac, vel64, state, F, rd, W, out, out_c64, records, R, G, tc, 1, partial, gr); \
+        else bounce_synth_f32_kernel<SS, false><<<grid, blk, 0, s>>>(vf, txoff, fac, vel64, state, F, rd, W, out, out_c64, records, R, G, tc, NCH, partial, gr); \
+    } while (0)
     switch (S) {
     case 16: BART_DB_LAUNCH32(16); break;
     case 8: BART_DB_LAUNCH32(8); break;
@@ -1444,7 +1782,13 @@ void launch_bounce_synth(const BounceFacet *vf, const int64_t *txoff, const Face
     default: BART_DB_LAUNCH32(1); break;
     }
 #undef BART_DB_LAUNCH32
-    if (NCH > 1) {
+    if (grouped) {
+        bounce_node_kernel<<<dim3((unsigned int)gr.groups, 16), 256, 0, s>>>(gr, rd, tc, partial,
+                                                                            gr.node, gr.ref);
+        const int tiles = ((M + kDbExM - 1) / kDbExM) * ((rd.N + kDbExN - 1) / kDbExN);
+        bounce_expand_kernel<<<dim3((unsigned int)tiles, (unsigned int)rd.O), 256, 0, s>>>(
+            gr, rd, gr.node, gr.ref, out, out_c64);
+    } else if (NCH > 1) {
         const int64_t n = (int64_t)rd.O * rd.N * M;
         bounce_reduce_kernel<<<(unsigned int)((n + 255) / 256), 256, 0, s>>>(partial, n, NCH,
                                                                            out, out_c64);

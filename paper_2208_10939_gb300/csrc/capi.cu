@@ -207,6 +207,11 @@ struct bart_ctx {
     DevBuf<int64_t> db_txoff;           // first virtual facet of each TX [P + 1]
     DevBuf<unsigned char> db_rows;      // FP32 evaluation: slow-time rows and geometry
     DevBuf<double2> db_part;            // FP32 evaluation: the chunks' partial sums
+    DevBuf<uint32_t> db_keys, db_sort;  // rate groups: keys (twice), sort scratch
+    DevBuf<int32_t> db_perm, db_gcnt;   // order (twice), counts and turns of the keys
+    DevBuf<BounceGroup> db_group;
+    DevBuf<int64_t> db_gtot;
+    DevBuf<float2> db_node, db_gref;    // node rows, reference phases
     int64_t db_n = 0;
     DevBuf<uint32_t> mkeys, skeys;      // batched sort scratch
     int tpi_override = 0;               // synthesis tiles per item (autotuner), 0 = default
@@ -289,6 +294,8 @@ struct bart_ctx {
         vcnt.release(); mkeys.release(); skeys.release();
         db_cnt.release(); db_off.release(); db_blk.release(); db_vf.release();
         db_cand.release(); db_pcnt.release(); db_poff.release(); db_pblk.release();
+        db_keys.release(); db_sort.release(); db_perm.release(); db_gcnt.release();
+        db_group.release(); db_gtot.release(); db_node.release(); db_gref.release();
         db_txoff.release(); db_rows.release(); db_part.release(); db_roots.release();
         if (count_host) cudaFreeHost(count_host);
     }
@@ -704,6 +711,55 @@ static int synth_band_target()
     return 6 * 16 * std::max(sms, 1);
 }
 
+// Rate groups of the frame's `total` virtual facets (bounce.cuh), with a host
+// read of their sizes; gr.group stays NULL, and the chirps are all evaluated,
+// where they would save less than a fifth of the records (a group's
+// interpolation costs about a record per chirp) or their scratch exceeds 8 GB
+// or is not to be had.  A 20k-facet car on 3.2k facets of road, 12 channels of
+// 128 x 256: 33.8 ms with every chirp, 3.0 in groups (0.17 of it their plan).
+static int plan_bounce_groups(bart_ctx *ctx, const RadarDev &rd, const BandArgs &bt, int64_t total,
+                              cudaStream_t s, BounceGroups &gr, int &launches)
+{
+    const int64_t keys = bounce_group_keys();
+    if (ctx->db_keys.ensure((size_t)(2 * total), "rate group keys") != BART_OK ||
+        ctx->db_perm.ensure((size_t)(2 * total), "rate group order") != BART_OK ||
+        ctx->db_sort.ensure((size_t)radix_sort_temp_words(total), "rate group sort") != BART_OK ||
+        ctx->db_gcnt.ensure((size_t)(2 * keys), "rate group counts") != BART_OK ||
+        ctx->db_group.ensure((size_t)std::min(total, keys), "rate groups") != BART_OK ||
+        ctx->db_gtot.ensure(5, "rate group totals") != BART_OK) {
+        g_err.clear();
+        return BART_OK;
+    }
+    launch_bounce_groups(ctx->db_vf.p, total, ctx->db_rows.p + total * bounce_geo_bytes(), rd, bt.sh,
+                         ctx->db_keys.p, ctx->db_perm.p, ctx->db_keys.p + total,
+                         ctx->db_perm.p + total, ctx->db_sort.p, ctx->db_gcnt.p, ctx->db_group.p,
+                         ctx->db_gtot.p, s);
+    launches += 8;
+    int64_t tot[5];
+    CUDA_TRY(cudaMemcpyAsync(tot, ctx->db_gtot.p, sizeof tot, cudaMemcpyDeviceToHost, s),
+             "rate group totals copy");
+    CUDA_TRY(cudaStreamSynchronize(s), "cudaStreamSynchronize");
+    const int64_t groups = tot[0];
+    if (5 * (tot[4] + groups * rd.N) > 4 * total * rd.N ||
+        rd.M * (tot[2] * 16 + tot[3] * 8) > ((int64_t)8 << 30) || tot[1] > ((int64_t)1 << 31))
+        return BART_OK;
+    if (ctx->db_part.ensure((size_t)(tot[2] * rd.M), "rate group partial sums") != BART_OK ||
+        ctx->db_node.ensure((size_t)(tot[3] * rd.M), "rate group nodes") != BART_OK ||
+        ctx->db_gref.ensure((size_t)(groups * rd.N), "rate group references") != BART_OK) {
+        g_err.clear();
+        return BART_OK;
+    }
+    gr.group = ctx->db_group.p;
+    gr.perm = ctx->db_perm.p;
+    gr.nodes = bt.nodes;
+    gr.wn = bt.wn;
+    gr.node = ctx->db_node.p;
+    gr.ref = ctx->db_gref.p;
+    gr.groups = (int)groups;
+    gr.items = tot[1];
+    return BART_OK;
+}
+
 static int run_frame(bart_ctx *ctx, double t0, int32_t path, void *adc, int32_t dtype,
                      bart_stats *stats)
 {
@@ -1097,6 +1153,7 @@ static int run_frame(bart_ctx *ctx, double t0, int32_t path, void *adc, int32_t 
                                ctx->vcnt.p, s);
             launches += 1;
         }
+        BounceGroups db_groups{};
         // 3b. double-bounce virtual facets, in two passes, each a count, a
         // scan, a host read of the total (frame graphs are off with double
         // bounce), an allocation and a fill: the candidates (a, b) of each
@@ -1149,14 +1206,16 @@ static int run_frame(bart_ctx *ctx, double t0, int32_t path, void *adc, int32_t 
                     BART_TRY(ctx->db_rows.ensure((size_t)(total * (bounce_row_bytes(rd) +
                                                                    bounce_geo_bytes())),
                                                  "double-bounce rows"));
-                    const int nch = bounce_synth_chunks(rd);
-                    if (nch > 1)
-                        BART_TRY(ctx->db_part.ensure((size_t)nch * O * rd.N * rd.M,
-                                                     "double-bounce partial sums"));
                     launch_bounce_rows(ctx->db_vf.p, total, ctx->fac.p, ctx->vel64.p, rd,
                                        ctx->db_rows.p + total * bounce_geo_bytes(),
                                        ctx->db_rows.p, s);
                     launches += 1;
+                    if (band && bounce_groups_apply(rd, bt.sh))
+                        BART_TRY(plan_bounce_groups(ctx, rd, bt, total, s, db_groups, launches));
+                    const int nch = bounce_synth_chunks(rd);
+                    if (!db_groups.group && nch > 1)
+                        BART_TRY(ctx->db_part.ensure((size_t)nch * O * rd.N * rd.M,
+                                                     "double-bounce partial sums"));
                 }
             }
             launch_bounce_tx_offsets(ctx->db_off.p, ctx->db_blk.p + tw - 1, ctx->db_poff.p,
@@ -1244,9 +1303,11 @@ static int run_frame(bart_ctx *ctx, double t0, int32_t path, void *adc, int32_t 
                                 dtype == BART_C64, path != BART_PATH_FP64,
                                 ctx->db_rows.p + ctx->db_n * bounce_geo_bytes(), ctx->db_rows.p,
                                 path != BART_PATH_FP64 ? bounce_synth_chunks(rd) : 1,
-                                ctx->db_part.p, ctx->counters.p + 4, s);
+                                ctx->db_part.p, db_groups.group ? &db_groups : nullptr,
+                                ctx->counters.p + 4, s);
             if (tm) CUDA_TRY(cudaEventRecord(ctx->ev_db[3], s), "cudaEventRecord");
-            launches += (path != BART_PATH_FP64 && bounce_synth_chunks(rd) > 1) ? 2 : 1;
+            launches += db_groups.group ? 3
+                        : (path != BART_PATH_FP64 && bounce_synth_chunks(rd) > 1) ? 2 : 1;
         }
         ctx->timed_bounce = tm && bounce;
         if (tm) CUDA_TRY(cudaEventRecord(ctx->ev[4], s), "cudaEventRecord");
