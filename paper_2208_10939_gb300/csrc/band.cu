@@ -204,7 +204,7 @@ band_table_kernel(BandShape sh, BandChol ch, float *__restrict__ nodes, float *_
 __global__ void band_plan_kernel(BandArgs b, RadarDev rd, MixConsts K, const float *__restrict__ vel32)
 {
     const int i = blockIdx.x;
-    const BandBounds q = band_bounds(b.box, i, rd, K, vel32);
+    const BandBounds q = band_bounds(b.box, i, i, rd, K, vel32);
     if (threadIdx.x != 0) return;
     BandPlan pl;
     for (int r = 0; r < 3; ++r) pl.c[r] = q.c[r];

@@ -136,14 +136,78 @@ __global__ void __launch_bounds__(256) band64_table_kernel(Band64Shape sh, doubl
     }
 }
 
+// Cells of an instance of nf facets: each at least 256, since a cell's
+// interpolation costs about as much as the direct sum of one lit facet in it.
+// A 5k-facet car on 12 channels of 32 x 256: a frame of 2.74 ms with one cell,
+// 1.89 with four, and no less with eight (sums 1.52 and 1.46, interpolation 0.13
+// and 0.21).
+__device__ __forceinline__ int band64_cells(const Band64Args &b, int64_t nf)
+{
+    int n = 1;
+    while (2 * n <= b.cells && nf >= 512 * (int64_t)n) n *= 2;
+    return n;
+}
+
+// each facet's cell (by its centroid, the box halved along its longest sides)
+// and the cells' boxes
+__global__ void __launch_bounds__(128)
+band64_cell_kernel(Band64Args b, const FacetRec *__restrict__ fac, int64_t F)
+{
+    const int64_t k = (int64_t)blockIdx.x * 128 + threadIdx.x;
+    int body = -1;
+    unsigned int bx[7] = {0u, 0u, 0u, 0u, 0u, 0u, 0u};
+    if (k < F) {
+        const FacetRec f = fac[k];
+        const int n = band64_cells(b, b.ioff[f.inst + 1] - b.ioff[f.inst]);
+        float lo[3], h[3];
+        int cut[3] = {1, 1, 1}, at = 0;
+        for (int r = 0; r < 3; ++r) {
+            lo[r] = ord_f(~b.box[8 * f.inst + r]);
+            h[r] = ord_f(b.box[8 * f.inst + 3 + r]) - lo[r];
+        }
+        for (int m = 1; m < n; m *= 2) {
+            int r = 0;
+            for (int q = 1; q < 3; ++q)
+                if (h[q] * cut[r] > h[r] * cut[q]) r = q;
+            cut[r] *= 2;
+        }
+        for (int r = 0; r < 3; ++r) {
+            const float x = h[r] > 0.f ? (f.c[r] - lo[r]) / h[r] * (float)cut[r] : 0.f;
+            at = at * cut[r] + min(cut[r] - 1, max(0, (int)x));
+        }
+        body = f.inst * b.cells + at;
+        b.cell[k] = (uint8_t)at;
+        float rad2 = 0.f;
+        for (int r = 0; r < 3; ++r) {
+            const float a0 = f.dv[r], a1 = f.dv[3 + r], a2 = f.dv[6 + r];
+            const float pad = 1e-6f * fabsf(f.c[r]);            // the FP32 centroid's rounding
+            bx[r] = ~ord_u(f.c[r] + fminf(fminf(a0, a1), a2) - pad);
+            bx[3 + r] = ord_u(f.c[r] + fmaxf(fmaxf(a0, a1), a2) + pad);
+        }
+        for (int v = 0; v < 3; ++v)
+            rad2 = fmaxf(rad2, f.dv[3 * v] * f.dv[3 * v] + f.dv[3 * v + 1] * f.dv[3 * v + 1] +
+                                   f.dv[3 * v + 2] * f.dv[3 * v + 2]);
+        bx[6] = ord_u(rad2);
+    }
+    const int b0 = __shfl_sync(0xffffffffu, body, 0);
+    if (__all_sync(0xffffffffu, body == b0)) {
+        for (int r = 0; r < 7; ++r) {
+            const unsigned int m = __reduce_max_sync(0xffffffffu, bx[r]);
+            if ((threadIdx.x & 31) == 0 && b0 >= 0) atomicMax(b.cbox + 8 * (int64_t)b0 + r, m);
+        }
+    } else if (body >= 0) {
+        for (int r = 0; r < 7; ++r) atomicMax(b.cbox + 8 * (int64_t)body + r, bx[r]);
+    }
+}
+
 // -------------------------------------------------------------------------
 // plan and reference phases
 // -------------------------------------------------------------------------
 __global__ void band64_plan_kernel(Band64Args b, RadarDev rd, MixConsts K,
                                    const float *__restrict__ vel32, const FacetRec *__restrict__ fac)
 {
-    const int i = blockIdx.x;
-    const BandBounds q = band_bounds(b.box, i, rd, K, vel32);
+    const int body = blockIdx.x, i = body / b.cells;
+    const BandBounds q = band_bounds(b.cells > 1 ? b.cbox : b.box, body, i, rd, K, vel32);
     if (threadIdx.x != 0) return;
     Band64Plan pl;
     for (int r = 0; r < 3; ++r) pl.c[r] = q.c[r];
@@ -162,7 +226,7 @@ __global__ void band64_plan_kernel(Band64Args b, RadarDev rd, MixConsts K,
         for (int l = 2; l < b.sh.n_n && pl.in == 0; ++l)
             if (q.turn <= b.sh.an[l]) pl.in = l;
     }
-    b.plan[i] = pl;
+    b.plan[body] = pl;
 }
 
 __device__ __forceinline__ double two_sum(double a, double b, double &e)
@@ -231,7 +295,7 @@ band64_ref_kernel(Band64Args b, RadarDev rd, const double *__restrict__ vel64)
     if (pl.rotate) {
         const int p = o / rd.Q, q = o % rd.Q;
         const double n = node ? b.xn[b.sh.xn[pl.in] + k] : (double)k;
-        r = band64_ref(rd, pl.c, vel64 + 3 * i, p, q, chirp_start(rd, n, p));
+        r = band64_ref(rd, pl.c, vel64 + 3 * (i / b.cells), p, q, chirp_start(rd, n, p));
     }
     (node ? b.refn : b.ref)[(int64_t)v * N + k] = r;
 }
@@ -245,7 +309,7 @@ __global__ void band64_lists_kernel(Band64Args b, const int32_t *__restrict__ vi
     const int lane = threadIdx.x & 31;
     const int v = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (v >= b.I * b.O) return;
-    const int i = v / b.O, o = v % b.O;
+    const int i = v / b.O, o = v % b.O;          // one cell an instance
     const int32_t *list = vis_idx + (int64_t)o * F;
     const int lo = warp_lower_bound(list, vis_cnt[o], b.ioff[i], lane);
     const int n = warp_lower_bound(list + lo, vis_cnt[o] - lo, b.ioff[i + 1], lane);
@@ -255,20 +319,78 @@ __global__ void band64_lists_kernel(Band64Args b, const int32_t *__restrict__ vi
     }
 }
 
+// the same with cells: a block per (instance, channel) puts its part of the
+// list in cell order, each cell's facets in theirs
+__global__ void __launch_bounds__(256)
+band64_cell_lists_kernel(Band64Args b, const int32_t *__restrict__ vis_idx,
+                         const int32_t *__restrict__ vis_cnt, int64_t F)
+{
+    __shared__ int s_lo, s_n, s_cnt[kB64Cells], s_w[8][kB64Cells], s_run[kB64Cells];
+    const int i = blockIdx.x / b.O, o = blockIdx.x % b.O;
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int32_t *list = vis_idx + (int64_t)o * F;
+    if (warp == 0) {
+        const int lo = warp_lower_bound(list, vis_cnt[o], b.ioff[i], lane);
+        const int n = warp_lower_bound(list + lo, vis_cnt[o] - lo, b.ioff[i + 1], lane);
+        if (lane == 0) {
+            s_lo = lo;
+            s_n = n;
+        }
+    }
+    if (t < kB64Cells) s_cnt[t] = 0;
+    __syncthreads();
+    const int lo = s_lo, n = s_n;
+    for (int e = t; e < n; e += 256) atomicAdd(&s_cnt[b.cell[list[lo + e]]], 1);
+    __syncthreads();
+    if (t == 0) {
+        int at = lo;
+        for (int c = 0; c < kB64Cells; ++c) {
+            const int v = (i * b.cells + c) * b.O + o;
+            b.vstart[v] = s_run[c] = at;
+            b.vcnt[v] = s_cnt[c];
+            at += s_cnt[c];
+        }
+    }
+    __syncthreads();
+    int32_t *out = b.list + (int64_t)o * F;
+    for (int e0 = 0; e0 < n; e0 += 256) {
+        const int e = e0 + t;
+        const int32_t k = e < n ? list[lo + e] : 0;
+        const int c = e < n ? (int)b.cell[k] : -1;
+        int rank = 0;
+        for (int q = 0; q < kB64Cells; ++q) {
+            const unsigned int m = __ballot_sync(0xffffffffu, c == q);
+            if (c == q) rank = __popc(m & ((1u << lane) - 1u));
+            if (lane == 0) s_w[warp][q] = __popc(m);
+        }
+        __syncthreads();
+        if (c >= 0) {
+            int at = s_run[c] + rank;
+            for (int w = 0; w < warp; ++w) at += s_w[w][c];
+            out[at] = k;
+        }
+        __syncthreads();
+        if (t < kB64Cells)
+            for (int w = 0; w < 8; ++w) s_run[t] += s_w[w][t];
+        __syncthreads();
+    }
+}
+
 constexpr int kSeg = 64;             // nodes of a work item
 
 // parts of an (instance, channel)'s facets, by its own list and layout alone:
 // the sums do not depend on what else is in the call
-__device__ __forceinline__ int band64_chunks(const Band64Shape &sh, const Band64Plan &pl, int cnt)
+__device__ __forceinline__ int band64_chunks(const Band64Args &b, const Band64Plan &pl, int cnt)
 {
-    const int64_t room = (int64_t)kB64Room * sh.N * sh.M / ((int64_t)sh.kn[pl.in] * sh.km[pl.im]);
+    const Band64Shape &sh = b.sh;
+    const int64_t room = (int64_t)b.room * sh.N * sh.M / ((int64_t)sh.kn[pl.in] * sh.km[pl.im]);
     return (int)max((int64_t)1, min(room, (int64_t)min(kB64Chunks, (cnt + 127) / 128)));
 }
 
-__device__ __forceinline__ int band64_item_count(const Band64Shape &sh, const Band64Plan &pl, int cnt)
+__device__ __forceinline__ int band64_item_count(const Band64Args &b, const Band64Plan &pl, int cnt)
 {
-    return cnt == 0 ? 0 : sh.kn[pl.in] * ((sh.km[pl.im] + kSeg - 1) / kSeg) *
-                              band64_chunks(sh, pl, cnt);
+    return cnt == 0 ? 0 : b.sh.kn[pl.in] * ((b.sh.km[pl.im] + kSeg - 1) / kSeg) *
+                              band64_chunks(b, pl, cnt);
 }
 
 // the adjoint's items: a chirp node and kAdjFacets facets each
@@ -295,7 +417,7 @@ __global__ void __launch_bounds__(1024) band64_items_kernel(Band64Args b, int ad
         const int v = v0 + t;
         const int items = v >= V ? 0
                           : adjoint ? band64_adjoint_count(b.sh, b.plan[v / b.O], b.vcnt[v])
-                                    : band64_item_count(b.sh, b.plan[v / b.O], b.vcnt[v]);
+                                    : band64_item_count(b, b.plan[v / b.O], b.vcnt[v]);
         int x = items;
         for (int off = 1; off < 32; off <<= 1) {
             const int u = __shfl_up_sync(0xffffffffu, x, off);
@@ -500,7 +622,7 @@ synth_band64_kernel(SynthArgs A, Band64Args b)
         const int i = v / b.O, o = v % b.O, cnt = b.vcnt[v];
         const Band64Plan pl = b.plan[i];
         const int nj = b.sh.kn[pl.in], Km = b.sh.km[pl.im], segs = (Km + kSeg - 1) / kSeg;
-        const int C = band64_chunks(b.sh, pl, cnt);
+        const int C = band64_chunks(b, pl, cnt);
         int at = s_item - b.item0[v];
         const int chunk = at % C;
         at /= C;
@@ -515,7 +637,7 @@ synth_band64_kernel(SynthArgs A, Band64Args b)
         const Node64 n0 = band64_node(rd, xm[s0], ref);
         const Node64 n1 = band64_node(rd, xm[two ? s0 + 32 : s0], ref);
         double re0 = 0.0, im0 = 0.0, re1 = 0.0, im1 = 0.0;
-        const int32_t *list = A.vis_idx + (int64_t)o * A.F + b.vstart[v];
+        const int32_t *list = (b.cells > 1 ? b.list : A.vis_idx) + (int64_t)o * A.F + b.vstart[v];
         const int part = chunk * kB64Warps + warp;
         const int beg = (int)((int64_t)cnt * part / (C * kB64Warps));
         const int end = (int)((int64_t)cnt * (part + 1) / (C * kB64Warps));
@@ -543,7 +665,7 @@ synth_band64_kernel(SynthArgs A, Band64Args b)
                 re1 += s_sum[k][lane + 32].x;
                 im1 += s_sum[k][lane + 32].y;
             }
-            double2 *out = b.coarse + (int64_t)v * kB64Room * b.sh.N * b.sh.M +
+            double2 *out = b.coarse + (int64_t)v * b.room * b.sh.N * b.sh.M +
                            ((int64_t)chunk * nj + j) * Km;
             out[s0] = make_double2(re0, im0);
             if (two) out[s0 + 32] = make_double2(re1, im1);
@@ -557,10 +679,10 @@ __global__ void __launch_bounds__(256) band64_reduce_kernel(Band64Args b)
     const int v = blockIdx.x, cnt = b.vcnt[v];
     if (cnt == 0) return;
     const Band64Plan pl = b.plan[v / b.O];
-    const int C = band64_chunks(b.sh, pl, cnt);
+    const int C = band64_chunks(b, pl, cnt);
     if (C == 1) return;
     const int n = b.sh.kn[pl.in] * b.sh.km[pl.im];
-    double2 *x = b.coarse + (int64_t)v * kB64Room * b.sh.N * b.sh.M;
+    double2 *x = b.coarse + (int64_t)v * b.room * b.sh.N * b.sh.M;
     for (int e = blockIdx.y * 256 + threadIdx.x; e < n; e += gridDim.y * 256) {
         double2 a = x[e];
         for (int k = 1; k < C; ++k) {
@@ -594,12 +716,12 @@ band64_expand_kernel(Band64Args b, RadarDev rd, void *__restrict__ out, int out_
     double2 acc[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) acc[k] = make_double2(0.0, 0.0);
-    for (int i = b.scene_inst[scene]; i < b.scene_inst[scene + 1]; ++i) {
+    for (int i = b.scene_inst[scene] * b.cells; i < b.scene_inst[scene + 1] * b.cells; ++i) {
         const int v = i * b.O + o;
         if (b.vcnt[v] == 0) continue;
         const Band64Plan pl = b.plan[i];
         const int nj = b.sh.kn[pl.in], Km = b.sh.km[pl.im];
-        const double2 *x = b.coarse + (int64_t)v * kB64Room * N * M;
+        const double2 *x = b.coarse + (int64_t)v * b.room * N * M;
         // rows: the chirp nodes, or (every chirp kept) the block's chirps
         const int j0 = pl.in == 0 ? n0 : 0, rows = pl.in == 0 ? min(kExpN, N - n0) : nj;
         __syncthreads();
@@ -709,12 +831,12 @@ band64_gather_kernel(Band64Args b, RadarDev rd, const void *__restrict__ grad, i
     const int mm = threadIdx.x & (kExpM - 1), nn = threadIdx.x / kExpM;
     const int m = blockIdx.x * kExpM + mm;
     int scene = 0;
-    while (b.scene_inst[scene + 1] <= i) ++scene;
+    while (b.scene_inst[scene + 1] * b.cells <= i) ++scene;
     const double fm = rd.f0 + rd.slope * (double)m / rd.fs, km = 2.0 * kPi * fm / kC0;
     const double sc = 2.0 * sqrt(kPi) / pow(4.0 * kPi, 1.5) / (km * km);
     const double tau = (m - 0.5 * (rd.M - 1)) / rd.fs;
     const int64_t row = ((int64_t)scene * b.O + o) * N;
-    double2 *Y = b.coarse + (int64_t)v * kB64Room * N * M;
+    double2 *Y = b.coarse + (int64_t)v * b.room * N * M;
     const auto h_at = [&](int n) -> double2 {
         double2 g;
         if (grad_c64) {
@@ -769,8 +891,8 @@ __global__ void __launch_bounds__(128) band64_gather_samples_kernel(Band64Args b
     if (b.vcnt[v] == 0) return;
     const Band64Plan pl = b.plan[v / b.O];
     const int M = b.sh.M, nj = b.sh.kn[pl.in], Km = b.sh.km[pl.im];
-    const double2 *Y = b.coarse + (int64_t)v * kB64Room * b.sh.N * M;
-    double2 *H = b.coarse + ((int64_t)v * kB64Room + 1) * b.sh.N * M;
+    const double2 *Y = b.coarse + (int64_t)v * b.room * b.sh.N * M;
+    double2 *H = b.coarse + ((int64_t)v * b.room + 1) * b.sh.N * M;
     for (int e = blockIdx.x * 128 + threadIdx.x; e < nj * Km; e += gridDim.x * 128) {
         const int j = e / Km, s = e - j * Km;
         const double2 *y = Y + (int64_t)j * M;
@@ -974,8 +1096,8 @@ adjoint_band64_kernel(SynthArgs A, Band64Args b, double *__restrict__ gfac)
         const double tn = chirp_start(rd, b.xn[b.sh.xn[pl.in] + j], tx);
         const double *ptx = rd.ant[tx], *prx = rd.ant[rd.P + rx];
         const double4 ref = b.refn[(int64_t)v * b.sh.N + j];
-        const double2 *H = b.coarse + ((int64_t)v * kB64Room + 1) * b.sh.N * b.sh.M + (int64_t)j * Km;
-        const int64_t k = valid ? A.vis_idx[(int64_t)o * A.F + b.vstart[v] + e] : 0;
+        const double2 *H = b.coarse + ((int64_t)v * b.room + 1) * b.sh.N * b.sh.M + (int64_t)j * Km;
+        const int64_t k = valid ? (b.cells > 1 ? b.list : A.vis_idx)[(int64_t)o * A.F + b.vstart[v] + e] : 0;
         int kind = -1, flags = 0, quartic = 0;
         if (valid) {
             Rec64 R;
@@ -1143,15 +1265,28 @@ void launch_band64_tables(const Band64Args &b, cudaStream_t s)
 void launch_band64_plan(const Band64Args &b, const SynthArgs &a, cudaStream_t s)
 {
     const MixConsts K = mix_consts(a.rd);
+    if (b.cells > 1) {
+        cudaMemsetAsync(b.cbox, 0, (size_t)b.I * 8 * sizeof(unsigned int), s);
+        band64_cell_kernel<<<(unsigned int)((a.F + 127) / 128), 128, 0, s>>>(b, a.fac, a.F);
+    }
     band64_plan_kernel<<<b.I, 32, 0, s>>>(b, a.rd, K, a.vel32, a.fac);
     const dim3 g((unsigned int)((2 * b.sh.N + 127) / 128), (unsigned int)(b.I * b.O));
     band64_ref_kernel<<<g, 128, 0, s>>>(b, a.rd, a.vel64);
 }
 
+static void launch_lists(const Band64Args &b, const SynthArgs &a, cudaStream_t s)
+{
+    const int V = b.I * b.O;
+    if (b.cells > 1)
+        band64_cell_lists_kernel<<<V / b.cells, 256, 0, s>>>(b, a.vis_idx, a.vis_cnt, a.F);
+    else
+        band64_lists_kernel<<<(V + 3) / 4, 128, 0, s>>>(b, a.vis_idx, a.vis_cnt, a.F);
+}
+
 void launch_synth_band64(const Band64Args &b, const SynthArgs &a, cudaStream_t s)
 {
     const int V = b.I * b.O;
-    band64_lists_kernel<<<(V + 3) / 4, 128, 0, s>>>(b, a.vis_idx, a.vis_cnt, a.F);
+    launch_lists(b, a, s);
     band64_items_kernel<<<1, 1024, 0, s>>>(b, 0);
     int dev = 0, sms = 0, per_sm = 0;
     cudaGetDevice(&dev);
@@ -1169,7 +1304,7 @@ void launch_adjoint_band64(const Band64Args &b, const SynthArgs &a, const void *
 {
     const int V = b.I * b.O;
     cudaMemsetAsync(gfac, 0, (size_t)a.F * 10 * sizeof(double), s);
-    band64_lists_kernel<<<(V + 3) / 4, 128, 0, s>>>(b, a.vis_idx, a.vis_cnt, a.F);
+    launch_lists(b, a, s);
     band64_items_kernel<<<1, 1024, 0, s>>>(b, 1);
     band64_gather_kernel<<<dim3((unsigned int)(b.sh.M / kExpM), (unsigned int)V), 256, 0, s>>>(
         b, a.rd, grad, grad_c64);

@@ -9,13 +9,16 @@
 // 1e4 cycles in FP64: 1e-11 radians).  The reference is a quadratic in fast
 // time whose constant is formed in double-double, so that its rounding, which
 // the whole instance shares, stays below a facet's.
+// An instance of many facets is cut into cells of its box first, each a
+// rigid body of its own: half the extent needs half the nodes (see
+// band64_cells).
 //
 // The direct sum is bound by the FP64 pipe (a 64th of the FP32 rate, 86 % busy):
 // its time goes with the samples it evaluates.  So it is with the adjoint, whose
 // facet sums over samples become sums over nodes once the cube's gradient has
 // gone through the interpolation's transpose (a 1.5k-facet car, 8 channels of 32
-// x 128: 7.95 ms, now 0.84 and 0.06 for the transpose).  A 5k-facet car on 12 channels
-// of 32 x 256 needs 12 x 64 of them and takes 2.7 ms against 33.1.
+// x 128: 7.95 ms, now 0.45 and 0.07 for the transpose).  A 5k-facet car on 12 channels
+// of 32 x 256 takes 1.9 ms against 33.1.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -28,6 +31,7 @@ namespace bart {
 constexpr int kB64N = 16;           // chirp layouts, at most
 constexpr int kB64M = 18;           // sample layouts, at most
 constexpr int kB64MaxNodes = 128;   // chirp nodes of a layout that is not every chirp
+constexpr int kB64Cells = 4;         // cells of an instance, at most
 constexpr int kB64Chunks = 16;      // partial sums of a node, at most
 
 // Layout 0 keeps every chirp / sample; chirp layout 1 is static (one chirp).
@@ -39,7 +43,7 @@ struct Band64Shape {
     int64_t wn[kB64N], wm[kB64M];   // first weight in the tables
 };
 
-struct Band64Plan {                 // per instance
+struct Band64Plan {                 // per body
     int in, im, rotate;
     float c[3];
 };
@@ -49,18 +53,22 @@ struct Band64Args {
     const double *xn, *xm;          // node positions (chirps, samples)
     const double *wn, *wm;          // weights [N][kn], [km][M]
     const double2 *turn;            // [256] exp(j 2 pi i / 256)
-    int I, B, O;
-    const unsigned int *box;        // [I][8] (see launch_build_facets)
+    int I, B, O;                    // bodies: instances x cells
+    int cells;                      // kB64Cells or 1
+    int room;                       // partial sums' room of a body and channel, in cubes
+    const unsigned int *box;        // [instances][8] (see launch_build_facets)
     const int32_t *scene_inst;      // [B + 1]
-    const int64_t *ioff;            // [I + 1]
+    const int64_t *ioff;            // [instances + 1]
+    uint8_t *cell;                  // [F] cell of each facet (cells > 1)
+    unsigned int *cbox;             // [I][8] the cells' boxes
+    int32_t *list;                  // [O][F] the lists in cell order
     Band64Plan *plan;
     double4 *ref, *refn;            // [I O][N] phase quadratics at the chirps, at the nodes
     int32_t *vstart, *vcnt;         // [I O] list parts
     int32_t *item0;                 // [I O + 1]
     int *ticket;
-    double2 *coarse;                // [I O][kB64Room N M] partial node sums
+    double2 *coarse;                // [I O][room N M] partial node sums
 };
-constexpr int kB64Room = 4;         // partial sums' room, in cubes
 
 void band64_shape(int N, int M, Band64Shape &sh);
 struct Band64Sizes {

@@ -9,6 +9,12 @@
 
 namespace bart {
 
+// floats as unsigned integers of the same order, and back
+__device__ __forceinline__ unsigned int ord_u(float f)
+{
+    const unsigned int u = __float_as_uint(f);
+    return (u & 0x80000000u) ? ~u : u | 0x80000000u;
+}
 __device__ __forceinline__ float ord_f(unsigned int u)
 {
     return __uint_as_float((u & 0x80000000u) ? (u & 0x7fffffffu) : ~u);
@@ -38,19 +44,20 @@ struct BandBounds {
     bool ok;         // the bounds hold
 };
 
-// by one warp, a lane per antenna; the result in lane 0
-__device__ __forceinline__ BandBounds band_bounds(const unsigned int *__restrict__ box, int i,
+// of box bi, moving with instance i, by one warp, a lane per antenna; the
+// result in lane 0
+__device__ __forceinline__ BandBounds band_bounds(const unsigned int *__restrict__ box, int bi, int i,
                                                   const RadarDev &rd, const MixConsts &K,
                                                   const float *__restrict__ vel32)
 {
     const int a = threadIdx.x & 31;
     float c[3], h[3];
     for (int r = 0; r < 3; ++r) {
-        const float lo = ord_f(~box[8 * i + r]), hi = ord_f(box[8 * i + 3 + r]);
+        const float lo = ord_f(~box[8 * bi + r]), hi = ord_f(box[8 * bi + 3 + r]);
         c[r] = 0.5f * (lo + hi);
         h[r] = fmaxf(hi - c[r], c[r] - lo);
     }
-    const float rf = sqrtf(ord_f(box[8 * i + 6]));          // largest facet radius
+    const float rf = sqrtf(ord_f(box[8 * bi + 6]));          // largest facet radius
     const float v[3] = {vel32[4 * i], vel32[4 * i + 1], vel32[4 * i + 2]};
     const float speed = sqrtf(v[0] * v[0] + v[1] * v[1] + v[2] * v[2]);
     const float diag = sqrtf(h[0] * h[0] + h[1] * h[1] + h[2] * h[2]);

@@ -691,11 +691,11 @@ static bool use_band(const bart_ctx *ctx, const RadarDev &rd, int32_t path, int6
 
 // The FP64 path's two evaluations: band-limited (band64.cuh) unless the delay
 // form is not the facet's own, the frame is longer than its tables go, or its
-// scratch (kB64Room cubes an instance) would exceed 16 GB.  However small the
+// scratch (four cubes an instance) would exceed 16 GB.  However small the
 // instances, interpolating one costs about what the direct sum spends on one
 // lit facet (100 FP64 operations a sample), so their size is no condition, and
 // a scene gives the same bits alone and in a batch.  A 5k-facet car on 12
-// channels of 32 x 256: 33.1 ms by the direct sum, 2.7 ms band-limited.
+// channels of 32 x 256: 33.1 ms by the direct sum, 1.9 ms band-limited.
 static bool use_band64(const RadarDev &rd, int I)
 {
     return !rd.far_field && !rd.delay_ref && rd.N <= 1024 && (int64_t)I * rd.O <= 65535 &&
@@ -1008,8 +1008,13 @@ static int run_frame(bart_ctx *ctx, double t0, int32_t path, void *adc, int32_t 
     bool band64 = (path == BART_PATH_FP64 || path == kPathAdjoint) && use_band64(rd, I);
     Band64Args b64{};
     if (band64) {
-        const int64_t V = (int64_t)I * O;
-        if (ctx->band64_coarse.ensure((size_t)(V * kB64Room * rd.N * rd.M),
+        // bodies: the instances, or their cells where the scratch stays within 16 GB
+        b64.cells = (int64_t)I * O * kB64Cells <= 65535 &&
+                            (int64_t)I * O * rd.N * rd.M <= ((int64_t)1 << 27)
+                        ? kB64Cells : 1;
+        b64.room = b64.cells > 1 ? 2 : 4;
+        const int64_t V = (int64_t)I * b64.cells * O;
+        if (ctx->band64_coarse.ensure((size_t)(V * b64.room * rd.N * rd.M),
                                       "band coarse samples") != BART_OK) {
             g_err.clear();
             band64 = false;
@@ -1027,7 +1032,7 @@ static int run_frame(bart_ctx *ctx, double t0, int32_t path, void *adc, int32_t 
             }
             b64.sh = ctx->band64_sh;
             band64_tables(ctx->band64_tab.p, b64);
-            b64.I = I;
+            b64.I = I * b64.cells;
             b64.B = B;
             b64.O = O;
             b64.box = ctx->box.p;
@@ -1043,11 +1048,16 @@ static int run_frame(bart_ctx *ctx, double t0, int32_t path, void *adc, int32_t 
                 };
                 take(b64.ref, V * rd.N);
                 take(b64.refn, V * rd.N);
-                take(b64.plan, I);
+                take(b64.plan, b64.I);
                 take(b64.vstart, V);
                 take(b64.vcnt, V);
                 take(b64.item0, V + 1);
                 take(b64.ticket, 1);
+                if (b64.cells > 1) {
+                    take(b64.list, (int64_t)O * F);
+                    take(b64.cbox, 8 * (int64_t)b64.I);
+                    take(b64.cell, F);
+                }
                 return n;
             };
             BART_TRY(ctx->band64_ws.ensure(carve(nullptr), "band plans and items"));
@@ -1270,7 +1280,7 @@ static int run_frame(bart_ctx *ctx, double t0, int32_t path, void *adc, int32_t 
             if (path == kPathAdjoint && band64) {
                 launch_band64_plan(b64, a, s);
                 launch_adjoint_band64(b64, a, ctx->adj_grad, ctx->adj_grad_c64, ctx->gfac.p, s);
-                launches += 6;
+                launches += 6 + (b64.cells > 1);
             } else if (path == kPathAdjoint)
                 launch_adjoint_fp64(a, ctx->adj_grad, ctx->adj_grad_c64, ctx->gfac.p, s);
             else
@@ -1288,7 +1298,7 @@ static int run_frame(bart_ctx *ctx, double t0, int32_t path, void *adc, int32_t 
                 launch_band64_plan(b64, a, s);
                 launch_synth_band64(b64, a, s);
                 if (stats) launch_count_records64(a, s);
-                launches += stats ? 8 : 7;
+                launches += 7 + (b64.cells > 1) + (stats ? 1 : 0);
             } else {
                 launch_synth_fp64(a, s);
                 launches += fp64_chunks > 1 ? 2 : 1;
