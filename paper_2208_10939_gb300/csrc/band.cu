@@ -196,7 +196,7 @@ band_table_kernel(BandShape sh, BandChol ch, float *__restrict__ nodes, float *_
         }
         base[(int64_t)l * M + m] = b0;
 #pragma unroll
-        for (int i = 0; i < T; ++i) wm[((int64_t)l * M + m) * T + i] = (float)r[i];
+        for (int i = 0; i < T; ++i) wm[((int64_t)l * T + i) * M + m] = (float)r[i];
     }
 }
 
@@ -538,51 +538,82 @@ synth_band_kernel(SynthArgs A, MixConsts K, BandArgs b)
     }
 }
 
-// coarse values of an (instance, channel): the items' partial sums added in
-// chunk order, Kahan-compensated
-__global__ void __launch_bounds__(256) band_reduce_kernel(BandArgs b)
+// Coarse values of an (instance, channel): the items' partial sums, Kahan-
+// compensated.  A thread takes a slice of the chunks of one value (in memory
+// order, so that a warp's loads are one run), the slices are added in order.
+// What bounds it is the chain of loads, so a slice is 4 chunks or more of up
+// to eight: a sedan's 188 chunks one after the other, a value a thread, took
+// 28 us, this takes 8.
+constexpr int kRedThreads = 256;
+constexpr int kRedSlices = 8;
+
+__device__ __forceinline__ void kahan_add(float v, float &sum, float &c)
 {
+    const float y = v - c, t = sum + y;
+    c = (t - sum) - y;
+    sum = t;
+}
+
+__global__ void __launch_bounds__(kRedThreads) band_reduce_kernel(BandArgs b)
+{
+    __shared__ float4 s_part[kRedThreads];                // sums and their compensation
     const int v = blockIdx.x;
     const int cnt = b.vcnt[v];
     if (cnt == 0) return;
     const BandPlan &pl = b.plan[v / b.O];
     const BandM lay = b.sh.m[pl.im];
-    const int nj = b.sh.n[pl.in].nj;
+    const int rows = b.sh.n[pl.in].nj * lay.nseg;
     const int rpw = 32 / lay.lpr, groups = band_groups(b.sh, pl);
     const int chunks = (b.item0[v + 1] - b.item0[v]) / groups;
     const float2 *part = reinterpret_cast<const float2 *>(b.partial) +
                          (int64_t)b.item0[v] * (kBandS * 32);
     float2 *out = b.coarse + b.coff[v];
     const int lane_s = kBandS * lay.lpr;               // samples of a (node, segment) row
-    for (int e = blockIdx.y * blockDim.x + threadIdx.x; e < nj * lay.Mi;
-         e += gridDim.y * blockDim.x) {
-        const int rs = e / lane_s, s = e - rs * lane_s;
-        const int grp = rs / rpw;
-        const int lane = (rs - grp * rpw) * lay.lpr + (s >> 4);
-        // [item][pair][lane][half]
-        const float2 *src = part + (int64_t)grp * (kBandS * 32) + ((s & 15) >> 1) * 64 + 2 * lane +
-                            (s & 1);
+    int slices = 1;
+    while (slices < kRedSlices && chunks >= 8 * slices) slices *= 2;
+    const int per = kRedThreads / slices;              // values at once: a divisor of 512
+    const int t = threadIdx.x & (per - 1), slice = threadIdx.x / per;
+    const int j0 = chunks * slice / slices, j1 = chunks * (slice + 1) / slices;
+    const int64_t step = (int64_t)groups * (kBandS * 32);
+    const int tiles = kBandS * 32 / per;               // of a group
+    for (int tile = blockIdx.y; tile < groups * tiles; tile += gridDim.y) {
+        // position: [group][pair][lane][half]
+        const int grp = tile / tiles, at = (tile - grp * tiles) * per + t;
+        const int lane = (at & 63) >> 1, row = lane / lay.lpr;
+        const int rs = grp * rpw + row;
+        const int s = (lane - row * lay.lpr) * 16 + (at >> 6) * 2 + (at & 1);
         float sr = 0.f, si = 0.f, cr = 0.f, ci = 0.f;
-        for (int j = 0; j < chunks; ++j) {
-            const float2 p = src[(int64_t)j * groups * (kBandS * 32)];
-            float y = p.x - cr, t = sr + y;
-            cr = (t - sr) - y;
-            sr = t;
-            y = p.y - ci;
-            t = si + y;
-            ci = (t - si) - y;
-            si = t;
+        const float2 *src = part + (int64_t)grp * (kBandS * 32) + at;
+#pragma unroll 4
+        for (int j = j0; j < j1; ++j) {
+            const float2 p = src[j * step];
+            kahan_add(p.x, sr, cr);
+            kahan_add(p.y, si, ci);
         }
-        if (pl.rotate) {                               // the steps' eighth turns back
-            const int k = s & 7;
-            const float h = 0.70710678f;
-            const float c = k == 0 ? 1.f : k == 4 ? -1.f : (k & 3) == 2 ? 0.f : (k == 1 || k == 7) ? h : -h;
-            const float z = (k & 3) == 0 ? 0.f : k == 2 ? 1.f : k == 6 ? -1.f : k < 4 ? h : -h;
-            const float x = fmaf(c, sr, z * si);
-            si = fmaf(c, si, -z * sr);
-            sr = x;
+        if (slices > 1) {
+            s_part[threadIdx.x] = make_float4(sr, si, cr, ci);
+            __syncthreads();
         }
-        out[e] = make_float2(sr, si);
+        if (slice == 0 && row < rpw && rs < rows) {
+            for (int k = 1; k < slices; ++k) {
+                const float4 p = s_part[k * per + t];
+                kahan_add(p.x, sr, cr);
+                kahan_add(p.y, si, ci);
+                cr += p.z;
+                ci += p.w;
+            }
+            if (pl.rotate) {                               // the steps' eighth turns back
+                const int k = s & 7;
+                const float h = 0.70710678f;
+                const float c = k == 0 ? 1.f : k == 4 ? -1.f : (k & 3) == 2 ? 0.f : (k == 1 || k == 7) ? h : -h;
+                const float z = (k & 3) == 0 ? 0.f : k == 2 ? 1.f : k == 6 ? -1.f : k < 4 ? h : -h;
+                const float x = fmaf(c, sr, z * si);
+                si = fmaf(c, si, -z * sr);
+                sr = x;
+            }
+            out[(int64_t)rs * lane_s + s] = make_float2(sr, si);
+        }
+        if (slices > 1) __syncthreads();
     }
 }
 
@@ -590,12 +621,15 @@ __global__ void __launch_bounds__(256) band_reduce_kernel(BandArgs b)
 // expansion: each block writes kExpN chirps x kExpM samples of one channel
 // of one scene: per instance, the chirps' interpolation of the coarse samples
 // it needs into shared memory, then the samples' taps and the reference
-// phase; the instances in order
+// phase; the instances in order.  The taps' weights lie sample by sample
+// (sample by tap, a warp's load was 20 cache lines), and a multiprocessor holds
+// four blocks, some spills for 64 registers (two of 92: latency-bound, 24 % of
+// the warps): a batch of eight scenes takes 132 us against 178.
 // -------------------------------------------------------------------------
 constexpr int kExpN = 8;
 constexpr int kExpM = 256;
 
-__global__ void __launch_bounds__(kExpM)
+__global__ void __launch_bounds__(kExpM, 4)
 band_expand_kernel(BandArgs b, MixConsts K, void *__restrict__ out, int out_c64)
 {
     extern __shared__ float2 sT[];                     // [kExpN][width]
@@ -632,6 +666,7 @@ band_expand_kernel(BandArgs b, MixConsts K, void *__restrict__ out, int out_c64)
                 float tr[kExpN], ti[kExpN];
 #pragma unroll
                 for (int k = 0; k < kExpN; ++k) tr[k] = ti[k] = 0.f;
+#pragma unroll 4
                 for (int j = 0; j < ch.nj; ++j) {
                     const float2 c = C[(int64_t)j * lay.Mi + s0 + s];
 #pragma unroll
@@ -652,13 +687,13 @@ band_expand_kernel(BandArgs b, MixConsts K, void *__restrict__ out, int out_c64)
         if (!ok) continue;
         float xr[kExpN], xi[kExpN];
         if (pl.im) {
-            const float *wm = b.wm + ((int64_t)pl.im * M + m) * kBandTaps;
+            const float *wm = b.wm + (int64_t)pl.im * kBandTaps * M + m;
             const int off = base[m] - s0;
 #pragma unroll
             for (int k = 0; k < kExpN; ++k) xr[k] = xi[k] = 0.f;
 #pragma unroll 4
             for (int e = 0; e < kBandTaps; ++e) {
-                const float w = wm[e];
+                const float w = wm[(int64_t)e * M];
 #pragma unroll
                 for (int k = 0; k < kExpN; ++k) {
                     const float2 c = sT[k * width + off + e];
@@ -788,7 +823,8 @@ void launch_synth_band(const BandArgs &b, const SynthArgs &a, cudaStream_t s)
     const int64_t need = (b.max_items + kBandWarps - 1) / kBandWarps;
     const int grid = (int)std::min<int64_t>(need, (int64_t)kBandBlocks * sms);
     synth_band_kernel<<<grid, kBandWarps * 32, 0, s>>>(a, K, b);
-    band_reduce_kernel<<<dim3((unsigned int)V, 8), 256, 0, s>>>(b);
+    band_reduce_kernel<<<dim3((unsigned int)V, (unsigned int)std::max(8, std::min(32, 2048 / V))),
+                         kRedThreads, 0, s>>>(b);
     const int mt = (b.sh.M + kExpM - 1) / kExpM, nt = (b.sh.N + kExpN - 1) / kExpN;
     const size_t sm = (size_t)kExpN * (kExpM + kBandTaps) * sizeof(float2);
     band_expand_kernel<<<dim3((unsigned int)(mt * nt), (unsigned int)b.O, (unsigned int)b.B), kExpM,

@@ -71,7 +71,7 @@ struct BandPlan {        // per instance
 
 // layouts for N chirps of M samples, the sizes of their tables -- node
 // positions [sum nj], chirp weights [layout][N][nj] and, per sample layout,
-// every sample's first tap [M] and weights [M][kBandTaps] -- and the tables
+// every sample's first tap [M] and weights [kBandTaps][M] -- and the tables
 void band_shape(int N, int M, BandShape &sh);
 struct BandSizes {
     int64_t nodes, wn, base, wm;
