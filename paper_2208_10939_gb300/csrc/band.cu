@@ -91,8 +91,10 @@ int64_t band_max_items(const BandShape &sh, int64_t V, int target, int64_t lit_m
         groups = std::max<int64_t>(groups, ((int64_t)sh.N * sh.m[l].nseg + rpw - 1) / rpw);
     }
     // ceil(count / chunk) chunks per group: one each, and the target spread
-    // over them (a fixed chunk: the whole list's chunks)
-    const int64_t more = fixed_chunk > 0 ? groups * (lit_max / fixed_chunk + 1) : target;
+    // over them, a chunk at least 32 facets (a fixed chunk: the whole list's
+    // chunks)
+    const int64_t more = fixed_chunk > 0 ? groups * (lit_max / fixed_chunk + 1)
+                                         : std::min<int64_t>(target, groups * (lit_max / 32 + 1));
     return V * groups + more;
 }
 
@@ -122,13 +124,16 @@ __device__ __host__ __forceinline__ double band_sinc(double x)
 #endif
 }
 
-__global__ void __launch_bounds__(128)
+// one warp a block: the FP64 work spread over the multiprocessors
+constexpr int kTabRows = 32;         // blocks of a layout
+
+__global__ void __launch_bounds__(32)
 band_table_kernel(BandShape sh, BandChol ch, float *__restrict__ nodes, float *__restrict__ wn,
                   int *__restrict__ base, float *__restrict__ wm)
 {
     constexpr int T = kBandTaps;
     const int N = sh.N, M = sh.M, tid = threadIdx.x;
-    __shared__ double x[128], w[128];
+    __shared__ double x[128], w[128], r[T][32];
     if ((int)blockIdx.x < sh.n_n) {
         const int l = blockIdx.x;
         const BandN lay = sh.n[l];
@@ -145,14 +150,17 @@ band_table_kernel(BandShape sh, BandChol ch, float *__restrict__ nodes, float *_
         }
         __syncthreads();
         for (int j = tid; j < K; j += blockDim.x) {
-            double p = 1.0;
-            for (int i = 0; i < K; ++i)
-                if (i != j) p *= (x[j] - x[i]) * (4.0 / (N - 1));
-            w[j] = 1.0 / p;
+            double p[4] = {1.0, 1.0, 1.0, 1.0};                // four chains of products
+            const double xj = x[j], sc = 4.0 / (N - 1);
+            for (int i = 0; i < K; i += 4)
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    if (i + q != j && i + q < K) p[q] *= (xj - x[i + q]) * sc;
+            w[j] = 1.0 / ((p[0] * p[1]) * (p[2] * p[3]));
         }
         __syncthreads();
-        const int lane = tid & 31, warps = blockDim.x >> 5;
-        for (int n = blockIdx.y * warps + (tid >> 5); n < N; n += gridDim.y * warps) {
+        const int lane = tid;
+        for (int n = blockIdx.y; n < N; n += kTabRows) {
             double sum = 0.0;
             int hit = -1;
             for (int j = lane; j < K; j += 32) {
@@ -179,24 +187,39 @@ band_table_kernel(BandShape sh, BandChol ch, float *__restrict__ nodes, float *_
         const double pos = ((double)m + lay.off) / lay.d;
         const int b0 = max(0, min(lay.Mi - T, (int)floor(pos) - T / 2 + 1));
         const double w2 = 1.0 / kBandOver;                // twice the band edge
-        double r[T];
-#pragma unroll
+        // sines of the taps' arguments by turns of w2 (their spacing), then both
+        // triangular solves column by column: the updates of a step are
+        // independent, where row by row each waited for the last.  Rolled, in
+        // shared memory: the table is made once a frame size, so that unrolled
+        // code comes from memory (55 us a table, now 43)
+        double sn, cs, ds, dc;
+        sincospi(w2 * (b0 - pos), &sn, &cs);
+        sincospi(w2, &ds, &dc);
+#pragma unroll 1
         for (int i = 0; i < T; ++i) {
-            double a = w2 * band_sinc(w2 * (b0 + i - pos));
-#pragma unroll
-            for (int k = 0; k < i; ++k) a -= ch.L[i * (i + 1) / 2 + k] * r[k];
-            r[i] = a * ch.L[i * (i + 1) / 2 + i];          // the diagonal is stored inverted
+            const double x = w2 * (b0 + i - pos);
+            r[i][tid] = x == 0.0 ? w2 : w2 * sn / (kPi * x);
+            const double c2 = cs * dc - sn * ds;
+            sn = sn * dc + cs * ds;
+            cs = c2;
         }
-#pragma unroll
-        for (int i = T - 1; i >= 0; --i) {
-            double a = r[i];
-#pragma unroll
-            for (int k = i + 1; k < T; ++k) a -= ch.L[k * (k + 1) / 2 + i] * r[k];
-            r[i] = a * ch.L[i * (i + 1) / 2 + i];
+#pragma unroll 1
+        for (int k = 0; k < T; ++k) {
+            const double v = r[k][tid] * ch.L[k * (k + 1) / 2 + k];   // the diagonal is stored inverted
+            r[k][tid] = v;
+#pragma unroll 4
+            for (int i = k + 1; i < T; ++i) r[i][tid] -= ch.L[i * (i + 1) / 2 + k] * v;
+        }
+#pragma unroll 1
+        for (int k = T - 1; k >= 0; --k) {
+            const double v = r[k][tid] * ch.L[k * (k + 1) / 2 + k];
+            r[k][tid] = v;
+#pragma unroll 4
+            for (int i = 0; i < k; ++i) r[i][tid] -= ch.L[k * (k + 1) / 2 + i] * v;
         }
         base[(int64_t)l * M + m] = b0;
-#pragma unroll
-        for (int i = 0; i < T; ++i) wm[((int64_t)l * T + i) * M + m] = (float)r[i];
+#pragma unroll 4
+        for (int i = 0; i < T; ++i) wm[((int64_t)l * T + i) * M + m] = (float)r[i][tid];
     }
 }
 
@@ -798,8 +821,8 @@ void launch_band_tables(const BandShape &sh, float *nodes, float *wn, int *base,
             }
         return c;
     }();
-    band_table_kernel<<<dim3((unsigned int)(sh.n_n + sh.n_m), 8), 128, 0, s>>>(sh, chol, nodes, wn,
-                                                                               base, wm);
+    band_table_kernel<<<dim3((unsigned int)(sh.n_n + sh.n_m), kTabRows), 32, 0, s>>>(sh, chol, nodes,
+                                                                                    wn, base, wm);
 }
 
 void launch_band_plan(const BandArgs &b, const SynthArgs &a, cudaStream_t s)
