@@ -50,8 +50,13 @@ BOUNCE = ("moving sedan 20k tris on a 20 m x 20 m static ground (0.5 m cells, 32
 # algorithmic work of one echo term in the mixed path: 3 vertex phases, 3 unit
 # phasors, 3 real x complex weighted accumulates and their compensation, about
 # 24 FP32 FMA-pipe operations (plus 6 SFU operations when the phasors come from
-# sincos); the roofline counts operations of the FMA pipe, whatever their kind
+# sincos); the roofline counts operations of the FMA pipe, whatever their kind.
+# A term is one of the direct sum: the band-limited evaluation (16 samples a
+# lane, the default) evaluates a fraction of them and interpolates, so that its
+# rate in these operations is an equivalent and no share of a peak
 OPS_PER_TERM = 24
+BAND_NOTE = ("band-limited: direct-sum operations per second of the synthesis stage; the kernel "
+             "evaluates the nodes of each instance only, so this is no fraction of the peak")
 # DRAM traffic of one synthesis launch and the FMA-pipe activity, from ncu
 # captures of the synthesis kernel on 4 TX x 4 RX cuts of the frame.  A work
 # item takes one record chunk of a channel through all its chirps, so a
@@ -59,15 +64,18 @@ OPS_PER_TERM = 24
 # other chirps: reads grow with those pairs (terms / (N M)), not with the
 # terms (16 and 64 chirps read 3.41 and 3.28 GB); the items' partial sums
 # grow with the (channel, chirp) rows.  Valid only while the kernel's sources
-# hash to the value they had at the capture.
+# hash to the value they had at the capture (the direct kernel's; the
+# band-limited evaluation has no such capture).
 SYNTH_PROFILE = {"sources_sha256_16": "4239e3318de9d32c", "samples_per_lane": 16,
                  "dram_read_bytes_per_channel_facet": 3.277169152e9 / (4 * 50804670464 / (64 * 512)),
                  "dram_write_bytes_per_row": 75.109632e6 / (16 * 64),
                  "fma_pipe_active": 0.686}
 SYNTH_SOURCES = ("synth.cu", "bart_internal.cuh", "record_fp64.cuh", "mixed_record.cuh")
 # the double-bounce synthesis: 3 centres x (2 accumulates + 4 rotation
-# operations) per vertex-form term; ncu figures of its launch on the
-# sedan-over-ground frame, valid while its sources hash as at the capture
+# operations) per vertex-form term of the direct evaluation, which the rate
+# groups (bounce.cuh) replace by their nodes where they apply; ncu figures of the
+# direct launch on the sedan-over-ground frame, valid while its sources hash as
+# at the capture
 BOUNCE_OPS_PER_TERM = 18
 BOUNCE_SOURCES = ("bounce.cu", "bounce.cuh", "geom64.cuh", "record_fp64.cuh", "bart_internal.cuh")
 BOUNCE_PROFILE = {"sources_sha256_16": "0ad733dd979e3494", "fma_pipe_active": 0.324, "fp64_pipe_active": 0.528,
@@ -701,7 +709,11 @@ def sedan_lines(pkg, sg, torch, dev, args, peaks) -> dict:
                                         "synthesis_ms", "rdm_ms")}}
         if peaks:
             ach = terms * OPS_PER_TERM / (synth_avg / 1e3) / 1e12
-            out["roofline_frac_of_measured_fp32"] = ach / peaks["fp32_fma_pipe_tops"]
+            if layout_samples(r.M, 0 if tune is None else tune["best"][0]) == 16:
+                out["direct_sum_equivalent_tops"] = ach
+                out["direct_sum_equivalent_note"] = BAND_NOTE
+            else:
+                out["roofline_frac_of_measured_fp32"] = ach / peaks["fp32_fma_pipe_tops"]
         # plain FP64 path on the same frame (the parity reference path)
         adc64 = torch.empty((r.O, r.N, r.M), dtype=torch.complex128, device=dev)
         if args.fp64_steps > 0:
@@ -765,14 +777,15 @@ def double_bounce_lines(pkg, sg, torch, dev, args, peaks) -> dict:
                     prof = (BOUNCE_PROFILE if BOUNCE_PROFILE["sources_sha256_16"] ==
                             synth_sources_hash(BOUNCE_SOURCES) else None)
                     out["roofline"] = {
-                        "bound": "alu", "kernel": "bounce_synth_f32_kernel<8>",
+                        "bound": "alu", "kernel": "bounce_synth_f32_kernel<8, true>",
                         "ops_per_term": BOUNCE_OPS_PER_TERM, "achieved": ach,
-                        "peak": peaks["fp32_fma_pipe_tops"], "frac": ach / peaks["fp32_fma_pipe_tops"],
+                        "peak": peaks["fp32_fma_pipe_tops"], "frac": None,
                         "unit": "Top/s (FP32 FMA-pipe operations)",
                         "peak_basis": "measured (bart_measure_peaks)",
                         "ncu": prof,
-                        "note": "per-record work (FP64 rows and phases, per-lane start "
-                                "phasors) is amortised over 8 samples per lane"}
+                        "note": "direct-sum operations per second: virtual facets are "
+                                "evaluated at the chirp nodes of their rate groups only, so "
+                                "this is no fraction of the peak"}
                 out.update({
                     "facets": st["n_facets"], "virtual_facets": st["n_bounce_facets"],
                     "double_bounce_terms_per_frame": bt,
@@ -931,16 +944,19 @@ def main():
     synth_avg_ms = statistics.mean(tf["synth_ms"]) / synth_launches
     achieved = terms / synth_launches * OPS_PER_TERM / (synth_avg_ms / 1e3) / 1e12
     S_used = layout_samples(M, 0 if layout is None else layout["samples_per_lane"])
-    prof = synth_profile(S_used)
+    band = S_used == 16
+    prof = None if band else synth_profile(S_used)
     if peaks:
         peak, peak_basis = peaks["fp32_fma_pipe_tops"], (
             "measured: FP32 FMA-pipe operations/s of this GPU (bart_measure_peaks, the faster "
             "of scalar and packed f32x2 FMA chains)")
     else:
         peak, peak_basis = 152 * 128 * 2.070e9 / 1e12, "nominal: 152 SM x 128 lanes x 2070 MHz"
-    roofline = {"bound": "alu", "kernel": f"synth_mixed_kernel<{S_used}, *>",
+    roofline = {"bound": "alu",
+                "kernel": "synth_band_kernel" if band else f"synth_mixed_kernel<{S_used}, *>",
                 "achieved": achieved, "peak": peak, "unit": "Top/s (FP32 FMA-pipe operations)",
-                "frac": achieved / peak,
+                "frac": None if band else achieved / peak,
+                "note": BAND_NOTE if band else None,
                 "traffic": None if prof is None
                 else (prof["dram_read_bytes_per_channel_facet"] * terms / (N * M)
                       + prof["dram_write_bytes_per_row"] * O * N) / synth_launches,

@@ -333,6 +333,11 @@ int bart_simulate_frame(bart_ctx *ctx, double t0, int32_t path, void *adc,
 int bart_add_noise(bart_ctx *ctx, void *adc, int32_t dtype, double snr_db, uint64_t seed,
                    uint32_t frame);
 
+/* The mixed-path frame with every chirp and sample evaluated: the forward
+ * that bart_simulate_adjoint_mixed differentiates (bart_simulate_frame's mixed
+ * path interpolates between nodes).  As bart_simulate_frame otherwise. */
+int bart_simulate_mixed_direct(bart_ctx *ctx, double t0, void *adc, int32_t dtype);
+
 /* Adjoint of the plain FP64 echo synthesis (the differentiable echo).  For
  * a real loss L of the ADC cube of the frame at t0, given
  * grad_adc = dL/dRe(adc) + i dL/dIm(adc) (device, the layout

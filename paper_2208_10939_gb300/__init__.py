@@ -37,7 +37,7 @@ EXPORTED = ["bart_last_error", "bart_version", "bart_create", "bart_destroy",
             "bart_sync", "bart_form_rdm_static", "bart_add_noise", "bart_detect",
             "bart_scene_partition", "bart_set_graph", "bart_set_synth_layout",
             "bart_autotune", "bart_rdm_adjoint", "bart_simulate_adjoint",
-            "bart_simulate_adjoint_mixed",
+            "bart_simulate_adjoint_mixed", "bart_simulate_mixed_direct",
             "bart_mesh_update", "bart_measure_peaks", "bart_inject_alloc_failure",
             "bart_selftest_wait_timeout", "bart_get_bounce_facets", "bart_get_dims",
             "bart_mesh_dims", "bart_get_bvh"]
@@ -179,6 +179,7 @@ def load_library() -> ctypes.CDLL:
         L.bart_mesh_dims.argtypes = [P, I32, ctypes.POINTER(I64), ctypes.POINTER(I64)]
         L.bart_radar_set.argtypes = [P, ctypes.POINTER(bart_radar)]
         L.bart_simulate_frame.argtypes = [P, D, I32, P, I32, ctypes.POINTER(bart_stats)]
+        L.bart_simulate_mixed_direct.argtypes = [P, D, P, I32]
         L.bart_form_rdm.argtypes = [P, P, I32, P]
         L.bart_frame_host.argtypes = [P, D, I32, P, ctypes.POINTER(bart_stats)]
         L.bart_get_visibility.argtypes = [P, P, ctypes.POINTER(I64)]
@@ -420,6 +421,15 @@ def bart_simulate_frame(ctx: int, t0: float, path: int, adc, stats: bool = False
         ctx, float(t0), int(path), ctypes.c_void_p(_ptr(adc)), _dtype_code(adc),
         ctypes.byref(st) if st is not None else None))
     return st.as_dict() if st is not None else None
+
+
+def bart_simulate_mixed_direct(ctx: int, t0: float, adc) -> None:
+    """The mixed-path frame at every chirp and sample, the forward of
+    ``bart_simulate_adjoint(..., mixed=True)``, into ``adc`` ([O][N][M])."""
+    d = _dims(ctx)
+    _device_buffer(adc, "adc", d, _cube(d))
+    _check(load_library().bart_simulate_mixed_direct(ctx, float(t0), ctypes.c_void_p(_ptr(adc)),
+                                                     _dtype_code(adc)))
 
 
 def bart_form_rdm(ctx: int, adc, rdm) -> None:

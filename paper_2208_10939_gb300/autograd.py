@@ -15,16 +15,16 @@ from typing import List
 
 import torch
 
-from . import (PATH_FP64, PATH_MIXED, Simulator, bart_form_rdm, bart_mesh_update,
-               bart_rdm_adjoint, bart_simulate_adjoint, bart_simulate_frame)
+from . import (PATH_FP64, Simulator, bart_form_rdm, bart_mesh_update, bart_rdm_adjoint,
+               bart_simulate_adjoint, bart_simulate_frame, bart_simulate_mixed_direct)
 
 
 class EchoScene:
     """A scene whose every instance has its own mesh, so that the instance
     vertices are the mesh vertices (the differentiable parameters).
 
-    ``precision="mixed"`` runs the mixed-path forward (complex64 cube) and
-    the adjoint with FP32 per-sample work (``bart_simulate_adjoint_mixed``);
+    ``precision="mixed"`` runs the mixed-path forward at every chirp and sample
+    (complex64 cube) and the adjoint with FP32 per-sample work (``bart_simulate_adjoint_mixed``);
     the default ``"fp64"`` runs both in FP64."""
 
     def __init__(self, sim: Simulator, scene, precision: str = "fp64"):
@@ -63,7 +63,10 @@ class _Echo(torch.autograd.Function):
         adc = torch.empty(scene.sim.adc_shape(),
                           dtype=torch.complex64 if mixed else torch.complex128,
                           device=verts.device)
-        bart_simulate_frame(scene.sim.ctx, scene.t0, PATH_MIXED if mixed else PATH_FP64, adc)
+        if mixed:
+            bart_simulate_mixed_direct(scene.sim.ctx, scene.t0, adc)
+        else:
+            bart_simulate_frame(scene.sim.ctx, scene.t0, PATH_FP64, adc)
         ctx.scene = scene
         ctx.has_rho = rho is not None
         ctx.shapes = (verts.shape, None if rho is None else rho.shape)

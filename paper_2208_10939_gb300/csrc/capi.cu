@@ -670,6 +670,12 @@ int bart_radar_set(bart_ctx *ctx, const bart_radar *r)
 // with its vertex-form per-sample work in FP32 (bart_simulate_adjoint_mixed)
 constexpr int kPathAdjoint = 100;
 constexpr int kPathAdjointMixed = 101;
+// the mixed path at every chirp and sample (bart_simulate_mixed_direct): the
+// forward of the mixed adjoint, which goes through them too.  Its rounding is
+// what the adjoint's gradients of weakly reflecting facets depend on.
+constexpr int kPathMixedDirect = 102;
+// a caller's path: not that one
+static int32_t public_path(int32_t path) { return path == kPathMixedDirect ? -1 : path; }
 
 // The mixed path's two evaluations: band-limited (band.cuh) unless
 //  - another lane layout than 16 samples was asked for,
@@ -763,6 +769,8 @@ static int plan_bounce_groups(bart_ctx *ctx, const RadarDev &rd, const BandArgs 
 static int run_frame(bart_ctx *ctx, double t0, int32_t path, void *adc, int32_t dtype,
                      bart_stats *stats)
 {
+    const bool direct = path == kPathMixedDirect;
+    if (direct) path = BART_PATH_MIXED;
     if (!ctx->have_radar) return fail(BART_ESTATE, "bart_simulate_frame: radar not set");
     if (ctx->insts.empty()) return fail(BART_ESTATE, "bart_simulate_frame: scene has no instances");
     if (path != BART_PATH_FP64 && path != BART_PATH_MIXED && path != BART_PATH_SPECTRAL &&
@@ -905,7 +913,8 @@ static int run_frame(bart_ctx *ctx, double t0, int32_t path, void *adc, int32_t 
                         ? ctx->tpi_override
                         : synth_tiles_per_item(*std::max_element(scene_F.begin(), scene_F.end()));
     int64_t max_items = 0;
-    const bool band = (path == BART_PATH_MIXED || path == BART_PATH_SPECTRAL) && use_band(ctx, rd, path, F, I);
+    const bool band = !direct && (path == BART_PATH_MIXED || path == BART_PATH_SPECTRAL) &&
+                      use_band(ctx, rd, path, F, I);
     BandArgs bt{};
     const bool mixed_rows = path == BART_PATH_MIXED || path == BART_PATH_SPECTRAL ||
                             path == kPathAdjointMixed;
@@ -1333,7 +1342,7 @@ static int run_frame(bart_ctx *ctx, double t0, int32_t path, void *adc, int32_t 
                            path != kPathAdjointMixed && !bounce;
     if (use_graph) {
         bart_ctx::FrameGraph &g = ctx->fg;
-        const bool hit = g.exec && g.version == ctx->version && g.path == path &&
+        const bool hit = g.exec && g.version == ctx->version && g.path == (direct ? kPathMixedDirect : path) &&
                          g.dtype == dtype && g.adc == adc && g.stream == s;
         if (!hit) {
             g.release();
@@ -1378,7 +1387,7 @@ static int run_frame(bart_ctx *ctx, double t0, int32_t path, void *adc, int32_t 
                 return fail(BART_ECUDA, "frame graph: world-facet kernel node not found");
             }
             g.version = ctx->version;
-            g.path = path;
+            g.path = direct ? kPathMixedDirect : path;
             g.dtype = dtype;
             g.adc = adc;
             g.stream = s;
@@ -1440,7 +1449,14 @@ int bart_simulate_frame(bart_ctx *ctx, double t0, int32_t path, void *adc, int32
 {
     g_err.clear();
     if (!ctx) return fail(BART_EINVAL, "bart_simulate_frame: ctx is NULL");
-    return run_frame(ctx, t0, path, adc, dtype, stats);
+    return run_frame(ctx, t0, public_path(path), adc, dtype, stats);
+}
+
+int bart_simulate_mixed_direct(bart_ctx *ctx, double t0, void *adc, int32_t dtype)
+{
+    g_err.clear();
+    if (!ctx) return fail(BART_EINVAL, "bart_simulate_mixed_direct: ctx is NULL");
+    return run_frame(ctx, t0, kPathMixedDirect, adc, dtype, nullptr);
 }
 
 static int run_adjoint(bart_ctx *ctx, double t0, const void *grad_adc, int32_t dtype,
@@ -1785,7 +1801,7 @@ int bart_frame_host(bart_ctx *ctx, double t0, int32_t path, float *rdm_host, bar
     const size_t B = (size_t)ctx->n_scenes;
     BART_TRY(ctx->adc_own.ensure(B * r.P * r.Q * r.N * r.M * esz, "frame adc"));
     BART_TRY(ctx->rdm_own.ensure(B * r.M * r.N, "frame rdm"));
-    BART_TRY(run_frame(ctx, t0, path, ctx->adc_own.p, dtype, stats));
+    BART_TRY(run_frame(ctx, t0, public_path(path), ctx->adc_own.p, dtype, stats));
     BART_TRY(run_rdm(ctx, ctx->adc_own.p, dtype, ctx->rdm_own.p));
     CUDA_TRY(cudaMemcpyAsync(rdm_host, ctx->rdm_own.p, B * r.M * r.N * sizeof(float),
                              cudaMemcpyDeviceToHost, ctx->stream), "rdm copy");
