@@ -344,7 +344,7 @@ __device__ __forceinline__ int band_groups(const BandShape &sh, const BandPlan &
 }
 
 // facets per work item, then the item and coarse-value prefixes (one block)
-__global__ void __launch_bounds__(1024) band_items_kernel(BandArgs b)
+__device__ __forceinline__ void band_items(const BandArgs &b)
 {
     __shared__ long long s_w[32], s_c[32], s_work;
     __shared__ long long s_run, s_crun;
@@ -415,15 +415,16 @@ __global__ void __launch_bounds__(1024) band_items_kernel(BandArgs b)
     if (t == 0) b.item0[V] = (int)s_run;
 }
 
-// a block per (instance, channel): its items, chunk by chunk through the row
-// groups, so that a chunk's facet records come from HBM once
-__global__ void band_fill_kernel(BandArgs b)
+__global__ void __launch_bounds__(1024) band_items_kernel(BandArgs b) { band_items(b); }
+
+// the items of (instance, channel) v, chunk by chunk through the row groups, so
+// that a chunk's facet records come from HBM once; by threads first, first + step, ...
+__device__ __forceinline__ void band_fill(const BandArgs &b, int v, int first, int step)
 {
-    const int v = blockIdx.x;
     const int n = b.item0[v + 1] - b.item0[v];
     const int groups = band_groups(b.sh, b.plan[v / b.O]);
     const int chunk = *b.chunk, cnt = b.vcnt[v];
-    for (int k = threadIdx.x; k < n; k += blockDim.x) {
+    for (int k = first; k < n; k += step) {
         const int j = k / groups;
         BandItem it;
         it.v = v;
@@ -432,6 +433,38 @@ __global__ void band_fill_kernel(BandArgs b)
         it.rend = min(cnt, it.rbeg + chunk);
         b.items[b.item0[v] + k] = it;
     }
+}
+
+__global__ void band_fill_kernel(BandArgs b) 
+{
+    band_fill(b, blockIdx.x, threadIdx.x, blockDim.x);
+}
+
+// All three in one block for up to kBandSmall (instance, channel) pairs: the
+// launches, not their work, are what such a frame spends there (a sedan's 12
+// pairs: 14.5 us in three launches and their gaps, 10.8 in one).
+constexpr int kBandSmall = 48;
+
+__global__ void __launch_bounds__(1024)
+band_small_kernel(BandArgs b, const int32_t *__restrict__ vis_idx,
+                  const int32_t *__restrict__ vis_cnt, int64_t F)
+{
+    __shared__ int s_lim[2 * kBandSmall];
+    const int lane = threadIdx.x & 31, V = b.I * b.O;
+    for (int w = threadIdx.x >> 5; w < 2 * V; w += 32) {
+        const int v = w >> 1, i = v / b.O, o = v % b.O;
+        const int at = warp_lower_bound(vis_idx + (int64_t)o * F, vis_cnt[o], b.ioff[i + (w & 1)], lane);
+        if (lane == 0) s_lim[w] = at;
+    }
+    __syncthreads();
+    if (threadIdx.x < V) {
+        b.vstart[threadIdx.x] = s_lim[2 * threadIdx.x];
+        b.vcnt[threadIdx.x] = s_lim[2 * threadIdx.x + 1] - s_lim[2 * threadIdx.x];
+    }
+    __syncthreads();
+    band_items(b);
+    __syncthreads();
+    for (int v = threadIdx.x >> 5; v < V; v += 32) band_fill(b, v, lane, 32);
 }
 
 // -------------------------------------------------------------------------
@@ -837,9 +870,13 @@ void launch_synth_band(const BandArgs &b, const SynthArgs &a, cudaStream_t s)
 {
     const MixConsts K = mix_consts(a.rd);
     const int V = b.I * b.O;
-    band_lists_kernel<<<(V + 3) / 4, 256, 0, s>>>(b, a.vis_idx, a.vis_cnt, a.F);
-    band_items_kernel<<<1, 1024, 0, s>>>(b);
-    band_fill_kernel<<<V, 64, 0, s>>>(b);
+    if (V <= kBandSmall) {
+        band_small_kernel<<<1, 1024, 0, s>>>(b, a.vis_idx, a.vis_cnt, a.F);
+    } else {
+        band_lists_kernel<<<(V + 3) / 4, 256, 0, s>>>(b, a.vis_idx, a.vis_cnt, a.F);
+        band_items_kernel<<<1, 1024, 0, s>>>(b);
+        band_fill_kernel<<<V, 64, 0, s>>>(b);
+    }
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -853,6 +890,8 @@ void launch_synth_band(const BandArgs &b, const SynthArgs &a, cudaStream_t s)
     band_expand_kernel<<<dim3((unsigned int)(mt * nt), (unsigned int)b.O, (unsigned int)b.B), kExpM,
                          sm, s>>>(b, K, a.out, a.out_c64);
 }
+
+int launch_synth_band_count(const BandArgs &b) { return b.I * b.O <= kBandSmall ? 4 : 6; }
 
 void launch_count_records(const SynthArgs &a, cudaStream_t s)
 {

@@ -115,6 +115,7 @@ int64_t band_max_items(const BandShape &sh, int64_t V, int target, int64_t lit_m
 void launch_band_plan(const BandArgs &b, const SynthArgs &a, cudaStream_t s);
 // after the lists and the kinematics rows: items, coarse sums, expansion
 void launch_synth_band(const BandArgs &b, const SynthArgs &a, cudaStream_t s);
+int launch_synth_band_count(const BandArgs &b);      // its launches
 // per-form record counts of the whole frame (stats)
 void launch_count_records(const SynthArgs &a, cudaStream_t s);
 

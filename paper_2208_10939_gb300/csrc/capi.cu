@@ -1266,7 +1266,7 @@ static int run_frame(bart_ctx *ctx, double t0, int32_t path, void *adc, int32_t 
             }
             if (tm) CUDA_TRY(cudaEventRecord(ctx->ev_syn[1], s), "cudaEventRecord");
             ctx->chunks = 1;
-            launches += band ? (stats ? 8 : 6) : 4;
+            launches += band ? launch_synth_band_count(bt) + (stats ? 2 : 0) : 4;
         } else if (path == BART_PATH_SPECTRAL) {
             a.kin = ctx->kin.p;
             a.kquad = ctx->kquad.p;
