@@ -157,7 +157,7 @@ void launch_visibility(const double *tri64, const float4 *trel, const double *c6
                        int *status, cudaStream_t s);
 // lists 0..O-1: facets lit from both antennas of each channel; O..O+A-1: facets
 // lit from each antenna.  vis_idx is [O+A][F], vis_cnt [O+A].
-void launch_compact(const uint8_t *state, int64_t F, const RadarDev &rd,
+int launch_compact(const uint8_t *state, int64_t F, const RadarDev &rd,
                     int32_t *blk_cnt, int32_t *vis_idx, int32_t *vis_cnt, cudaStream_t s);
 int64_t compact_blk_words(int64_t F, int L);
 // per (scene, channel) sub-ranges of the channel lists: vstart[b O + o] is

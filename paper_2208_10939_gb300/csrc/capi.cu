@@ -1165,8 +1165,7 @@ static int run_frame(bart_ctx *ctx, double t0, int32_t path, void *adc, int32_t 
                           ctx->wide.p,
                           F >= 2 ? ctx->vals.p : nullptr, F, rd, split, ctx->state.p,
                           ctx->counters.p + 3, ctx->status.p, s);
-        launch_compact(ctx->state.p, F, rd, ctx->blk_cnt.p, ctx->vis_idx.p, ctx->vis_cnt.p, s);
-        launches += 1 + 3;
+        launches += 1 + launch_compact(ctx->state.p, F, rd, ctx->blk_cnt.p, ctx->vis_idx.p, ctx->vis_cnt.p, s);
         if (B > 1 && !((band || band64) && !stats)) {
             launch_scene_lists(ctx->vis_idx.p, ctx->vis_cnt.p, F, O, ctx->d_foff.p, B, ctx->vstart.p,
                                ctx->vcnt.p, s);
