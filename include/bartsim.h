@@ -43,7 +43,9 @@ extern "C" {
 #define BART_EDEVICE  (-6)   /* device-side check failed (see bart_last_error) */
 
 /* echo-synthesis precision paths */
-#define BART_PATH_FP64  0    /* every quantity in FP64, exact per-sample delay */
+#define BART_PATH_FP64  0    /* every quantity in FP64, exact delay at every sample or, band-
+                                limited (csrc/band64.cuh), at nodes between which FP64
+                                interpolation is exact to 1e-13 */
 #define BART_PATH_MIXED 1    /* FP64 path length + mod-1 reduction, FP32 phasors,
                                 compensated (Kahan) accumulation */
 #define BART_PATH_SPECTRAL 2 /* the mixed path's records, each chirp row summed by the
