@@ -224,7 +224,8 @@ band_table_kernel(BandShape sh, BandChol ch, float *__restrict__ nodes, float *_
 }
 
 // one warp per instance
-__global__ void band_plan_kernel(BandArgs b, RadarDev rd, MixConsts K, const float *__restrict__ vel32)
+__global__ void band_plan_kernel(BandArgs b, RadarDev rd, MixConsts K, const float *__restrict__ vel32,
+                                 const FacetRec *__restrict__ fac)
 {
     const int i = blockIdx.x;
     const BandBounds q = band_bounds(b.box, i, i, rd, K, vel32);
@@ -242,9 +243,12 @@ __global__ void band_plan_kernel(BandArgs b, RadarDev rd, MixConsts K, const flo
                 break;
             }
         }
+    // a facet lit from both sides has a kink where its obliquity changes sign
+    // (interpolated: 1 to 4 % off on a plate that passes edge-on): every chirp is kept
+    const bool smooth = b.ioff[i] < b.ioff[i + 1] && !fac[b.ioff[i]].two_sided;
     if (q.speed == 0.f) {
         pl.in = 1;
-    } else if (q.ok) {
+    } else if (q.ok && smooth) {
         for (int l = 2; l < b.sh.n_n; ++l)
             if (q.turn <= b.sh.n[l].amax) {
                 pl.in = l;
@@ -861,7 +865,7 @@ void launch_band_tables(const BandShape &sh, float *nodes, float *wn, int *base,
 void launch_band_plan(const BandArgs &b, const SynthArgs &a, cudaStream_t s)
 {
     const MixConsts K = mix_consts(a.rd);
-    band_plan_kernel<<<b.I, 32, 0, s>>>(b, a.rd, K, a.vel32);
+    band_plan_kernel<<<b.I, 32, 0, s>>>(b, a.rd, K, a.vel32, a.fac);
     dim3 g((unsigned int)((2 * b.sh.N + 127) / 128), (unsigned int)(b.I * b.O));
     band_ref_kernel<<<g, 128, 0, s>>>(b, a.rd, a.vel64);
 }

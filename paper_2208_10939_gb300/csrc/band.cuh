@@ -18,7 +18,8 @@
 // band |f| <= 0.5 / kBandOver of the grid's rate (at most 2e-6 at the band's
 // edge, 1e-7 rms).  Static instances have one chirp.  An instance whose
 // bounds exceed the tables keeps every chirp and every sample (n_j = n,
-// d = 1), which is the direct sum.
+// d = 1), which is the direct sum; a moving one lit from both sides keeps every
+// chirp, since its facets' obliquity |o| has a kink where they pass edge-on.
 //
 // What it gives: a 20k-facet sedan on 12 channels of 128 x 256 needs 12
 // chirps of 48 samples instead of 128 of 256; its synthesis took 1.19 ms by
