@@ -1354,16 +1354,39 @@ __global__ void bounce_reduce_kernel(const double2 *__restrict__ partial, int64_
 // Rate groups (BounceGroup in bounce.cuh): virtual facets of one TX whose paths
 // lengthen at nearly the same rate.
 // -------------------------------------------------------------------------
-constexpr int kDbRateBins = 2048;            // per TX; the last: rows without expansion
+constexpr int kDbRateBins = 2048;            // per TX; the last: every chirp kept
 constexpr int kDbKeys = kDbMaxTx * kDbRateBins;
 static_assert(kDbKeys <= 65536 && kDbKeys % 1024 == 0, "16-bit keys, a run of them per thread");
 constexpr int kDbChunk = 256;                // virtual facets of a work item
 
+// does the facet's plane keep the point at x + v t on one side over [0, T]: the
+// distance is linear in t, so that its ends decide; fac's normal is rounded,
+// 1e-6 of the distance to the point
+__device__ __forceinline__ bool one_side(const FacetRec &fr, const double *c, const double *vel,
+                                         const double *x, const double *v, double T)
+{
+    double h0 = 0.0, h1 = 0.0, far = 0.0;
+    for (int r = 0; r < 3; ++r) {
+        const double d = x[r] - c[r], e = d + ((v ? v[r] : 0.0) - vel[r]) * T;
+        h0 += d * (double)fr.n[r];
+        h1 += e * (double)fr.n[r];
+        far = fmax(far, fmax(fabs(d), fabs(e)));
+    }
+    const double margin = 1e-5 * far;
+    return h0 > 0.0 ? h0 > margin && h1 > margin : h0 < -margin && h1 < -margin;
+}
+
 // key, and the largest phase turn of the key's facets over half the frame
-// after their group's reference: every vertex's path of every RX
+// after their group's reference: every vertex's path of every RX.  A second
+// facet lit from both sides has a kink where its obliquity changes sign
+// (interpolated: 1 to 3 % off on a plate that passes edge-on): unless the image
+// source and every RX stay on their side of its plane, it goes where every
+// chirp is kept (a 20k-facet car on its road, all two-sided: a frame of 38.8 ms
+// with every such facet there, 9.6 with those that may turn).
 __global__ void __launch_bounds__(128)
 bounce_key_kernel(const BounceFacet *__restrict__ vf, int64_t V, const BounceRow *__restrict__ rows,
-                  RadarDev rd, double h, float width, float kmax, uint32_t *__restrict__ keys,
+                  const FacetRec *__restrict__ fac, const double *__restrict__ vel64, RadarDev rd,
+                  double h, float width, float kmax, uint32_t *__restrict__ keys,
                   int32_t *__restrict__ perm, int32_t *__restrict__ cnt,
                   unsigned int *__restrict__ turn)
 {
@@ -1374,6 +1397,13 @@ bounce_key_kernel(const BounceFacet *__restrict__ vf, int64_t V, const BounceRow
     int bin = kDbRateBins - 1;
     bool ok = isfinite(rate);
     for (int l = 0; l <= rd.Q; ++l) ok = ok && R[l].a[0] >= 0.0;
+    const FacetRec &fr = fac[vf[v].b];
+    if (ok && fr.two_sided) {
+        const double *c = vf[v].tri, *vel = vel64 + 3 * fr.inst;
+        const double T = (double)(rd.N * rd.slots - 1) * rd.Tc;
+        ok = one_side(fr, c, vel, vf[v].src, vf[v].usrc, T);
+        for (int q = 0; q < rd.Q && ok; ++q) ok = one_side(fr, c, vel, rd.ant[rd.P + q], nullptr, T);
+    }
     float a = 3e38f;
     if (ok) {
         bin = (int)fminf(fmaxf(floorf(rate / width) + 1023.f, 0.f), (float)(kDbRateBins - 2));
@@ -1717,10 +1747,11 @@ bool bounce_groups_apply(const RadarDev &rd, const BandShape &sh)
 
 int64_t bounce_group_keys() { return kDbKeys; }
 
-void launch_bounce_groups(const BounceFacet *vf, int64_t V, const void *rows, const RadarDev &rd,
-                          const BandShape &sh, uint32_t *keys, int32_t *perm, uint32_t *keys_tmp,
-                          int32_t *perm_tmp, uint32_t *sort_temp, int32_t *cnt, BounceGroup *group,
-                          int64_t *tot, cudaStream_t s)
+void launch_bounce_groups(const BounceFacet *vf, int64_t V, const void *rows, const FacetRec *fac,
+                          const double *vel64, const RadarDev &rd, const BandShape &sh,
+                          uint32_t *keys, int32_t *perm, uint32_t *keys_tmp, int32_t *perm_tmp,
+                          uint32_t *sort_temp, int32_t *cnt, BounceGroup *group, int64_t *tot,
+                          cudaStream_t s)
 {
     unsigned int *turn = reinterpret_cast<unsigned int *>(cnt) + kDbKeys;
     cudaMemsetAsync(cnt, 0, (size_t)2 * kDbKeys * sizeof(int32_t), s);
@@ -1728,7 +1759,8 @@ void launch_bounce_groups(const BounceFacet *vf, int64_t V, const void *rows, co
     const double kmax = 2.0 * kPi * (rd.f0 + rd.slope * (rd.M - 1) / rd.fs) / kC0;
     const float width = (float)(2.0 * kDbGroupTurn / (kmax * h));
     bounce_key_kernel<<<(unsigned int)((V + 127) / 128), 128, 0, s>>>(
-        vf, V, static_cast<const BounceRow *>(rows), rd, h, width, (float)kmax, keys, perm, cnt, turn);
+        vf, V, static_cast<const BounceRow *>(rows), fac, vel64, rd, h, width, (float)kmax, keys, perm,
+        cnt, turn);
     radix_sort_pairs(keys, perm, keys_tmp, perm_tmp, sort_temp, V, 16, s);
     int S = 16;
     while ((rd.M / 32) % S) S /= 2;

@@ -88,10 +88,11 @@ bool bounce_groups_apply(const RadarDev &rd, const BandShape &sh);
 int64_t bounce_group_keys();
 // groups of the virtual facets from their rows; cnt: 2 x keys words; tot:
 // groups, work items, partial rows, node rows, records per RX
-void launch_bounce_groups(const BounceFacet *vf, int64_t V, const void *rows, const RadarDev &rd,
-                          const BandShape &sh, uint32_t *keys, int32_t *perm, uint32_t *keys_tmp,
-                          int32_t *perm_tmp, uint32_t *sort_temp, int32_t *cnt, BounceGroup *group,
-                          int64_t *tot, cudaStream_t s);
+void launch_bounce_groups(const BounceFacet *vf, int64_t V, const void *rows, const FacetRec *fac,
+                          const double *vel64, const RadarDev &rd, const BandShape &sh,
+                          uint32_t *keys, int32_t *perm, uint32_t *keys_tmp, int32_t *perm_tmp,
+                          uint32_t *sort_temp, int32_t *cnt, BounceGroup *group, int64_t *tot,
+                          cudaStream_t s);
 // adds the double-bounce echo of every channel into the cube, the
 // per-sample work in FP32 (fp32_eval: records from slow-time rows, FP32
 // phasors, the record lists cut into NCH chunks whose partial sums a

@@ -736,10 +736,10 @@ static int plan_bounce_groups(bart_ctx *ctx, const RadarDev &rd, const BandArgs 
         g_err.clear();
         return BART_OK;
     }
-    launch_bounce_groups(ctx->db_vf.p, total, ctx->db_rows.p + total * bounce_geo_bytes(), rd, bt.sh,
-                         ctx->db_keys.p, ctx->db_perm.p, ctx->db_keys.p + total,
-                         ctx->db_perm.p + total, ctx->db_sort.p, ctx->db_gcnt.p, ctx->db_group.p,
-                         ctx->db_gtot.p, s);
+    launch_bounce_groups(ctx->db_vf.p, total, ctx->db_rows.p + total * bounce_geo_bytes(),
+                         ctx->fac.p, ctx->vel64.p, rd, bt.sh, ctx->db_keys.p, ctx->db_perm.p,
+                         ctx->db_keys.p + total, ctx->db_perm.p + total, ctx->db_sort.p,
+                         ctx->db_gcnt.p, ctx->db_group.p, ctx->db_gtot.p, s);
     launches += 8;
     int64_t tot[5];
     CUDA_TRY(cudaMemcpyAsync(tot, ctx->db_gtot.p, sizeof tot, cudaMemcpyDeviceToHost, s),

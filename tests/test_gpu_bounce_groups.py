@@ -48,3 +48,37 @@ def test_groups(sim, M, N, P, Q, tdm, speed):
     err = float((got - ref).norm() / ref.norm())
     print(f"{M} x {N}, {P * Q} channels, {speed} m/s: {err:.2e}")
     assert float(ref.norm()) > 0 and err <= TOL
+
+
+@pytest.mark.parametrize("beside", [False, True])
+@pytest.mark.parametrize("at", [0.15, 0.5, 0.8])
+def test_two_sided_second_facets_edge_on(sim, at, beside):
+    """An upright two-sided plate over the ground that passes the antennas'
+    plane at the fraction `at` of the frame: the second facets' obliquity |o|
+    has a kink there; alone, or beside a weak one-sided plate whose facets are
+    worth grouping.  Cubes in complex128, so that the part's difference
+    takes no rounding from the ground's own echo."""
+    m = sg.plate(0.4, 0.4, 8)
+    m.two_sided = True
+    radar = sg.make_radar(128, 64, 1, 2, 5.12e6, 30e12, 2.0, centre=(0.0, 0.0, 1.5))
+    upright = np.array([[0.0, -1.0, 0.0], [1.0, 0.0, 0.0], [0.0, 0.0, 1.0]])
+    speed, T = 12.0, 63 * radar.Tc
+    sc = sg.Scene([m, sg.ground(6.0, 6, centre=(0.0, 7.0))],
+                  [sg.Instance(0, (-speed * T * at, 10.0, 0.6), upright, (speed, 0.0, 0.0)),
+                   sg.Instance(1, (0.0, 0.0, 0.0), np.eye(3), (0.0, 0.0, 0.0))], radar)
+    if beside:
+        sc.meshes.append(sg.plate(0.6, 0.6, 20, rho=1e-3))
+        sc.instances.append(sg.Instance(2, (1.0, 11.0, 0.6), np.eye(3), (0.0, -9.0, 0.0)))
+
+    def bounce(path):
+        out = []
+        for on in (True, False):
+            sc.radar.double_bounce = on
+            sim.load_scene(sc)
+            out.append(sim.simulate(path, dtype=torch.complex128))
+        return out[0] - out[1]
+
+    got, ref = bounce(pkg.PATH_MIXED), bounce(pkg.PATH_FP64)
+    err = float((got - ref).norm() / ref.norm())
+    print(f"edge-on at {at}: {err:.2e}")
+    assert float(ref.norm()) > 0 and err <= TOL
