@@ -77,7 +77,9 @@ bool injected_alloc_failure()
     return false;
 }
 
+// moves: the owner's count of buffers whose address went stale
 template <typename T> struct DevBuf {
+    uint64_t *moves = nullptr;
     T *p = nullptr;
     size_t cap = 0;
     int ensure(size_t n, const char *what)
@@ -101,6 +103,7 @@ template <typename T> struct DevBuf {
     void release()
     {
         if (p) cudaFree(p);
+        if (p && moves) ++*moves;
         p = nullptr;
         cap = 0;
     }
@@ -122,6 +125,8 @@ int set_last_error(int code, const char *msg) { return fail(code, "%s", msg); }
 }  // namespace bart
 
 struct bart_ctx {
+    uint64_t moves = 0;         // device buffers below that were freed or grew; first, since
+                                // they count themselves here
     int device = 0;
     cudaStream_t stream = nullptr;
     std::vector<MeshStore *> pool;     // reused across bart_mesh_clear
@@ -135,55 +140,55 @@ struct bart_ctx {
     int frame_A = 0;
     int frame_B = 1;            // scenes of the last frame's partition
 
-    DevBuf<MeshDesc> d_meshes;
-    DevBuf<InstDev> d_insts;
-    DevBuf<double> tri64, c64, vel64;
-    DevBuf<float> tri32;                // only with double bounce
-    DevBuf<float4> trel;
-    DevBuf<WideNode> wide;
-    DevBuf<float> vel32, aabb;
-    DevBuf<double> ref64;               // instance origins at t0 (delay reference points)
-    DevBuf<float> ref32;
-    DevBuf<FacetRec> fac;
-    DevBuf<float> fac_lo;
-    DevBuf<unsigned int> bounds;
-    DevBuf<uint32_t> keys, keys_tmp, sort_temp;
-    DevBuf<int32_t> vals, vals_tmp;
-    DevBuf<BvhNode> nodes;
-    DevBuf<float4> levels;              // boxes of runs of the sorted leaves
-    DevBuf<int> ticket;                 // block counter of their kernel, zero between frames
-    DevBuf<uint8_t> state;
-    DevBuf<int32_t> blk_cnt, vis_idx, vis_cnt;
-    DevBuf<float4> kin;                 // kinematics Taylor rows [A][F][9]
-    DevBuf<double> kquad;               // FP64 row data [A][F][kKinQuadWords]
-    DevBuf<float2> partial;             // mixed-path per-item partial sums
-    DevBuf<int32_t> item_off;
-    DevBuf<int> item_counter;
+    DevBuf<MeshDesc> d_meshes{&moves};
+    DevBuf<InstDev> d_insts{&moves};
+    DevBuf<double> tri64{&moves}, c64{&moves}, vel64{&moves};
+    DevBuf<float> tri32{&moves};                // only with double bounce
+    DevBuf<float4> trel{&moves};
+    DevBuf<WideNode> wide{&moves};
+    DevBuf<float> vel32{&moves}, aabb{&moves};
+    DevBuf<double> ref64{&moves};               // instance origins at t0 (delay reference points)
+    DevBuf<float> ref32{&moves};
+    DevBuf<FacetRec> fac{&moves};
+    DevBuf<float> fac_lo{&moves};
+    DevBuf<unsigned int> bounds{&moves};
+    DevBuf<uint32_t> keys{&moves}, keys_tmp{&moves}, sort_temp{&moves};
+    DevBuf<int32_t> vals{&moves}, vals_tmp{&moves};
+    DevBuf<BvhNode> nodes{&moves};
+    DevBuf<float4> levels{&moves};              // boxes of runs of the sorted leaves
+    DevBuf<int> ticket{&moves};                 // block counter of their kernel, zero between frames
+    DevBuf<uint8_t> state{&moves};
+    DevBuf<int32_t> blk_cnt{&moves}, vis_idx{&moves}, vis_cnt{&moves};
+    DevBuf<float4> kin{&moves};                 // kinematics Taylor rows [A][F][9]
+    DevBuf<double> kquad{&moves};               // FP64 row data [A][F][kKinQuadWords]
+    DevBuf<float2> partial{&moves};             // mixed-path per-item partial sums
+    DevBuf<int32_t> item_off{&moves};
+    DevBuf<int> item_counter{&moves};
     // band-limited mixed path (band.cuh): instance boxes, tables of the (N, M)
     // they were made for, plans, references, lists and items
-    DevBuf<unsigned int> box;
-    DevBuf<float> band_tab;
+    DevBuf<unsigned int> box{&moves};
+    DevBuf<float> band_tab{&moves};
     BandShape band_sh{};
-    DevBuf<unsigned char> band_ws;
-    DevBuf<int64_t> d_ioff;             // facet offsets of the instances [I + 1]
-    DevBuf<int32_t> d_sinst;            // first instance of each scene [B + 1]
-    DevBuf<float2> band_coarse;
+    DevBuf<unsigned char> band_ws{&moves};
+    DevBuf<int64_t> d_ioff{&moves};             // facet offsets of the instances [I + 1]
+    DevBuf<int32_t> d_sinst{&moves};            // first instance of each scene [B + 1]
+    DevBuf<float2> band_coarse{&moves};
     // the FP64 path's band-limited evaluation
     Band64Shape band64_sh = {};
-    DevBuf<double> band64_tab;
-    DevBuf<unsigned char> band64_ws;
-    DevBuf<double2> band64_coarse;
-    DevBuf<unsigned long long> counters;   // 0 vertex, 1 series, 2 edge, 3 grazing
-    DevBuf<int> status;
-    DevBuf<unsigned char> rdm_ws, adc_own;
-    DevBuf<double> noise_scratch;
-    DevBuf<float> rdm_own;
-    DevBuf<float> spec_tab;             // spectral path: 1 / kernel transforms [2][M]
+    DevBuf<double> band64_tab{&moves};
+    DevBuf<unsigned char> band64_ws{&moves};
+    DevBuf<double2> band64_coarse{&moves};
+    DevBuf<unsigned long long> counters{&moves};   // 0 vertex, 1 series, 2 edge, 3 grazing
+    DevBuf<int> status{&moves};
+    DevBuf<unsigned char> rdm_ws{&moves}, adc_own{&moves};
+    DevBuf<double> noise_scratch{&moves};
+    DevBuf<float> rdm_own{&moves};
+    DevBuf<float> spec_tab{&moves};             // spectral path: 1 / kernel transforms [2][M]
     int spec_M = 0;
-    DevBuf<unsigned char> det_ws;       // detection: cube, RDM, steering table, lists
-    DevBuf<unsigned char> adj_ws;       // adjoints: RDM cube scratch
-    DevBuf<double> gfac;                // synthesis adjoint: per-facet gradients [F][10]
-    DevBuf<int64_t> d_voff;             // first mesh vertex of each instance (adjoint output)
+    DevBuf<unsigned char> det_ws{&moves};       // detection: cube, RDM, steering table, lists
+    DevBuf<unsigned char> adj_ws{&moves};       // adjoints: RDM cube scratch
+    DevBuf<double> gfac{&moves};                // synthesis adjoint: per-facet gradients [F][10]
+    DevBuf<int64_t> d_voff{&moves};             // first mesh vertex of each instance (adjoint output)
     const void *adj_grad = nullptr;     // the pending adjoint call's arguments
     int adj_grad_c64 = 0;
     double *adj_gverts = nullptr, *adj_grho = nullptr;
@@ -192,28 +197,28 @@ struct bart_ctx {
     // scene_first[b+1]) form scene b; empty = one scene
     std::vector<int32_t> scene_first;
     int n_scenes = 1;
-    DevBuf<int64_t> d_foff;             // facet offsets of the scenes [B + 1]
-    DevBuf<int32_t> d_root;             // BVH root of each scene [B]
-    DevBuf<int32_t> vstart, vcnt;       // per (scene, channel) list ranges [B O]
+    DevBuf<int64_t> d_foff{&moves};             // facet offsets of the scenes [B + 1]
+    DevBuf<int32_t> d_root{&moves};             // BVH root of each scene [B]
+    DevBuf<int32_t> vstart{&moves}, vcnt{&moves};       // per (scene, channel) list ranges [B O]
     // double bounce: pieces per (TX, lit facet) item, their offsets, the scan
     // scratch (its last word the total) and the virtual facets of the frame
-    DevBuf<int32_t> db_cnt;
-    DevBuf<int32_t> db_roots;           // the candidate traversal's subtree roots
-    DevBuf<int64_t> db_off, db_blk;
-    DevBuf<BounceFacet> db_vf;
-    DevBuf<BounceCand> db_cand;         // candidates (a, b) of every (TX, lit facet a)
-    DevBuf<int32_t> db_pcnt;            // virtual facets per candidate
-    DevBuf<int64_t> db_poff, db_pblk;   // their offsets and scan scratch
-    DevBuf<int64_t> db_txoff;           // first virtual facet of each TX [P + 1]
-    DevBuf<unsigned char> db_rows;      // FP32 evaluation: slow-time rows and geometry
-    DevBuf<double2> db_part;            // FP32 evaluation: the chunks' partial sums
-    DevBuf<uint32_t> db_keys, db_sort;  // rate groups: keys (twice), sort scratch
-    DevBuf<int32_t> db_perm, db_gcnt;   // order (twice), counts and turns of the keys
-    DevBuf<BounceGroup> db_group;
-    DevBuf<int64_t> db_gtot;
-    DevBuf<float2> db_node, db_gref;    // node rows, reference phases
+    DevBuf<int32_t> db_cnt{&moves};
+    DevBuf<int32_t> db_roots{&moves};           // the candidate traversal's subtree roots
+    DevBuf<int64_t> db_off{&moves}, db_blk{&moves};
+    DevBuf<BounceFacet> db_vf{&moves};
+    DevBuf<BounceCand> db_cand{&moves};         // candidates (a, b) of every (TX, lit facet a)
+    DevBuf<int32_t> db_pcnt{&moves};            // virtual facets per candidate
+    DevBuf<int64_t> db_poff{&moves}, db_pblk{&moves};   // their offsets and scan scratch
+    DevBuf<int64_t> db_txoff{&moves};           // first virtual facet of each TX [P + 1]
+    DevBuf<unsigned char> db_rows{&moves};      // FP32 evaluation: slow-time rows and geometry
+    DevBuf<double2> db_part{&moves};            // FP32 evaluation: the chunks' partial sums
+    DevBuf<uint32_t> db_keys{&moves}, db_sort{&moves};  // rate groups: keys (twice), sort scratch
+    DevBuf<int32_t> db_perm{&moves}, db_gcnt{&moves};   // order (twice), counts and turns of the keys
+    DevBuf<BounceGroup> db_group{&moves};
+    DevBuf<int64_t> db_gtot{&moves};
+    DevBuf<float2> db_node{&moves}, db_gref{&moves};    // node rows, reference phases
     int64_t db_n = 0;
-    DevBuf<uint32_t> mkeys, skeys;      // batched sort scratch
+    DevBuf<uint32_t> mkeys{&moves}, skeys{&moves};      // batched sort scratch
     int tpi_override = 0;               // synthesis tiles per item (autotuner), 0 = default
     int layout_S = 0;                   // synthesis samples per lane request, 0 = default
     uint64_t version = 1;               // bumped by every change of meshes/scene/radar/layout
@@ -224,7 +229,7 @@ struct bart_ctx {
         cudaGraphNode_t t0_node = nullptr;
         cudaKernelNodeParams t0_params{};
         int t0_arg = 0, n_args = 0;
-        uint64_t version = 0;
+        uint64_t version = 0, moves = 0;
         int path = -1, dtype = -1;
         void *adc = nullptr;
         cudaStream_t stream = nullptr;
@@ -1341,8 +1346,11 @@ static int run_frame(bart_ctx *ctx, double t0, int32_t path, void *adc, int32_t 
                            path != kPathAdjointMixed && !bounce;
     if (use_graph) {
         bart_ctx::FrameGraph &g = ctx->fg;
-        const bool hit = g.exec && g.version == ctx->version && g.path == (direct ? kPathMixedDirect : path) &&
-                         g.dtype == dtype && g.adc == adc && g.stream == s;
+        // the graph holds the buffers' addresses: none may have moved since, not
+        // even in a frame that is not replayed (timed, with stats, an adjoint)
+        const bool hit = g.exec && g.version == ctx->version && g.moves == ctx->moves &&
+                         g.path == (direct ? kPathMixedDirect : path) && g.dtype == dtype &&
+                         g.adc == adc && g.stream == s;
         if (!hit) {
             g.release();
             // record on a private stream (the legacy default stream, torch's
@@ -1386,6 +1394,7 @@ static int run_frame(bart_ctx *ctx, double t0, int32_t path, void *adc, int32_t 
                 return fail(BART_ECUDA, "frame graph: world-facet kernel node not found");
             }
             g.version = ctx->version;
+            g.moves = ctx->moves;
             g.path = direct ? kPathMixedDirect : path;
             g.dtype = dtype;
             g.adc = adc;

@@ -198,6 +198,50 @@ def test_graph_frame_at_new_t0_matches_oracle(sim):
     assert rel_l2(out.cpu().numpy(), ref) <= TOL_FP64
 
 
+def test_graph_after_its_buffers_moved():
+    """A frame that is not replayed (timed, or with stats) may let a buffer grow
+    that a recorded frame uses: the next graph frame records anew.  Both mixed
+    evaluations share the partial sums, at sizes of their own."""
+    def band(s, out):
+        s.simulate(pkg.PATH_MIXED, out=out)
+
+    def direct(s, out):
+        pkg.bart_simulate_mixed_direct(s.ctx, 0.0, out)
+
+    def timed(f):
+        def run(s, out):
+            pkg.bart_set_timing(s.ctx, True)
+            f(s, out)
+            torch.cuda.synchronize()
+            pkg.bart_set_timing(s.ctx, False)
+        return run
+
+    def fp64_stats(s, out):
+        s.simulate(pkg.PATH_FP64, stats=True)
+
+    # 512-float2 items of the partial sums, direct / band-limited: 18432 / 15360 at
+    # 128 chirps, 9216 / 14976 at 64
+    for first, between, N in [(band, timed(direct), 128), (direct, timed(band), 64),
+                              (band, fp64_stats, 64), (direct, fp64_stats, 64)]:
+        sc = sg.car_scene(seed=4, ntri=12000, M=256, N=N, P=3, Q=4)
+        s = pkg.Simulator(0)                          # buffers as the first frame needs them
+        try:
+            s.load_scene(sc)
+            pkg.bart_set_graph(s.ctx, True)
+            out = torch.empty(s.adc_shape(), dtype=torch.complex64, device="cuda")
+            other = torch.empty_like(out)
+            first(s, out)
+            ref = out.clone()
+            between(s, other)
+            out.zero_()
+            for _ in range(2):
+                first(s, out)
+                torch.cuda.synchronize()
+                assert torch.equal(out, ref)
+        finally:
+            s.close()
+
+
 @pytest.mark.parametrize("S,tpi", [(16, 8), (16, 64), (8, 8), (8, 512), (0, 0)])
 def test_synth_layouts_match_oracle(sim, S, tpi):
     scenes, frames, refs = reference()
