@@ -222,6 +222,7 @@ struct bart_ctx {
     int tpi_override = 0;               // synthesis tiles per item (autotuner), 0 = default
     int layout_S = 0;                   // synthesis samples per lane request, 0 = default
     uint64_t version = 1;               // bumped by every change of meshes/scene/radar/layout
+    uint64_t band_denied = 0;           // version whose band-limited scratch was not to be had
     bool graph = false;                 // replay frames as CUDA graphs
     struct FrameGraph {
         cudaGraph_t graph = nullptr;
@@ -690,8 +691,10 @@ static int32_t public_path(int32_t path) { return path == kPathMixedDirect ? -1 
 //    cube costs more than summing its facets over it (12 channels of 64 x
 //    256, direct against band-limited synthesis: 1 x 200 facets 0.20 / 0.09
 //    ms, 16 x 160 0.46 / 0.16, 64 x 96 0.48 / 0.37, 64 x 2 0.07 / 0.31, 256 x
-//    160 0.87 / 1.24), or
-//  - the per-instance coarse cubes could exceed 16 GB.
+//    160 0.87 / 1.24),
+//  - the per-instance coarse cubes could exceed 17 GB (its partial sums take
+//    as much again, up to 32 GB where lanes idle, M = 544), or
+//  - its scratch is not to be had (prepare_band).
 // A short frame gains too (one sedan, 1 chirp: 0.21 / 0.15 ms).
 static bool use_band(const bart_ctx *ctx, const RadarDev &rd, int32_t path, int64_t F, int I)
 {
@@ -768,6 +771,70 @@ static int plan_bounce_groups(bart_ctx *ctx, const RadarDev &rd, const BandArgs 
     gr.ref = ctx->db_gref.p;
     gr.groups = (int)groups;
     gr.items = tot[1];
+    return BART_OK;
+}
+
+// Tables, scratch and pointers of the band-limited mixed evaluation of I
+// instances in B scenes.  BART_ENOMEM: its scratch (up to 17 GB of coarse cubes
+// and 32 of partial sums) is not to be had, and the frame takes the direct sum.
+static int prepare_band(bart_ctx *ctx, const RadarDev &rd, int I, int B, int64_t F, BandArgs &bt,
+                        cudaStream_t s)
+{
+    const int O = rd.O;
+    if (ctx->band_sh.N != rd.N || ctx->band_sh.M != rd.M) {
+        BandShape sh;
+        band_shape(rd.N, rd.M, sh);
+        const BandSizes z = band_sizes(sh);
+        ctx->band_sh = BandShape{};
+        BART_TRY(ctx->band_tab.ensure((size_t)(z.nodes + z.wn + z.wm + z.base), "band tables"));
+        launch_band_tables(sh, ctx->band_tab.p, ctx->band_tab.p + z.nodes,
+                           reinterpret_cast<int *>(ctx->band_tab.p + z.nodes + z.wn + z.wm),
+                           ctx->band_tab.p + z.nodes + z.wn, s);
+        CUDA_TRY(cudaGetLastError(), "band table launch");
+        ctx->band_sh = sh;
+    }
+    const BandSizes z = band_sizes(ctx->band_sh);
+    const int64_t V = (int64_t)I * O;
+    bt.sh = ctx->band_sh;
+    bt.nodes = ctx->band_tab.p;
+    bt.wn = bt.nodes + z.nodes;
+    bt.wm = bt.wn + z.wn;
+    bt.base = reinterpret_cast<const int *>(bt.wm + z.wm);
+    bt.I = I;
+    bt.B = B;
+    bt.O = O;
+    bt.chunk_target = synth_band_target();
+    bt.fixed_chunk = 32 * ctx->tpi_override;
+    bt.max_items = band_max_items(bt.sh, V, bt.chunk_target, (int64_t)O * F, bt.fixed_chunk);
+    BART_TRY(ctx->partial.ensure((size_t)bt.max_items * 32 * kBandS, "synthesis partials"));
+    BART_TRY(ctx->band_coarse.ensure((size_t)(V * rd.N * rd.M), "band coarse samples"));
+    bt.box = ctx->box.p;
+    bt.scene_inst = ctx->d_sinst.p;
+    bt.ioff = ctx->d_ioff.p;
+    bt.partial = reinterpret_cast<float4 *>(ctx->partial.p);
+    bt.coarse = ctx->band_coarse.p;
+    // the small arrays in one allocation, widest elements first
+    auto carve = [&](unsigned char *p) -> size_t {
+        size_t n = 0;
+        auto take = [&](auto *&field, int64_t count) {
+            using T = std::remove_reference_t<decltype(*field)>;
+            field = reinterpret_cast<T *>(p + n);
+            n += ((size_t)count * sizeof(T) + 15) / 16 * 16;
+        };
+        take(bt.ref, V * rd.N);
+        take(bt.refn, V * rd.N);
+        take(bt.items, bt.max_items);
+        take(bt.plan, I);
+        take(bt.coff, V);
+        take(bt.vstart, V);
+        take(bt.vcnt, V);
+        take(bt.item0, V + 1);
+        take(bt.item_counter, 1);
+        take(bt.chunk, 1);
+        return n;
+    };
+    BART_TRY(ctx->band_ws.ensure(carve(nullptr), "band plans and items"));
+    carve(ctx->band_ws.p);
     return BART_OK;
 }
 
@@ -918,9 +985,22 @@ static int run_frame(bart_ctx *ctx, double t0, int32_t path, void *adc, int32_t 
                         ? ctx->tpi_override
                         : synth_tiles_per_item(*std::max_element(scene_F.begin(), scene_F.end()));
     int64_t max_items = 0;
-    const bool band = !direct && (path == BART_PATH_MIXED || path == BART_PATH_SPECTRAL) &&
-                      use_band(ctx, rd, path, F, I);
+    bool band = !direct && (path == BART_PATH_MIXED || path == BART_PATH_SPECTRAL) &&
+                ctx->band_denied != ctx->version && use_band(ctx, rd, path, F, I);
     BandArgs bt{};
+    if (band) {
+        const int rc = prepare_band(ctx, rd, I, B, F, bt, s);
+        if (rc == BART_ENOMEM) {
+            // the direct sum, for all frames until the configuration changes
+            g_err.clear();
+            ctx->band_coarse.release();
+            ctx->band_ws.release();
+            ctx->band_denied = ctx->version;
+            band = false;
+        } else if (rc != BART_OK) {
+            return rc;
+        }
+    }
     const bool mixed_rows = path == BART_PATH_MIXED || path == BART_PATH_SPECTRAL ||
                             path == kPathAdjointMixed;
     const bool kin_rows = mixed_rows && (!band || stats);
@@ -942,62 +1022,7 @@ static int run_frame(bart_ctx *ctx, double t0, int32_t path, void *adc, int32_t 
             BART_TRY(ctx->kin.ensure((size_t)A * F * kKinRowWords, "kinematics rows"));
             BART_TRY(ctx->kquad.ensure((size_t)A * F * kKinQuadWords, "kinematics quadratics"));
         }
-        if (band) {
-            if (ctx->band_sh.N != rd.N || ctx->band_sh.M != rd.M) {
-                BandShape sh;
-                band_shape(rd.N, rd.M, sh);
-                const BandSizes z = band_sizes(sh);
-                ctx->band_sh = BandShape{};
-                BART_TRY(ctx->band_tab.ensure((size_t)(z.nodes + z.wn + z.wm + z.base), "band tables"));
-                launch_band_tables(sh, ctx->band_tab.p, ctx->band_tab.p + z.nodes,
-                                   reinterpret_cast<int *>(ctx->band_tab.p + z.nodes + z.wn + z.wm),
-                                   ctx->band_tab.p + z.nodes + z.wn, s);
-                CUDA_TRY(cudaGetLastError(), "band table launch");
-                ctx->band_sh = sh;
-            }
-            const BandSizes z = band_sizes(ctx->band_sh);
-            const int64_t V = (int64_t)I * O;
-            bt.sh = ctx->band_sh;
-            bt.nodes = ctx->band_tab.p;
-            bt.wn = bt.nodes + z.nodes;
-            bt.wm = bt.wn + z.wn;
-            bt.base = reinterpret_cast<const int *>(bt.wm + z.wm);
-            bt.I = I;
-            bt.B = B;
-            bt.O = O;
-            bt.chunk_target = synth_band_target();
-            bt.fixed_chunk = 32 * ctx->tpi_override;
-            bt.max_items = band_max_items(bt.sh, V, bt.chunk_target, (int64_t)O * F, bt.fixed_chunk);
-            BART_TRY(ctx->partial.ensure((size_t)bt.max_items * 32 * kBandS, "synthesis partials"));
-            BART_TRY(ctx->band_coarse.ensure((size_t)(V * rd.N * rd.M), "band coarse samples"));
-            bt.box = ctx->box.p;
-            bt.scene_inst = ctx->d_sinst.p;
-            bt.ioff = ctx->d_ioff.p;
-            bt.partial = reinterpret_cast<float4 *>(ctx->partial.p);
-            bt.coarse = ctx->band_coarse.p;
-            // the small arrays in one allocation, widest elements first
-            auto carve = [&](unsigned char *p) -> size_t {
-                size_t n = 0;
-                auto take = [&](auto *&field, int64_t count) {
-                    using T = std::remove_reference_t<decltype(*field)>;
-                    field = reinterpret_cast<T *>(p + n);
-                    n += ((size_t)count * sizeof(T) + 15) / 16 * 16;
-                };
-                take(bt.ref, V * rd.N);
-                take(bt.refn, V * rd.N);
-                take(bt.items, bt.max_items);
-                take(bt.plan, I);
-                take(bt.coff, V);
-                take(bt.vstart, V);
-                take(bt.vcnt, V);
-                take(bt.item0, V + 1);
-                take(bt.item_counter, 1);
-                take(bt.chunk, 1);
-                return n;
-            };
-            BART_TRY(ctx->band_ws.ensure(carve(nullptr), "band plans and items"));
-            carve(ctx->band_ws.p);
-        } else if (path == BART_PATH_MIXED) {
+        if (!band && path == BART_PATH_MIXED) {
             BART_TRY(ctx->partial.ensure((size_t)synth_partial_words(scene_F.data(), B, rd, rd.N,
                                                                      tpi, ctx->layout_S),
                                          "synthesis partials"));

@@ -82,3 +82,47 @@ def test_bounded_wait_expiry_reports_etimeout_and_the_context_stays_usable():
         assert np.abs(rdm - ref).max() <= 1e-5 * ref.max()
     finally:
         sim.close()
+
+
+@pytest.mark.parametrize("path", [pkg.PATH_MIXED, pkg.PATH_SPECTRAL])
+def test_frames_run_without_the_band_limited_scratch(path):
+    """Where the scratch of the band-limited evaluation is not to be had, the
+    frame goes through the direct sum (the spectral kernel), as a long frame
+    does, until the configuration changes; no call fails that needs less."""
+    sc = sg.car_scene(seed=3, ntri=2500, M=128, N=24, P=2, Q=2)
+    sim = pkg.Simulator(0)
+    try:
+        sim.load_scene(sc)
+        band = sim.simulate(path).clone()
+        ref = sim.simulate(pkg.PATH_FP64)
+    finally:
+        sim.close()
+    denied = 0
+    for nth in range(1, 8):
+        sim = pkg.Simulator(0)
+        try:
+            sim.load_scene(sc)
+            direct = torch.empty_like(band)
+            pkg.bart_simulate_mixed_direct(sim.ctx, 0.0, direct)     # the common buffers
+            pkg.bart_inject_alloc_failure(nth)
+            try:
+                got = sim.simulate(path)
+            except pkg.BartError as e:                               # the spectral kernel's own table
+                assert path == pkg.PATH_SPECTRAL and "spectral" in str(e), e
+                continue
+            finally:
+                pkg.bart_inject_alloc_failure(0)
+            assert float((got.to(ref.dtype) - ref).norm() / ref.norm()) <= 1e-4
+            if torch.equal(got, band):
+                break                                                # nth beyond its allocations
+            denied += 1
+            again = sim.simulate(path)
+            assert not torch.equal(again, band)
+            if path == pkg.PATH_MIXED:                               # (the spectral kernel's order varies)
+                assert torch.equal(got, direct) and torch.equal(again, direct)
+            sim.load_scene(sc)
+            assert torch.equal(sim.simulate(path), band)
+        finally:
+            pkg.bart_inject_alloc_failure(0)
+            sim.close()
+    assert denied >= 2, denied                                       # tables, coarse sums, plans
