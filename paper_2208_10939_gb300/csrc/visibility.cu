@@ -430,7 +430,15 @@ __global__ void __launch_bounds__(kVisThreads) visibility_far_kernel(const __gri
 
 // Antennas of a group: all TX or all RX of up to 16 where that leaves 32k
 // (facet, group) pairs, fewer for small scenes (sedan, visibility and lists:
-// two groups 93 us, four 92, seven single antennas 117)
+// two groups 93 us, four 92, seven single antennas 117), and only neighbours: a
+// bundle visits every box between its antennas' directions, so that far-apart
+// ones are cheaper alone.  12 x 16 antennas over an intersection of 125k facets,
+// bundles of 16 / these / each alone: 0.03 m apart 1.24 / 1.24 / 2.99 ms, 0.1 m
+// 2.33 / 1.72 / 3.01, 0.2 m 3.14 / 2.06 / 2.99, 0.3 m 4.1 / 2.9 / 2.9, 5 m
+// 31.3 / 2.8 / 2.8; pairs 0.3 m apart over a 100k-facet sedan 1.16, each alone 0.50.
+constexpr double kBundleExtent = 0.5;        // metres along an axis
+constexpr double kBundleStep = 0.25;         // and for each antenna after the first
+
 static AntGroups ant_groups(const RadarDev &rd, int64_t F)
 {
     AntGroups ag;
@@ -439,21 +447,33 @@ static AntGroups ant_groups(const RadarDev &rd, int64_t F)
     while (size > 1 && F * ((rd.P + size - 1) / size + (rd.Q + size - 1) / size) < want) size /= 2;
     ag.n_groups = 0;
     auto add = [&](int first, int n) {
-        for (int s = 0; s < n; s += size) {
+        for (int s = first; s < first + n;) {
             const int g = ag.n_groups++;
-            ag.first[g] = first + s;
-            ag.n[g] = n - s < size ? n - s : size;
-            for (int r = 0; r < 3; ++r) {
-                double lo = rd.ant[first + s][r], hi = lo;
-                for (int i = 1; i < ag.n[g]; ++i) {
-                    lo = fmin(lo, rd.ant[first + s + i][r]);
-                    hi = fmax(hi, rd.ant[first + s + i][r]);
+            double lo[3], hi[3];
+            for (int r = 0; r < 3; ++r) lo[r] = hi[r] = rd.ant[s][r];
+            int e = s + 1;
+            for (; e < first + n && e - s < size; ++e) {
+                double l[3], h[3], ext = 0.0;
+                for (int r = 0; r < 3; ++r) {
+                    l[r] = fmin(lo[r], rd.ant[e][r]);
+                    h[r] = fmax(hi[r], rd.ant[e][r]);
+                    ext = fmax(ext, h[r] - l[r]);
                 }
-                const double m = 0.5 * (lo + hi);
+                if (ext > fmin(kBundleExtent, kBundleStep * (e - s))) break;
+                for (int r = 0; r < 3; ++r) {
+                    lo[r] = l[r];
+                    hi[r] = h[r];
+                }
+            }
+            ag.first[g] = s;
+            ag.n[g] = e - s;
+            for (int r = 0; r < 3; ++r) {
+                const double m = 0.5 * (lo[r] + hi[r]);
                 ag.mid[g][r] = (float)m;
                 ag.mid_lo[g][r] = (float)(m - (double)ag.mid[g][r]);
-                ag.half[g][r] = (float)((hi - lo) * 0.50001);
+                ag.half[g][r] = (float)((hi[r] - lo[r]) * 0.50001);
             }
+            s = e;
         }
     };
     add(0, rd.P);

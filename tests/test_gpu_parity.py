@@ -460,3 +460,17 @@ def test_large_facets_match_oracle(sim, name):
         err = rel_l2(sim.simulate(path).cpu().numpy(), ref)
         print(f"{name}: path {path} relL2 {err:.3e}")
         assert err <= TOL_MIXED
+
+
+@pytest.mark.parametrize("apart", [0.05, 0.24, 0.3, 4.0])
+def test_visibility_of_far_apart_antennas_matches_oracle(sim, apart):
+    """Rays of neighbouring antennas go down the hierarchy as bundles, those of
+    far-apart ones alone, or some of each: every state as the oracle's."""
+    sc = sg.car_scene(seed=3, ntri=20_000, M=32, N=2, P=5, Q=4)
+    r = sc.radar
+    r.tx = np.array([[apart * i * (1 + (i == 4)), 0.0, 5.0 + 0.1 * i] for i in range(5)])
+    r.rx = np.array([[-0.02, 0.3 * i * i * apart, 5.0] for i in range(4)])
+    fr = oracle.Frame(sc)
+    sim.load_scene(sc)
+    sim.simulate(pkg.PATH_MIXED)
+    assert np.array_equal(sim.visibility().cpu().numpy(), fr.state)
