@@ -656,8 +656,7 @@ fft64_kernel(const double2 *__restrict__ in, void *__restrict__ out, const float
             }
         }
         if (b0 == c0) {
-            fft64::fill_twiddles(tw, L);
-            fft64::fill_window(win, L, window);
+            fft64::fill_tables(tw, win, L, window);
         }
         asm volatile("cp.async.wait_all;" ::: "memory");
         __syncthreads();
@@ -721,8 +720,9 @@ static void fft64_launch(const void *in, void *out, const float *G, const RadarD
         const int64_t batches = (need + cap - 1) / cap;
         B = (need + batches - 1) / batches;
     }
+    // a thread a radix-8 butterfly; at least 192 for the tables (fft64.cuh)
     const int64_t want = (B * L / 8 + 31) / 32 * 32;
-    const int threads = (int)std::max<int64_t>(64, std::min<int64_t>(kFft64Threads, want));
+    const int threads = (int)std::max<int64_t>(192, std::min<int64_t>(kFft64Threads, want));
     cudaFuncSetAttribute(fft64_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)smem(B));
     fft64_kernel<MODE><<<(unsigned int)grid, threads, smem(B), s>>>(
