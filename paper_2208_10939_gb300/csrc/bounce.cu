@@ -1740,9 +1740,17 @@ int bounce_synth_chunks(const RadarDev &rd)
     return (int)std::max<int64_t>(1, std::min<int64_t>(16, (target + rows - 1) / rows));
 }
 
-bool bounce_groups_apply(const RadarDev &rd, const BandShape &sh)
+// Planning the groups and interpolating them takes 0.1 to 0.25 ms, so the
+// terms that they can save have to be worth it (a group has 8 nodes or more,
+// mostly 10).  A frame in groups / at every chirp: 634 virtual facets, 64 chirps
+// of 512, one channel (1.8e7) 0.90 / 0.67 ms; 3143, 64 of 128, 2 x 2 (4.3e7) 1.00 /
+// 0.98; 9437, 32 of 128, 2 x 2 (5.3e7) 1.46 / 1.44; 3143, 32 of 512, 2 x 2 (7.1e7)
+// 1.14 / 1.01; 1902, 32 of 512, 3 x 4 (8.6e7) 0.91 / 1.03; 9437, 64 of 128, 2 x 2
+// (1.3e8) 1.47 / 1.70; 14167, 64 of 128, 3 x 4 (3.9e8) 1.69 / 2.61.
+bool bounce_groups_apply(const RadarDev &rd, const BandShape &sh, int64_t total)
 {
-    return sh.n_n > 2 && bounce_mid_time(rd) > 0.0;
+    return sh.n_n > 2 && bounce_mid_time(rd) > 0.0 &&
+           (double)total * rd.Q * (rd.N - 10) * rd.M >= 8e7;
 }
 
 int64_t bounce_group_keys() { return kDbKeys; }

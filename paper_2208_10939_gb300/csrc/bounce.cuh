@@ -83,8 +83,9 @@ struct BounceGroups {
     int groups;
     int64_t items;
 };
-// whether the tables serve the frame; keys of the counting arrays
-bool bounce_groups_apply(const RadarDev &rd, const BandShape &sh);
+// whether the tables serve the frame of `total` virtual facets and may save more
+// than the groups cost; keys of the counting arrays
+bool bounce_groups_apply(const RadarDev &rd, const BandShape &sh, int64_t total);
 int64_t bounce_group_keys();
 // groups of the virtual facets from their rows; cnt: 2 x keys words; tot:
 // groups, work items, partial rows, node rows, records per RX

@@ -1258,7 +1258,7 @@ static int run_frame(bart_ctx *ctx, double t0, int32_t path, void *adc, int32_t 
                                        ctx->db_rows.p + total * bounce_geo_bytes(),
                                        ctx->db_rows.p, s);
                     launches += 1;
-                    if (band && bounce_groups_apply(rd, bt.sh))
+                    if (band && bounce_groups_apply(rd, bt.sh, total))
                         BART_TRY(plan_bounce_groups(ctx, rd, bt, total, s, db_groups, launches));
                     const int nch = bounce_synth_chunks(rd);
                     if (!db_groups.group && nch > 1)
