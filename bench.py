@@ -57,48 +57,10 @@ BOUNCE = ("moving sedan 20k tris on a 20 m x 20 m static ground (0.5 m cells, 32
 OPS_PER_TERM = 24
 BAND_NOTE = ("band-limited: direct-sum operations per second of the synthesis stage; the kernel "
              "evaluates the nodes of each instance only, so this is no fraction of the peak")
-# DRAM traffic of one synthesis launch and the FMA-pipe activity, from ncu
-# captures of the synthesis kernel on 4 TX x 4 RX cuts of the frame.  A work
-# item takes one record chunk of a channel through all its chirps, so a
-# (channel, lit facet) record's inputs come from HBM once and from L2 for the
-# other chirps: reads grow with those pairs (terms / (N M)), not with the
-# terms (16 and 64 chirps read 3.41 and 3.28 GB); the items' partial sums
-# grow with the (channel, chirp) rows.  Valid only while the kernel's sources
-# hash to the value they had at the capture (the direct kernel's; the
-# band-limited evaluation has no such capture).
-SYNTH_PROFILE = {"sources_sha256_16": "4239e3318de9d32c", "samples_per_lane": 16,
-                 "dram_read_bytes_per_channel_facet": 3.277169152e9 / (4 * 50804670464 / (64 * 512)),
-                 "dram_write_bytes_per_row": 75.109632e6 / (16 * 64),
-                 "fma_pipe_active": 0.686}
-SYNTH_SOURCES = ("synth.cu", "bart_internal.cuh", "record_fp64.cuh", "mixed_record.cuh")
 # the double-bounce synthesis: 3 centres x (2 accumulates + 4 rotation
 # operations) per vertex-form term of the direct evaluation, which the rate
-# groups (bounce.cuh) replace by their nodes where they apply; ncu figures of the
-# direct launch on the sedan-over-ground frame, valid while its sources hash as
-# at the capture
+# groups (bounce.cuh) replace by their nodes where they apply
 BOUNCE_OPS_PER_TERM = 18
-BOUNCE_SOURCES = ("bounce.cu", "bounce.cuh", "geom64.cuh", "record_fp64.cuh", "bart_internal.cuh")
-BOUNCE_PROFILE = {"sources_sha256_16": "0ad733dd979e3494", "fma_pipe_active": 0.324, "fp64_pipe_active": 0.528,
-                  "issue_active": 0.523, "warps_active": 0.179}
-
-
-def synth_sources_hash(sources=SYNTH_SOURCES) -> str:
-    import hashlib
-    h = hashlib.sha256()
-    for f in sources:
-        with open(os.path.join(ROOT, "paper_2208_10939_gb300", "csrc", f), "rb") as fh:
-            h.update(fh.read())
-    return h.hexdigest()[:16]
-
-
-def synth_profile(samples_per_lane: int):
-    """The captured per-term DRAM traffic and FMA-pipe activity, or None when
-    the kernel (its sources, or the template instance the layout picks)
-    differs from the captured one."""
-    if (samples_per_lane != SYNTH_PROFILE["samples_per_lane"]
-            or SYNTH_PROFILE["sources_sha256_16"] != synth_sources_hash()):
-        return None
-    return SYNTH_PROFILE
 
 
 def layout_samples(M: int, S_req: int) -> int:
@@ -774,15 +736,12 @@ def double_bounce_lines(pkg, sg, torch, dev, args, peaks) -> dict:
                 syn_s = statistics.median(syn) / 1e3
                 if peaks:
                     ach = bt * BOUNCE_OPS_PER_TERM / syn_s / 1e12
-                    prof = (BOUNCE_PROFILE if BOUNCE_PROFILE["sources_sha256_16"] ==
-                            synth_sources_hash(BOUNCE_SOURCES) else None)
                     out["roofline"] = {
                         "bound": "alu", "kernel": "bounce_synth_f32_kernel<8, true>",
                         "ops_per_term": BOUNCE_OPS_PER_TERM, "achieved": ach,
                         "peak": peaks["fp32_fma_pipe_tops"], "frac": None,
                         "unit": "Top/s (FP32 FMA-pipe operations)",
                         "peak_basis": "measured (bart_measure_peaks)",
-                        "ncu": prof,
                         "note": "direct-sum operations per second: virtual facets are "
                                 "evaluated at the chirp nodes of their rate groups only, so "
                                 "this is no fraction of the peak"}
@@ -945,7 +904,6 @@ def main():
     achieved = terms / synth_launches * OPS_PER_TERM / (synth_avg_ms / 1e3) / 1e12
     S_used = layout_samples(M, 0 if layout is None else layout["samples_per_lane"])
     band = S_used == 16
-    prof = None if band else synth_profile(S_used)
     if peaks:
         peak, peak_basis = peaks["fp32_fma_pipe_tops"], (
             "measured: FP32 FMA-pipe operations/s of this GPU (bart_measure_peaks, the faster "
@@ -957,13 +915,7 @@ def main():
                 "achieved": achieved, "peak": peak, "unit": "Top/s (FP32 FMA-pipe operations)",
                 "frac": None if band else achieved / peak,
                 "note": BAND_NOTE if band else None,
-                "traffic": None if prof is None
-                else (prof["dram_read_bytes_per_channel_facet"] * terms / (N * M)
-                      + prof["dram_write_bytes_per_row"] * O * N) / synth_launches,
-                "traffic_unit": "bytes per launch (ncu dram reads of a cut per (channel, lit facet) "
-                                "+ writes per (channel, chirp) row)",
                 "ops_per_term": OPS_PER_TERM, "launch_ms": synth_avg_ms,
-                "ncu_fma_pipe_active": None if prof is None else prof["fma_pipe_active"],
                 "peak_basis": peak_basis}
 
     e2e = e2e_run(pkg, torch, sim, scene, pkg.PATH_MIXED, args.e2e_steps, job_terms_per_step)

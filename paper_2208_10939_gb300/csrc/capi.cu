@@ -677,8 +677,10 @@ int bart_radar_set(bart_ctx *ctx, const bart_radar *r)
 constexpr int kPathAdjoint = 100;
 constexpr int kPathAdjointMixed = 101;
 // the mixed path at every chirp and sample (bart_simulate_mixed_direct): the
-// forward of the mixed adjoint, which goes through them too.  Its rounding is
-// what the adjoint's gradients of weakly reflecting facets depend on.
+// forward that the mixed adjoint differentiates, term by term.  A loss of the
+// band-limited cube under this adjoint moves the gradients of weakly reflecting
+// facets by the two evaluations' difference (8e-6 of the cube, mostly the direct
+// sum's own error); an adjoint of the band-limited evaluation is not built.
 constexpr int kPathMixedDirect = 102;
 // a caller's path: not that one
 static int32_t public_path(int32_t path) { return path == kPathMixedDirect ? -1 : path; }
@@ -704,12 +706,16 @@ static bool use_band(const bart_ctx *ctx, const RadarDev &rd, int32_t path, int6
 }
 
 // The FP64 path's two evaluations: band-limited (band64.cuh) unless the delay
-// form is not the facet's own, the frame is longer than its tables go, or its
-// scratch (four cubes an instance) would exceed 16 GB.  However small the
-// instances, interpolating one costs about what the direct sum spends on one
-// lit facet (100 FP64 operations a sample), so their size is no condition, and
-// a scene gives the same bits alone and in a batch.  A 5k-facet car on 12
-// channels of 32 x 256: 33.1 ms by the direct sum, 1.9 ms band-limited.
+// form is not the facet's own, the frame is longer than its tables go, its
+// scratch (four cubes an instance, or two for each of its four cells) would
+// exceed 16 GB, or that is not to be had.  However small the instances,
+// interpolating one costs about what the direct sum spends on one lit facet (100
+// FP64 operations a sample), so their size is no condition.  A scene gives the
+// same bits alone and in a batch as long as the batch keeps cells where the scene
+// alone has them (up to 2^27 instance samples, 341 instances on 12 channels of 128
+// x 256) or the evaluation (up to 2^28).  A 5k-facet car on 12 channels of 32 x 256:
+// 33.1 ms by the direct sum, 1.9 ms band-limited; 64 instances of two facets, 32 x
+// 256: 3.6 and 1.8.
 static bool use_band64(const RadarDev &rd, int I)
 {
     return !rd.far_field && !rd.delay_ref && rd.N <= 1024 && (int64_t)I * rd.O <= 65535 &&

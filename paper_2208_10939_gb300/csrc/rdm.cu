@@ -956,10 +956,8 @@ static int run_rdm_reg(const float2 *adc, const RadarDev &rd, int groups, float2
 }
 
 static void run_rdm32(const void *adc, const RadarDev &rd, int groups, void *ws, float *rdm,
-                    int *status, cudaStream_t s)
+                      int *status, cudaStream_t s)
 {
-    using T = float;
-    using C = float2;
     const int M = rd.M, N = rd.N, O = rd.O;
     const int64_t Oall = (int64_t)O * groups;
     const int64_t MN = (int64_t)M * N;
@@ -973,27 +971,28 @@ static void run_rdm32(const void *adc, const RadarDev &rd, int groups, void *ws,
         return;
     }
     // range pass, transposed output Xt[o][r][n]
-    const int TN = rdm_tn(N, M, sizeof(C));
-    const size_t sm1 = (size_t)(2 * TN * M + tw_len(M)) * sizeof(C);
-    cudaFuncSetAttribute(range_fft_t_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    const int TN = rdm_tn(N, M, sizeof(float2));
+    const size_t sm1 = (size_t)(2 * TN * M + tw_len(M)) * sizeof(float2);
+    cudaFuncSetAttribute(range_fft_t_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)sm1);
     const int t1 = std::min(1024, std::max(128, TN * M / 4));
-    range_fft_t_kernel<T><<<dim3((unsigned int)((N + TN - 1) / TN), (unsigned int)Oall), t1, sm1,
-                            s>>>(reinterpret_cast<const C *>(adc), reinterpret_cast<C *>(ws), N,
-                                 M, TN, rd.window);
+    const float2 *x = static_cast<const float2 *>(adc);
+    float2 *X = static_cast<float2 *>(ws);
+    range_fft_t_kernel<float><<<dim3((unsigned int)((N + TN - 1) / TN), (unsigned int)Oall), t1, sm1,
+                                s>>>(x, X, N, M, TN, rd.window);
     // Doppler pass and the per-group channel sums
     const int RB = rdm_rb(N, M);
     const int CPB = rdm_cpb(O, M / RB, groups);
     const int G = (O + CPB - 1) / CPB;
-    T *part = reinterpret_cast<T *>(reinterpret_cast<C *>(ws) + Oall * N * M);
-    const size_t sm2 = (size_t)(2 * RB * N + tw_len(N)) * sizeof(C) + (size_t)RB * N * sizeof(T);
-    cudaFuncSetAttribute(doppler_sum_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    float *part = reinterpret_cast<float *>(X + Oall * N * M);
+    const size_t sm2 =
+        (size_t)(2 * RB * N + tw_len(N)) * sizeof(float2) + (size_t)RB * N * sizeof(float);
+    cudaFuncSetAttribute(doppler_sum_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)sm2);
-    doppler_sum_kernel<T><<<dim3((unsigned int)(M / RB), (unsigned int)(G * groups)), 256, sm2,
-                            s>>>(reinterpret_cast<const C *>(ws), N, M, RB, CPB, O, rd.window,
-                                 part);
-    rdm_sum_kernel<T><<<(unsigned int)((MN * groups + 255) / 256), 256, 0, s>>>(part, G, MN,
-                                                                               groups, rdm);
+    doppler_sum_kernel<float><<<dim3((unsigned int)(M / RB), (unsigned int)(G * groups)), 256, sm2,
+                                s>>>(X, N, M, RB, CPB, O, rd.window, part);
+    rdm_sum_kernel<float><<<(unsigned int)((MN * groups + 255) / 256), 256, 0, s>>>(
+        part, G, MN, groups, rdm);
 }
 
 // complex128: range pass, Doppler pass to a power map a channel, sum of the maps
@@ -1030,31 +1029,27 @@ static void run_rdm_cube64(const void *adc, const RadarDev &rd, void *X, void *c
 }
 
 static void run_rdm_adjoint32(const void *adc, const float *grad_rdm, const RadarDev &rd,
-                            int groups, void *X, void *cube, float *rdm, void *grad_adc,
-                            cudaStream_t s)
+                              int groups, void *X, void *cube, void *grad_adc, cudaStream_t s)
 {
-    using T = float;
-    using C = float2;
     RadarDev all = rd;
     all.O = rd.O * groups;
     const int M = rd.M, N = rd.N;
-    // forward cube Y (and the RDM, unused) into `cube`
-    range_fft<T>(adc, all, X, s);
-    doppler<T>(X, all, cube, s);
+    // forward cube Y into `cube`
+    range_fft<float>(adc, all, X, s);
+    doppler<float>(X, all, cube, s);
     const int RB = rdm_rb(N, M);
-    const size_t sm2 = (size_t)(2 * RB * N + tw_len(N)) * sizeof(C);
-    cudaFuncSetAttribute(doppler_adjoint_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    const size_t sm2 = (size_t)(2 * RB * N + tw_len(N)) * sizeof(float2);
+    cudaFuncSetAttribute(doppler_adjoint_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)sm2);
-    doppler_adjoint_kernel<T><<<dim3((unsigned int)(M / RB), (unsigned int)all.O), 256, sm2, s>>>(
-        reinterpret_cast<const C *>(cube), grad_rdm, rd.O, N, M, RB, rd.window,
-        reinterpret_cast<C *>(X));
-    const size_t sm1 = (size_t)(2 * M + tw_len(M)) * sizeof(C);
+    doppler_adjoint_kernel<float><<<dim3((unsigned int)(M / RB), (unsigned int)all.O), 256, sm2, s>>>(
+        reinterpret_cast<const float2 *>(cube), grad_rdm, rd.O, N, M, RB, rd.window,
+        reinterpret_cast<float2 *>(X));
+    const size_t sm1 = (size_t)(2 * M + tw_len(M)) * sizeof(float2);
     const int t1 = M / 2 < 1024 ? (M / 2 < 32 ? 32 : M / 2) : 1024;
-    cudaFuncSetAttribute(range_adjoint_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaFuncSetAttribute(range_adjoint_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)sm1);
-    range_adjoint_kernel<T><<<(unsigned int)((int64_t)all.O * N), t1, sm1, s>>>(
-        reinterpret_cast<const C *>(X), M, rd.window, reinterpret_cast<C *>(grad_adc));
-    (void)rdm;
+    range_adjoint_kernel<float><<<(unsigned int)((int64_t)all.O * N), t1, sm1, s>>>(
+        reinterpret_cast<const float2 *>(X), M, rd.window, reinterpret_cast<float2 *>(grad_adc));
 }
 
 static void run_rdm_adjoint64(const void *adc, const float *grad_rdm, const RadarDev &rd,
@@ -1071,7 +1066,7 @@ void launch_rdm_adjoint(const void *adc, int dtype, const float *grad_rdm, const
                         int groups, void *X, void *cube, void *grad_adc, cudaStream_t s)
 {
     if (dtype == BART_C64)
-        run_rdm_adjoint32(adc, grad_rdm, rd, groups, X, cube, nullptr, grad_adc, s);
+        run_rdm_adjoint32(adc, grad_rdm, rd, groups, X, cube, grad_adc, s);
     else
         run_rdm_adjoint64(adc, grad_rdm, rd, groups, X, cube, grad_adc, s);
 }
