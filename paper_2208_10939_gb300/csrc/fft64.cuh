@@ -12,9 +12,10 @@
 //    the columns it transforms, and a twiddle table of L % 8 == 0 entries from
 //    one octant (an eighth of the sincospi).
 // Small maps wait for chains of dependent operations, so a block has at least 192
-// threads, and both tables come from one loop (the four launches of the map's
-// adjoint, 12 x 32 x 128: 51.5 us, 62.6 with 64 threads and two loops; 4 x 27 x
-// 288: 51.5 and 69.2; radix 2 and 3 in blocks of 8 rows took 51.5 and 57.6).
+// threads, and both tables come from one loop, a warp of either kind (the four
+// launches of the map's adjoint, 12 x 32 x 128: 47.4 us, 62.6 with 64 threads and
+// a loop for each; 4 x 27 x 288: 49.0 and 69.2; radix 2 and 3 in blocks of 8 rows
+// took 51.5 and 57.7).
 #pragma once
 
 #include <cuda_runtime.h>
@@ -98,12 +99,14 @@ __device__ inline void fill_tables(double2 *tw, double *win, int L, int kind)
 {
     const bool oct = (L & 7) == 0;
     const int h = L / 2, q = L / 4, nt = oct ? L / 8 + 1 : L;
-    for (int i = threadIdx.x; i < nt + (L + 1) / 2; i += blockDim.x) {
-        if (i >= nt) {
-            const int k = i - nt;
+    const int w0 = (nt + 31) & ~31;                  // the window from a warp of its own on
+    for (int i = threadIdx.x; i < w0 + (L + 1) / 2; i += blockDim.x) {
+        if (i >= w0) {
+            const int k = i - w0;
             win[k] = win[L - 1 - k] = window_val<double>(k, L, kind);
             continue;
         }
+        if (i >= nt) continue;
         double s, c;
         sincospi((double)(2 * i) / (double)L, &s, &c);
         if (!oct) {
