@@ -374,12 +374,13 @@ int bart_simulate_adjoint_mixed(bart_ctx *ctx, double t0, const void *grad_adc, 
 
 /* Frame graphs.  With enable = 1, bart_simulate_frame records its kernel
  * launches (world facets, hierarchy, visibility, lit lists, kinematics,
- * synthesis: some 25-40 launches on two streams) into a CUDA graph the
+ * synthesis: some 15-40 launches on two streams) into a CUDA graph the
  * first time it meets a configuration -- meshes, instances, partition,
  * radar, synthesis layout, path, dtype, output pointer and stream -- and
  * replays that graph, one launch, on later calls that differ at most in
  * t0 (the new t0 is written into the recorded world-facet launch).  Any
- * change of the configuration records again.  Calls that request stats,
+ * change of the configuration records again, and so does a device buffer
+ * of the context that another call had to move.  Calls that request stats,
  * or run with timing enabled, run directly.  enable = 0 (the default)
  * drops the graph.  Errors: EINVAL, ECUDA. */
 int bart_set_graph(bart_ctx *ctx, int32_t enable);
