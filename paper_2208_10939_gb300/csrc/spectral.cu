@@ -88,10 +88,23 @@ __device__ __forceinline__ void kernel_taps(const float (&c)[W][D + 1], float t,
     }
 }
 
-// cell of tap j for a line whose taps start at cell g0 (within a few cells of [0, G))
+// cell of tap j for a line whose taps start at cell g0, in [-G, 2G)
 __device__ __forceinline__ int wrap_cell(int g, int G)
 {
     return g < 0 ? g + G : (g >= G ? g - G : g);
+}
+
+// A line's whole cells from the record's own in [0, G), kept where wrap_cell
+// finds them: a vertex metres from its facet's centroid under a steep chirp (mu u
+// / (fs c) near or beyond a cycle per sample) is turns of G away, and the line is
+// its alias, since the samples are whole.  Not a number or infinite: 0.
+__device__ __forceinline__ float near_cell(float x, float G)
+{
+    if (fabsf(x) >= G - 16.f) {
+        x = fmodf(x, G);
+        x = x >= 0.5f * G ? x - G : x < -0.5f * G ? x + G : x;
+    }
+    return x;
 }
 
 // shared-memory reduction without a returned value
@@ -182,7 +195,7 @@ synth_spectral_kernel(SynthArgs A, MixConsts K, SpecConsts C, const float *__res
                 ci[v] = wv * s_;
                 const float xfl = floorf(xf);
                 t[v] = 2.f * (xf - xfl) - 1.f;
-                xi[v] = gi + (int)xfl;
+                xi[v] = gi + (int)near_cell(xfl, C.fG);
             }
             const int xmin = min(min(xi[0], xi[1]), xi[2]);
             const int xmax = max(max(xi[0], xi[1]), xi[2]);

@@ -86,3 +86,24 @@ def test_batch(sim):
     got = sim.simulate(pkg.PATH_SPECTRAL)
     for b, sc in enumerate(scenes):
         check(got[b], sc)
+
+
+@pytest.mark.parametrize("form", ["delay_ref", "far_field"])
+@pytest.mark.parametrize("M", [96, 128])
+def test_lines_beyond_a_cycle_per_sample(sim, form, M):
+    """Vertices up to 9 m from their facet's centroid under a steep, slowly
+    sampled chirp: lines two cycles per sample from it, whose cells are those of
+    the alias.  The FP32 line rate leaves 2^-23 x M / 2 cycles, 2e-5 rad at most,
+    and facets this large have no cancelling weights: the path's bar."""
+    radar = sg.make_radar(M, 3, 1, 2, 2e6, 80e12, 2.0, centre=(0.0, 0.0, 2.0))
+    setattr(radar, form, True)
+    a = np.deg2rad(50.0)
+    tilt = np.array([[1.0, 0.0, 0.0], [0.0, np.cos(a), -np.sin(a)], [0.0, np.sin(a), np.cos(a)]])
+    sc = sg.Scene([sg.plate(9.0, 24.0, 2)],
+                  [sg.Instance(0, (3.0, 60.0, 1.0), sg.rot_z(0.2) @ tilt, (0.5, -4.0, 0.0))], radar,
+                  name="panel")
+    c = sc.meshes[0].verts[sc.meshes[0].tris] @ sc.instances[0].rot.T
+    u = 2.0 * (c - c.mean(1, keepdims=True))[..., 1]           # about along the line of sight
+    assert np.abs(u).max() * radar.slope / (radar.fs * 299792458.0) > 1.2
+    sim.load_scene(sc)
+    check(sim.simulate(pkg.PATH_SPECTRAL), sc)
